@@ -56,6 +56,8 @@ struct aunmf_handle {
   cudaStream_t cap_stream = nullptr;  // private stream used only for graph capture
   std::string cuda_err;
   // workspace
+  Buf tick;                         // zeroed counters of the kernels whose last block finishes up
+  Buf GWr;                          // HALS: W^T W before the normalisation
   Buf Ht, PW, PHt, GH, GW, G64, gpart, dpart, n2a, ctr, relres, last;
   Buf Ax, At, Hk, Wt, parts, err;  // tensor-core path: layout copies, split partials, error flag
   Buf tcacc;                       // tensor-core path, k > 64: partial sums of wide products
@@ -92,7 +94,7 @@ int fail_cuda(aunmf_handle *h, cudaError_t e, const char *what) {
 
 // FP64 partial sums: residual partials, and the layout pass's per-block partials
 size_t dpart_bytes(const aunmf_handle *h) {
-  const size_t a = (size_t)h->n_dparts + 8, b = 2 * (size_t)tc::prepare_blocks();
+  const size_t a = 2 * (size_t)h->n_dparts + 8, b = 2 * (size_t)tc::prepare_blocks();
   return sizeof(double) * (a > b ? a : b);
 }
 
@@ -130,6 +132,23 @@ T *P(Buf &b) {
   return reinterpret_cast<T *>(b.p);
 }
 
+// The handle's ticket counters: one for the Gram kernels, one for the norm and
+// residual kernels (each leaves its own at 0, and a handle's work is in stream
+// order).  Zeroed once, when they are allocated.
+int ensure_tick(aunmf_handle *h) {
+  if (h->tick.p) return AUNMF_OK;
+  ENS(h, h->tick, 2 * sizeof(unsigned));
+  cudaError_t e = cudaMemsetAsync(h->tick.p, 0, 2 * sizeof(unsigned), h->stream);
+  return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "cudaMemsetAsync(tick)");
+}
+#define ENS_TICK(h)                        \
+  do {                                     \
+    int rc_ = ensure_tick(h);              \
+    if (rc_ != AUNMF_OK) return rc_;       \
+  } while (0)
+unsigned *gram_tick(aunmf_handle *h) { return P<unsigned>(h->tick); }
+unsigned *sum_tick(aunmf_handle *h) { return P<unsigned>(h->tick) + 1; }
+
 bool valid_matrix(const aunmf_matrix *A) {
   if (!A || A->m < 1 || A->n < 1) return false;
   if (A->dense) return A->lda >= A->n;
@@ -144,6 +163,7 @@ struct RunCtx {
   int warm;        // BPP starts from the previous iterate's support
   void *bppq;      // BPP scratch (G^{-1})
   float *W, *Ht, *PW, *PHt, *GH, *GW, *gpart;
+  float *GWr;  // HALS: W^T W before the normalisation, which writes GW
   double *GH64, *GW64;  // ABPP: the Grams in FP64 (GH / GW hold them rounded)
   double *dpart, *n2a, *relres_dev, *last;
   DevCounters *ctr;
@@ -317,8 +337,8 @@ cudaError_t gram(aunmf_handle *h, RunCtx &c, const float *X, int64_t rows, float
                  double *G64, cudaStream_t s) {
   if (c.algo == AUNMF_ABPP)
     return launch_gram_d(X, rows, c.k, c.k, G64, G32, reinterpret_cast<double *>(c.gpart),
-                         h->max_gram_blocks, s);
-  return launch_gram(X, rows, c.k, c.k, G32, c.gpart, h->max_gram_blocks, s, c.err);
+                         h->max_gram_blocks, s, gram_tick(h));
+  return launch_gram(X, rows, c.k, c.k, G32, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h));
 }
 
 // Projected-gradient norm of the current (W, H) into pg_dev[ctr->iter], from
@@ -351,11 +371,12 @@ cudaError_t iterate(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   {
     PhaseTimer t(c, s, kPhGram);
-    if ((e = gram(h, c, c.W, m, c.GW, c.GW64, s)) != cudaSuccess) return e;
+    float *G = c.algo == AUNMF_HALS && !printed ? c.GWr : c.GW;
+    if ((e = gram(h, c, c.W, m, G, c.GW64, s)) != cudaSuccess) return e;
   }
   if (c.algo == AUNMF_HALS && !printed) {
     PhaseTimer t(c, s, kPhUpdate);
-    if ((e = launch_hals_normalise(c.W, m, c.Ht, n, c.GW, k, s)) != cudaSuccess) return e;
+    if ((e = launch_hals_normalise(c.W, m, c.Ht, n, c.GWr, c.GW, k, s)) != cudaSuccess) return e;
   }
   if ((e = product_wta(h, c, s)) != cudaSuccess) return e;
   {
@@ -371,7 +392,7 @@ cudaError_t iterate(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   {
     PhaseTimer t(c, s, kPhOther);
     e = launch_relres(c.PHt, c.Ht, n * (int64_t)k, c.GW, c.GH, k, c.n2a, c.dpart, h->n_dparts,
-                      c.relres_dev, c.ctr, c.last, s);
+                      c.relres_dev, c.ctr, c.last, sum_tick(h), s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -523,7 +544,7 @@ int aunmf_set_stream(aunmf_handle *h, void *stream) {
 int aunmf_destroy(aunmf_handle *h) {
   if (!h) return AUNMF_E_INVAL;
   cudaStreamSynchronize(h->stream);
-  Buf *bufs[] = {&h->Ht, &h->PW, &h->PHt, &h->GH, &h->GW, &h->G64, &h->gpart, &h->dpart, &h->n2a,
+  Buf *bufs[] = {&h->tick, &h->GWr, &h->Ht, &h->PW, &h->PHt, &h->GH, &h->GW, &h->G64, &h->gpart, &h->dpart, &h->n2a,
                  &h->ctr, &h->relres, &h->last, &h->Ax, &h->At, &h->Hk, &h->Wt, &h->parts,
                  &h->err, &h->tcacc, &h->aux, &h->spl, &h->splpart, &h->colptr, &h->rowidx, &h->cval, &h->cscratch, &h->bppq, &h->dHt,
                  &h->batch, &h->batch_meta, &h->hA, &h->hW, &h->hH};
@@ -613,6 +634,8 @@ int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters
   ENS(h, h->PHt, sizeof(float) * n * k);
   ENS(h, h->GH, sizeof(float) * k * k);
   ENS(h, h->GW, sizeof(float) * k * k);
+  ENS(h, h->GWr, sizeof(float) * k * k);
+  ENS_TICK(h);
   ENS(h, h->G64, 2 * sizeof(double) * k * k);
   ENS(h, h->gpart, sizeof(double) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->dpart, dpart_bytes(h));
@@ -637,6 +660,7 @@ int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters
   c.PHt = P<float>(h->PHt);
   c.GH = P<float>(h->GH);
   c.GW = P<float>(h->GW);
+  c.GWr = P<float>(h->GWr);
   c.GH64 = P<double>(h->G64);
   c.GW64 = c.GH64 + (size_t)k * k;
   c.gpart = P<float>(h->gpart);
@@ -680,9 +704,9 @@ int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters
   if (A->dense && o.prec != AUNMF_FP32) {
     // ||A||^2 comes out of the layout pass (prepare_tc below)
   } else if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, s));
+    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   } else {
-    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (o.prec != AUNMF_FP32) {
     int prc = prepare_tc(h, c, s);
@@ -842,8 +866,9 @@ int aunmf_gram_w(aunmf_handle *h, const float *W, int64_t m, int k, float *G) {
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->err, sizeof(int));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
+  ENS_TICK(h);
   CK(h, launch_gram(W, m, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   return AUNMF_OK;
 }
 
@@ -853,9 +878,10 @@ int aunmf_gram_h(aunmf_handle *h, const float *H, int k, int64_t n, float *G) {
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->err, sizeof(int));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
+  ENS_TICK(h);
   CK(h, launch_transpose(H, k, n, P<float>(h->Ht), h->stream));
   CK(h, launch_gram(P<float>(h->Ht), n, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   return AUNMF_OK;
 }
 
@@ -970,14 +996,16 @@ int aunmf_update_w(aunmf_handle *h, int algo, float *W, const float *PW, const f
   if (algo == AUNMF_HALS) {
     ENS(h, h->GW, sizeof(float) * k * k);
     ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
-    CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s));
+    ENS_TICK(h);
+    CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s, nullptr,
+                      gram_tick(h)));
     if (H && n > 0) {
       ENS(h, h->Ht, sizeof(float) * n * k);
       CK(h, launch_transpose(H, k, n, P<float>(h->Ht), s));
-      CK(h, launch_hals_normalise(W, m, P<float>(h->Ht), n, P<float>(h->GW), k, s));
+      CK(h, launch_hals_normalise(W, m, P<float>(h->Ht), n, P<float>(h->GW), nullptr, k, s));
       CK(h, launch_transpose(P<float>(h->Ht), n, k, H, s));
     } else {
-      CK(h, launch_hals_normalise(W, m, nullptr, 0, P<float>(h->GW), k, s));
+      CK(h, launch_hals_normalise(W, m, nullptr, 0, P<float>(h->GW), nullptr, k, s));
     }
   }
   return AUNMF_OK;
@@ -1053,16 +1081,17 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
   float *Ht = P<float>(h->Ht), *PHt = P<float>(h->PHt);
   double *dp = P<double>(h->dpart);
   ENS(h, h->err, sizeof(int));
+  ENS_TICK(h);
   CK(h, cudaMemsetAsync(h->ctr.p, 0, sizeof(DevCounters), s));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), s));
   CK(h, launch_transpose(H, k, n, Ht, s));
   if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), s));
+    CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     ENS(h, h->parts, simt_parts_bytes(A->m > n ? A->m : n, k));
     CK(h, launch_wta_simt(A->dense, m, n, A->lda, W, k, PHt, P<float>(h->parts), P<int>(h->err),
                           s));
   } else {
-    CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     RunCtx c{};
     c.A = A;
     int rc = prepare_sparse(h, c, s);
@@ -1070,12 +1099,12 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
     CK(h, launch_wta_csc(c.colptr, c.rowidx, c.cval, n, m, A->nnz, W, k, PHt, &c.csc_long, s));
   }
   CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   CK(h, launch_gram(Ht, n, k, k, P<float>(h->GH), P<float>(h->gpart), h->max_gram_blocks, s,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   CK(h, launch_relres(PHt, Ht, n * (int64_t)k, P<float>(h->GW), P<float>(h->GH), k,
                       P<double>(h->n2a), dp, h->n_dparts, nullptr, P<DevCounters>(h->ctr),
-                      P<double>(h->last), s));
+                      P<double>(h->last), sum_tick(h), s));
   int herr = 0;
   CK(h, cudaMemcpyAsync(&herr, h->err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(h, cudaMemcpyAsync(relres, h->last.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1103,6 +1132,7 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->dpart, dpart_bytes(h));
   ENS(h, h->n2a, 2 * sizeof(double));
+  ENS_TICK(h);
   c.A = A;
   c.k = k;
   c.prec = prec;
@@ -1121,14 +1151,14 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
     int rc = prepare_tc(h, c, s);  // also writes ||A||^2
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, s));
+    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
     ENS(h, h->parts, simt_parts_bytes(m > n ? m : n, k));
     c.parts = P<float>(h->parts);
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));
   } else {
-    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (!A->dense) {
     int rc = prepare_sparse(h, c, s);
@@ -1147,10 +1177,10 @@ int aunmf_loss_fwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;
   CK(h, product_wta(h, c, s));
-  CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err));
-  CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err));
+  CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
+  CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
   CK(h, launch_loss(c.PHt, c.Ht, n * (int64_t)k, c.GW, c.GH, k, c.n2a, c.dpart, h->n_dparts, loss,
-                    s));
+                    sum_tick(h), s));
   if (WtA) CK(h, launch_transpose(c.PHt, n, k, WtA, s));
   return AUNMF_OK;
 }
@@ -1164,13 +1194,13 @@ int aunmf_loss_bwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;
   if (dW) {  // dL/dW = W (H H^T) - A H^T
-    CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err));
+    CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
     CK(h, product_aht(h, c, s));
     CK(h, launch_xg_minus_p(c.W, c.PW, c.GH, m, k, grad_out, dW, s));
   }
   if (dH) {  // dL/dH = (W^T W) H - W^T A, formed transposed
     ENS(h, h->dHt, sizeof(float) * n * k);
-    CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err));
+    CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
     if (WtA) {
       CK(h, launch_transpose(WtA, k, n, c.PHt, s));
     } else {

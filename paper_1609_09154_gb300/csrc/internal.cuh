@@ -103,14 +103,19 @@ __device__ __forceinline__ void two_fma_acc(float a, float b, float &hi, float &
 // err: the device error flag for the bounded waits of the wide-rank form
 // (k >= 96, which runs the TMA-fed product kernel on X^T X); null keeps the
 // k_gram_part form.
+// ticket: a zeroed counter (left at 0) that lets a small factor's last block
+// add the partials; null: always a second launch.  Launches that share a
+// ticket run in stream order, as they share the partials.
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr);
+                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr,
+                        unsigned *ticket = nullptr);
 int gram_partial_blocks(int64_t rows, int max_blocks);
 // The same Gram with every product formed exactly in FP64 (FP32 x FP32 fits a
 // double) and summed in FP64: G64 (k x k, FP64) for the BPP solves, and G32 =
 // G64 rounded to FP32 (may be null).  partials: max_blocks * k * k doubles.
 cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, double *G64,
-                          float *G32, double *partials, int max_blocks, cudaStream_t s);
+                          float *G32, double *partials, int max_blocks, cudaStream_t s,
+                          unsigned *ticket = nullptr);
 // G64 = G32 widened (k x k).
 cudaError_t launch_widen(const float *G32, int k, double *G64, cudaStream_t s);
 
@@ -186,9 +191,10 @@ cudaError_t launch_pgrad_partial(const float *X, const float *P, const float *G,
 cudaError_t launch_pgrad_final(const double *part, int n, const DevCounters *ctr, double *out,
                                cudaStream_t s);
 // HALS normalisation: s_i = sqrt(GW_ii); X(:, i) /= s_i; Y(:, i) *= s_i (Y = Ht,
-// may be null, rows_y rows); GW_ij /= s_i s_j.  Zero norms leave column i as is.
-cudaError_t launch_hals_normalise(float *X, int64_t rows_x, float *Y, int64_t rows_y, float *GW,
-                                  int k, cudaStream_t s);
+// may be null, rows_y rows); Gn_ij = GW_ij / (s_i s_j) (Gn may be null, not
+// GW: every block reads GW's diagonal).  Zero norms leave column i as is.
+cudaError_t launch_hals_normalise(float *X, int64_t rows_x, float *Y, int64_t rows_y,
+                                  const float *GW, float *Gn, int k, cudaStream_t s);
 // BPP: X(r, :) = argmin_{x>=0} ||C x - b|| given G = C^T C (FP64) and
 // R(r, :) = C^T b, in FP64.  warm != 0 starts each row from the support of
 // X's current row.  scratch: bpp_scratch_bytes(k, rows) bytes of device
@@ -199,21 +205,22 @@ cudaError_t launch_bpp(const double *G, const float *R, int64_t rows, int k, flo
 
 // Reductions for the relative residual.
 // sum of squares of A (dense) or of val (CSR) into *out (device double).
+// (ticket as for launch_gram, never null here; partials: 2 nparts doubles.)
 cudaError_t launch_norm2(const float *A, int64_t m, int64_t n, int64_t lda, double *partials,
-                         int nparts, double *out, cudaStream_t s);
+                         int nparts, double *out, unsigned *ticket, cudaStream_t s);
 cudaError_t launch_norm2_vec(const float *v, int64_t len, double *partials, int nparts,
-                             double *out, cudaStream_t s);
+                             double *out, unsigned *ticket, cudaStream_t s);
 // relres[ctr->iter++] = sqrt(max(0, n2a - 2 <P, Ht> + <GW, GH>) / n2a); also
 // copies the value to *last.
 cudaError_t launch_relres(const float *P, const float *Ht, int64_t len, const float *GW,
                           const float *GH, int k, const double *n2a, double *partials,
                           int nparts, double *relres_dev, DevCounters *ctr, double *last,
-                          cudaStream_t s);
+                          unsigned *ticket, cudaStream_t s);
 
 // 0.5 ||A - W H||^2 = 0.5 (n2a - 2 <P, Ht> + <GW, GH>) into *loss (device).
 cudaError_t launch_loss(const float *P, const float *Ht, int64_t len, const float *GW,
                         const float *GH, int k, const double *n2a, double *partials, int nparts,
-                        double *loss, cudaStream_t s);
+                        double *loss, unsigned *ticket, cudaStream_t s);
 // out = g (X G - P), X and P rows x k, G k x k, g = *gscale (NULL: 1).
 cudaError_t launch_xg_minus_p(const float *X, const float *P, const float *G, int64_t rows, int k,
                               const float *gscale, float *out, cudaStream_t s);

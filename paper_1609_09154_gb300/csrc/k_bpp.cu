@@ -64,6 +64,15 @@ __global__ void __launch_bounds__(32 * kBppWarps, 1)
        row += (int64_t)gridDim.x * nwb) {
     bool fnum, fcap;
     const int it = bpp_row_fast<KT>(w, R, row, k, X, warm, max_piv, &fnum, &fcap);
+    // with an ill-conditioned G (cond >= 1e8) a row at the full cap has been
+    // going round in circles on the solves' own rounding (an x_j within
+    // cond 2^-44 of 0 changes sign and back): the FP64 kernel, whose noise is
+    // ~500 times smaller, goes on from the set it reached.  Which rows these
+    // are depends on the last bits of G and R.
+    if (fcap && w.refine && max_piv >= 10 * k) {
+      fnum = true;
+      fcap = false;
+    }
     if (lane == 0) redo[row] = fnum ? 1 : 0;
     if (!fnum) {
       piv_total += it;

@@ -262,59 +262,52 @@ __global__ void __launch_bounds__(kLucThreads)
 }
 
 // HALS normalisation (Eq. halsupdate, w^i / ||w^i||, compensated in H):
-// s_i = sqrt(GW_ii); X(:, i) /= s_i; Y(:, i) *= s_i; GW_ij /= s_i s_j.
-// A warp per row, its lanes on the row's entries (no index division per
-// entry: a 64-bit remainder costs ~40 instructions and bound the pass at
-// 5.9e9 entries); the column scales are staged once per block.
-__global__ void k_hals_scale_rows(float *__restrict__ X, int64_t rows, int k,
-                                  const float *__restrict__ GW, bool divide) {
-  // the factor per column: 1 / s_i (divide) or s_i, 1 where G_ii <= 0; a
-  // product with the reciprocal differs from the quotient by at most an ulp,
-  // and a division per entry bound the pass (0.1 ms for 5e7 entries)
-  __shared__ float sc[AUNMF_K_MAX];
+// s_i = sqrt(GW_ii); X(:, i) /= s_i; Y(:, i) *= s_i; Gn_ij = GW_ij / (s_i s_j).
+// One launch over the rows of X, Y and the Gram matrix (three took 3.3 us each
+// at k = 10, and a one-block Gram rescale 58 us at k = 256).  A warp per row,
+// its lanes on the row's entries (no index division per entry: a 64-bit
+// remainder costs ~40 instructions and bound the pass at 5.9e9 entries); the
+// column scales are staged once per block.
+__global__ void k_hals_normalise(float *__restrict__ X, int64_t rows_x, float *__restrict__ Y,
+                                 int64_t rows_y, int k, const float *__restrict__ GW,
+                                 float *__restrict__ Gn) {
+  // the factor per column: 1 / s_i or s_i, 1 where G_ii <= 0; a product with
+  // the reciprocal differs from the quotient by at most an ulp, and a
+  // division per entry bound the pass (0.1 ms for 5e7 entries)
+  __shared__ float sc[AUNMF_K_MAX], rc[AUNMF_K_MAX];
   for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    const float g = GW[i * k + i];
+    const float g = GW[(size_t)i * k + i];
     const float si = g > 0.f ? sqrtf(g) : 1.f;  // >= 3.7e-23: 1 / si is finite
-    sc[i] = divide ? 1.f / si : si;
+    sc[i] = si;
+    rc[i] = 1.f / si;
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t ws = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if ((k & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 7) == 0) {
-    // even k: rows start on 8-byte boundaries, a lane scales two entries
-    for (int64_t r = w0; r < rows; r += ws) {
-      float2 *x = reinterpret_cast<float2 *>(X + r * k);
+  const bool even = (k & 1) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 7) == 0;
+  const int64_t total = rows_x + rows_y + (Gn ? k : 0);
+  for (int64_t r = w0; r < total; r += ws) {
+    if (r >= rows_x + rows_y) {
+      const int i = (int)(r - rows_x - rows_y);
+      const float si = sc[i];
+      for (int j = lane; j < k; j += 32) Gn[(size_t)i * k + j] = GW[(size_t)i * k + j] / (si * sc[j]);
+      continue;
+    }
+    const float *f = r < rows_x ? rc : sc;
+    float *row = r < rows_x ? X + r * k : Y + (r - rows_x) * k;
+    if (even) {
+      // even k: rows start on 8-byte boundaries, a lane scales two entries
+      float2 *x = reinterpret_cast<float2 *>(row);
       for (int i = lane; 2 * i < k; i += 32) {
         float2 v = x[i];
-        v.x *= sc[2 * i];
-        v.y *= sc[2 * i + 1];
+        v.x *= f[2 * i];
+        v.y *= f[2 * i + 1];
         x[i] = v;
       }
+    } else {
+      for (int i = lane; i < k; i += 32) row[i] *= f[i];
     }
-    return;
-  }
-  for (int64_t r = w0; r < rows; r += ws) {
-    float *x = X + r * k;
-    for (int i = lane; i < k; i += 32) x[i] *= sc[i];
-  }
-}
-
-__global__ void __launch_bounds__(512) k_hals_scale_gram(float *__restrict__ GW, int k) {
-  // one block of 32 x 16 threads: read the diagonal first, then rescale,
-  // 16 rows at a time with a warp along each (no index division per entry:
-  // with one it took 0.58 ms at k = 512)
-  __shared__ float sd[AUNMF_K_MAX];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  for (int i = tid; i < k; i += blockDim.x * blockDim.y) {
-    const float g = GW[i * k + i];
-    sd[i] = g > 0.f ? sqrtf(g) : 1.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < k; i += blockDim.y) {
-    const float si = sd[i];
-    float *row = GW + (size_t)i * k;
-    for (int j = threadIdx.x; j < k; j += blockDim.x) row[j] = row[j] / (si * sd[j]);
   }
 }
 
@@ -421,8 +414,8 @@ __global__ void __launch_bounds__(kTprThreads)
   const float g = (OP == kOpGrad && gscale) ? *gscale : 1.f;
   float *dst = OP == kOpGrad ? out : X;
   const int64_t groups = (rows + kTprRows - 1) / kTprRows;
-  for (int64_t grp = (int64_t)blockIdx.x * kTprWarps + wib; grp < groups;
-       grp += (int64_t)gridDim.x * kTprWarps) {
+  const int nwb = blockDim.x >> 5;  // kTprWarps, fewer for few rows
+  for (int64_t grp = (int64_t)blockIdx.x * nwb + wib; grp < groups; grp += (int64_t)gridDim.x * nwb) {
     const int64_t r0 = grp * kTprRows;
     const int nr = (int)min((int64_t)kTprRows, rows - r0);
     tile_in<KP>(X + r0 * k, nr, k, tile, lane);
@@ -486,9 +479,13 @@ cudaError_t launch_tpr(float *X, const float *P, const float *G, int64_t rows, i
     resident = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 152);
   }
   const int64_t groups = (rows + kTprRows - 1) / kTprRows;
-  int64_t nb = (groups + kTprWarps - 1) / kTprWarps;
+  // few rows: fewer warps a block, so that the row groups spread over the SMs
+  int64_t wpb = (groups + 151) / 152;
+  if (wpb > kTprWarps) wpb = kTprWarps;
+  int64_t nb = (groups + wpb - 1) / wpb;
   if (nb > resident) nb = resident;
-  k_luc_tpr<KP, OP><<<(unsigned)nb, kTprThreads, smem, s>>>(X, P, G, rows, k, eps, gscale, out);
+  k_luc_tpr<KP, OP><<<(unsigned)nb, (unsigned)(32 * wpb), smem, s>>>(X, P, G, rows, k, eps, gscale,
+                                                                    out);
   g_launches += 1;
   return cudaGetLastError();
 }
@@ -811,20 +808,15 @@ cudaError_t launch_xg_minus_p(const float *X, const float *P, const float *G, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_hals_normalise(float *X, int64_t rows_x, float *Y, int64_t rows_y, float *GW,
-                                  int k, cudaStream_t s) {
-  auto nb = [](int64_t total) {
-    int64_t b = (total + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
-    return (int)(b < 1 ? 1 : b);
-  };
-  auto scale = [&](float *Z, int64_t rows, bool divide) {
-    k_hals_scale_rows<<<nb(rows * 32), 256, 0, s>>>(Z, rows, k, GW, divide);
-  };
-  if (rows_x > 0) scale(X, rows_x, true);
-  if (Y && rows_y > 0) scale(Y, rows_y, false);
-  k_hals_scale_gram<<<1, dim3(32, 16), 0, s>>>(GW, k);
-  g_launches += 1 + (rows_x > 0) + (Y && rows_y > 0);
+cudaError_t launch_hals_normalise(float *X, int64_t rows_x, float *Y, int64_t rows_y,
+                                  const float *GW, float *Gn, int k, cudaStream_t s) {
+  if (!Y) rows_y = 0;
+  const int64_t rows = rows_x + rows_y + (Gn ? k : 0);
+  if (rows == 0) return cudaSuccess;
+  int64_t nb = (rows + 7) / 8;  // eight warps a block
+  if (nb > 152 * 16) nb = 152 * 16;
+  k_hals_normalise<<<(unsigned)nb, 256, 0, s>>>(X, rows_x, Y, rows_y, k, GW, Gn);
+  g_launches += 1;
   return cudaGetLastError();
 }
 

@@ -7,6 +7,7 @@
 // Internally H is held transposed (Ht, n x k) so that both factors are
 // row-major "rows x k" and share the same update kernels.
 #include <math.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -31,6 +32,19 @@ constexpr int kGramThreads = 256;
 // sum (FP32 path) or the FP64 sum (FP64-accurate path)
 constexpr int kGramSlab = 32;
 
+// True in exactly one block of the launch, the last to arrive, whose threads
+// then see what every block wrote before.  *ticket wraps back to 0.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+  __shared__ unsigned order;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) order = atomicInc(ticket, gridDim.x - 1);
+  __syncthreads();
+  if (order != gridDim.x - 1) return false;
+  __threadfence();
+  return true;
+}
+
 __device__ __forceinline__ int gram_groups(int ntiles) {
   return ntiles >= kGramThreads ? 1 : kGramThreads / ntiles;
 }
@@ -49,10 +63,14 @@ __device__ __forceinline__ int gram_groups(int ntiles) {
 //     positive definite.
 // The next 64-row slab is loaded into registers while the current one is
 // consumed from shared memory.  Dynamic shared memory: gram_smem_bytes().
+// ticket (may be null): the last block to finish adds all partials in FP64,
+// in block order, and writes G32 (FP64 form: G64, and G32 unless null), which
+// spares the reduction's launch; *ticket starts at 0 and is 0 again after.
 template <bool FP64>
 __global__ void __launch_bounds__(kGramThreads, 2)
     k_gram_part(const float *__restrict__ X, int64_t rows, int k, int64_t ldx, int64_t chunk,
-                typename std::conditional<FP64, double, float>::type *__restrict__ partials) {
+                typename std::conditional<FP64, double, float>::type *__restrict__ partials,
+                float *__restrict__ G32, double *__restrict__ G64, unsigned *ticket) {
   using T = typename std::conditional<FP64, double, float>::type;
   extern __shared__ __align__(16) float sX[];  // [kGramRows][kp], then the group sums
   constexpr int kPre = (kGramRows * 64 + kGramThreads - 1) / kGramThreads;  // k <= 64 prefetch
@@ -154,7 +172,10 @@ __global__ void __launch_bounds__(kGramThreads, 2)
         }
       }
     }
-    // the groups' sums, added in group order
+    // the groups' sums: every entry of every tile is added over the groups by a
+    // thread of its own, in group order (FP64: four interleaved chains; one
+    // thread per tile doing its 16 entries took most of a small factor's 11-44
+    // us: ngrp is 42 at k = 10)
     __syncthreads();
     if (act && ngrp > 1) {
 #pragma unroll
@@ -164,13 +185,33 @@ __global__ void __launch_bounds__(kGramThreads, 2)
           gsum[((size_t)g * ntiles + t) * 16 + 4 * p + q] = FP64 ? sum[p][q] : sum[p][q] - cmp[p][q];
     }
     __syncthreads();
-    if (act && g == 0) {
+    if (ngrp > 1) {
+      const int ne = ntiles * 16;
+      for (int e = threadIdx.x; e < ne; e += kGramThreads) {
+        constexpr int kChains = FP64 ? 4 : 1;
+        T c[kChains] = {};
+        int h = 0;
+#pragma unroll 4
+        for (; h + kChains <= ngrp; h += kChains)
+#pragma unroll
+          for (int u = 0; u < kChains; ++u) c[u] += gsum[(size_t)(h + u) * ne + e];
+        for (; h < ngrp; ++h) c[0] += gsum[(size_t)h * ne + e];
+        T v = c[0];
+        if constexpr (FP64) v = (c[0] + c[1]) + (c[2] + c[3]);
+        int rem = e >> 4, i = 0;
+        while (rem >= nt - i) { rem -= nt - i; ++i; }
+        const int gi = 4 * i + ((e >> 2) & 3), gj = 4 * (i + rem) + (e & 3);
+        if (gi < k && gj < k) {
+          out[gi * k + gj] = v;
+          out[gj * k + gi] = v;
+        }
+      }
+    } else if (act) {
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          T v = FP64 ? sum[p][q] : sum[p][q] - cmp[p][q];
-          for (int h = 1; h < ngrp; ++h) v += gsum[((size_t)h * ntiles + t) * 16 + 4 * p + q];
+          const T v = FP64 ? sum[p][q] : sum[p][q] - cmp[p][q];
           const int i = 4 * ti + p, j = 4 * tj + q;
           if (i < k && j < k) {
             out[i * k + j] = v;
@@ -178,6 +219,20 @@ __global__ void __launch_bounds__(kGramThreads, 2)
           }
         }
     }
+  }
+  if (!ticket) return;
+  if (!last_block(ticket)) return;
+  const int kk = k * k, nb = gridDim.x;
+  for (int e = threadIdx.x; e < kk; e += kGramThreads) {
+    double a[8] = {};
+    int b = 0;
+    for (; b + 8 <= nb; b += 8)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) a[u] += (double)__ldcg(&partials[(int64_t)(b + u) * kk + e]);
+    for (; b < nb; ++b) a[0] += (double)__ldcg(&partials[(int64_t)b * kk + e]);
+    const double v = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    if constexpr (FP64) G64[e] = v;
+    if (G32) G32[e] = (float)v;
   }
 }
 
@@ -348,14 +403,21 @@ size_t gram_smem_bytes(int k) {
   return slab + grp;
 }
 
-__global__ void __launch_bounds__(256)
+// G_e = sum_b partials[b]_e in FP64: 32 entries per block; each of the block's
+// warps sums its share of the partials in four interleaved chains (b
+// ascending within each), and the chains and then the warps' sums are added
+// in a fixed order, so the result does not depend on scheduling.  32 warps for
+// many partials (with eight, 188 partials at k = 50 took 10 us a call), eight
+// for few (a wide Gram's 13-19 partials: 11 us at k = 256, 29 us with 32).
+int gram_red_threads(int nb) { return nb >= 64 ? 1024 : 256; }
+__global__ void __launch_bounds__(1024)
     k_gram_reduce_d(const double *__restrict__ partials, int nb, int k, double *__restrict__ G64,
                     float *__restrict__ G32) {
-  __shared__ double sw[8][32];
+  __shared__ double sw[32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int kk = k * k;
   const int e = blockIdx.x * 32 + lane;
-  const int per = (nb + 7) / 8;
+  const int nw = blockDim.x >> 5, per = (nb + nw - 1) / nw;
   const int b0 = w * per, b1 = min(nb, b0 + per);
   // four independent chains (loads in flight, FP64 latency overlapped),
   // combined in a fixed order
@@ -374,7 +436,7 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   if (w == 0 && e < kk) {
     double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += sw[q][lane];
+    for (int q = 0; q < nw; ++q) s += sw[q][lane];
     G64[e] = s;
     if (G32) G32[e] = (float)s;
   }
@@ -385,17 +447,13 @@ __global__ void k_widen(const float *__restrict__ G32, int kk, double *__restric
     G64[e] = (double)G32[e];
 }
 
-// G_e = sum_b partials[b]_e in FP64: 32 entries per block; warp w sums the
-// w-th eighth of the blocks in four interleaved chains (b ascending within
-// each), and the chains and then the eight warp sums are added in a fixed
-// order, so the result does not depend on scheduling.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
     k_gram_reduce(const float *__restrict__ partials, int nb, int k, float *__restrict__ G) {
-  __shared__ double sw[8][32];
+  __shared__ double sw[32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int kk = k * k;
   const int e = blockIdx.x * 32 + lane;
-  const int per = (nb + 7) / 8;
+  const int nw = blockDim.x >> 5, per = (nb + nw - 1) / nw;
   const int b0 = w * per, b1 = min(nb, b0 + per);
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   if (e < kk) {
@@ -412,7 +470,7 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   if (w == 0 && e < kk) {
     double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += sw[i][lane];
+    for (int i = 0; i < nw; ++i) t += sw[i][lane];
     G[e] = (float)t;
   }
 }
@@ -426,12 +484,17 @@ int gram_partial_blocks(int64_t rows, int max_blocks) {
 }
 
 namespace {
+// The last block's sum of nb partials replaces the reduction's launch (~2 us)
+// while one block's reads of nb k^2 values take less.
+bool fused_final(int nb, int k) { return (int64_t)nb * k * k <= 24000; }
+
 bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partials, int max_blocks,
                    int *err, cudaStream_t s, cudaError_t *status);
 }  // namespace
 
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err) {
+                        float *partials, int max_blocks, cudaStream_t s, int *err,
+                        unsigned *ticket) {
   // wide ranks: the TMA-fed FP32 product kernel on X^T X (below)
   if (ldx == k && err) {
     cudaError_t st = cudaSuccess;
@@ -457,7 +520,7 @@ cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float 
     auto kern = (k & 1) ? k_gram8<false> : k_gram8<true>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kG8Smem);
     kern<<<(unsigned)nb, kG8Threads, kG8Smem, s>>>(X, rows, k, chunk, partials);
-    k_gram_reduce<<<(k * k + 31) / 32, 256, 0, s>>>(partials, (int)nb, k, G);
+    k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads((int)nb), 0, s>>>(partials, (int)nb, k, G);
     g_launches += 2;
     return cudaGetLastError();
   }
@@ -466,22 +529,30 @@ cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float 
   const size_t smem = gram_smem_bytes<false>(k);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_gram_part<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_gram_part<false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
-  k_gram_reduce<<<(k * k + 31) / 32, 256, 0, s>>>(partials, nb, k, G);
-  g_launches += 2;
+  if (!fused_final(nb, k)) ticket = nullptr;
+  k_gram_part<false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, G, nullptr,
+                                                   ticket);
+  if (!ticket) k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G);
+  g_launches += ticket ? 1 : 2;
   return cudaGetLastError();
 }
 
 cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, double *G64,
-                          float *G32, double *partials, int max_blocks, cudaStream_t s) {
-  const int nb = gram_partial_blocks(rows, max_blocks);
+                          float *G32, double *partials, int max_blocks, cudaStream_t s,
+                          unsigned *ticket) {
+  // 64 rows (one stage) per block while 128 would leave most SMs idle
+  int nb = gram_partial_blocks(rows, max_blocks);
+  if (nb <= max_blocks / 4) nb = (int)((rows + 63) / 64);
   const int64_t chunk = (rows + nb - 1) / nb;
   const size_t smem = gram_smem_bytes<true>(k);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_gram_part<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_gram_part<true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
-  k_gram_reduce_d<<<(k * k + 31) / 32, 256, 0, s>>>(partials, nb, k, G64, G32);
-  g_launches += 2;
+  if (!fused_final(nb, k)) ticket = nullptr;
+  k_gram_part<true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, G32, G64,
+                                                  ticket);
+  if (!ticket)
+    k_gram_reduce_d<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G64, G32);
+  g_launches += ticket ? 1 : 2;
   return cudaGetLastError();
 }
 
@@ -736,40 +807,79 @@ __global__ void __launch_bounds__(256, AUNMF_SIMT_MINB)
 // (thread 0 first waits, bounded, for the copies it has in flight).  The K
 // steps of a split are whole (its length is a multiple of 128); rows and
 // columns past either matrix are zero-filled by the copies.
-constexpr int kTBM = 256, kTBN = 64, kTBK = 16, kTStages = 7;
+constexpr int kTBK = 16, kTStages = 7;
 constexpr int kTThreads = 256;
 constexpr int kTSlabSteps = 8;  // K steps per compensated slab (128 K, as k_gemm_simt)
-constexpr int kTLdc = 68;       // floats per thread row of corrections (64 + pad)
-constexpr size_t kTStageA = (size_t)kTBM * kTBK * 4, kTStageB = (size_t)kTBK * kTBN * 4;
-constexpr size_t kTSmem = 1024 + kTStages * (kTStageA + kTStageB) +
-                          (size_t)kTThreads * kTLdc * 4 + 2 * kTStages * 8;
+// Shape of one form: RT rows and BN / 8 columns per thread, a tile of 32 RT
+// rows by BN columns.
+template <int RT, int BN>
+struct SimtTile {
+  static constexpr int BM = 32 * RT, TN = BN / 8, NE = RT * TN;
+  static constexpr int kLdc = NE + 4;  // floats per thread row of corrections (+ pad: no bank conflict)
+  static constexpr size_t kA = (size_t)BM * kTBK * 4, kB = (size_t)kTBK * BN * 4;
+  // after the corrections: the slab sums of the cluster form (slabs tiles)
+  static constexpr size_t smem(int slabs) {
+    return 1024 + kTStages * (kA + kB) + (slabs ? 0 : (size_t)kTThreads * kLdc * 4) +
+           (size_t)slabs * BM * BN * 4 + 2 * kTStages * 8 + 16;
+  }
+};
 
-template <bool AK>
+// Column j (0 .. TN - 1) of thread column tx within the tile.
+template <int TN>
+__device__ __forceinline__ int simt_col(int tx, int j) {
+  if constexpr (TN == 8)
+    return j < 4 ? tx * 4 + j : 32 + tx * 4 + j - 4;
+  else
+    return tx * TN + j;
+}
+
+template <bool AK, int RT, int BN, bool VEC>
 __global__ void __launch_bounds__(kTThreads, 1)
     k_gemm_simt_tma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                    int64_t M, int64_t K, int N, float *__restrict__ C, int ldc, int64_t kchunk,
-                    int *err, long long limit, int inject) {
+                    const float *__restrict__ A, int64_t lda, const float *__restrict__ B,
+                    int64_t M, int64_t K, int N, float *__restrict__ C,
+                    int ldc, int64_t kchunk, int clus, int group, int *err, long long limit,
+                    int inject) {
+  // The short form (RT = 4, few tiles) stages the factor's tile with 4-byte
+  // asynchronous copies straight from B (K x N, contiguous): it spares the
+  // launch that pads B's rows to 16 bytes for TMA (mapB is not used).  VEC
+  // false (short form only): A's rows are not 16-byte aligned, and its tile is
+  // copied the same way into the same places (mapA is not used).
+  static_assert(VEC || RT == 4, "unaligned rows: short form");
+  // clus > 0: the grid's clus K splits of a tile form one cluster (1, 1, clus):
+  // every block keeps its slab sums in shared memory, and the cluster folds all
+  // of them, in K order, through distributed shared memory: with Kahan's
+  // compensation within each `group` slabs, the groups' sums added plainly --
+  // the additions of an unclustered pass over K split every `group` slabs, so
+  // both give the same bits.  clus == 0: split z writes its partial at C + z M ldc.
   // inject (test hook): thread 0 never arrives on the first stage's barrier,
   // so every thread's bounded wait runs out
   using namespace aunmf::ptx;
+  using T = SimtTile<RT, BN>;
+  constexpr int BM = T::BM, TN = T::TN, NE = T::NE;
+  constexpr bool BCP = RT == 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023);
   float *sA = reinterpret_cast<float *>(smem);
-  float *sB = reinterpret_cast<float *>(smem + kTStages * kTStageA);
-  float *corr = reinterpret_cast<float *>(smem + kTStages * (kTStageA + kTStageB));
-  uint64_t *full = reinterpret_cast<uint64_t *>(corr + kTThreads * kTLdc);
+  float *sB = reinterpret_cast<float *>(smem + kTStages * T::kA);
+  float *corr = reinterpret_cast<float *>(smem + kTStages * (T::kA + T::kB));
+  const int nslab = clus > 0 ? (int)(kchunk / (kTBK * kTSlabSteps)) : 0;
+  uint64_t *full =
+      reinterpret_cast<uint64_t *>(corr + (clus > 0 ? nslab * BM * BN : kTThreads * T::kLdc));
   uint64_t *empty = full + kTStages;
+  int *flag = reinterpret_cast<int *>(empty + kTStages);  // 1: this block finished its K range
   const int tid = threadIdx.x;
-  const int64_t m0 = (int64_t)blockIdx.x * kTBM;
-  const int n0 = blockIdx.y * kTBN;
+  const int64_t m0 = (int64_t)blockIdx.x * BM;
+  const int n0 = blockIdx.y * BN;
   const int64_t kz0 = (int64_t)blockIdx.z * kchunk, kz1 = min(K, kz0 + kchunk);
   const int nsteps = kz1 > kz0 ? (int)((kz1 - kz0 + kTBK - 1) / kTBK) : 0;
   const bool producer = tid < 32;
   if (tid == 0) {
     for (int st = 0; st < kTStages; ++st) {
-      mbar_init(&full[st], 1);
+      mbar_init(&full[st], BCP ? 1 + kTThreads : 1);
       mbar_init(&empty[st], kTThreads);
     }
+    *flag = 1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -780,7 +890,11 @@ __global__ void __launch_bounds__(kTThreads, 1)
   auto fill = [&](int s) {
     const int st = s % kTStages;
     const int k0 = (int)(kz0 + (int64_t)s * kTBK);
-    const uint32_t bytes = (uint32_t)(kTStageA + kTStageB);
+    const uint32_t bytes = (uint32_t)(!VEC ? 0 : BCP ? T::kA : T::kA + T::kB);
+    if (!VEC) {
+      if (!(inject && s == 0)) mbar_arrive(&full[st]);
+      return;
+    }
     if (inject && s == 0)
       mbar_expect_tx_only(&full[st], bytes);
     else
@@ -791,49 +905,106 @@ __global__ void __launch_bounds__(kTThreads, 1)
                      AUNMF_CHECK_TMA_COORD))
       return;
     if (AK)
-      tma_load_2d(sA + (size_t)st * kTBM * kTBK, &mapA, &full[st], k0, (int)m0, pol_a);
+      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], k0, (int)m0, pol_a);
     else
-      tma_load_2d(sA + (size_t)st * kTBM * kTBK, &mapA, &full[st], (int)m0, k0, pol_a);
-    tma_load_2d(sB + (size_t)st * kTBK * kTBN, &mapB, &full[st], n0, k0, pol_b);
+      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], (int)m0, k0, pol_a);
+    if (!BCP) tma_load_2d(sB + (size_t)st * kTBK * BN, &mapB, &full[st], n0, k0, pol_b);
     ++issued;
   };
-  if (tid == 0)  // every stage starts empty: steps 0 .. kTStages - 1
-    for (int s = 0; s < kTStages && s < nsteps; ++s) fill(s);
+  auto fill_b = [&](int s) {  // every thread's share of the factor's tile
+    const int st = s % kTStages;
+    const int64_t k0 = kz0 + (int64_t)s * kTBK;
+#pragma unroll
+    for (int q = 0; q < kTBK * BN / kTThreads; ++q) {
+      const int e = tid + q * kTThreads, kk = e / BN, nn = e % BN;
+      const bool in = k0 + kk < kz1 && n0 + nn < N;
+      cp_async4(sB + (size_t)st * kTBK * BN + e, in ? B + (k0 + kk) * N + n0 + nn : B, in);
+    }
+    if constexpr (!VEC) {
+#pragma unroll
+      for (int q = 0; q < kTBK * BM / kTThreads; ++q) {
+        const int e = tid + q * kTThreads;
+        const int kk = AK ? e % kTBK : e / BM, mm = AK ? e / kTBK : e % BM;
+        const bool in = k0 + kk < kz1 && m0 + mm < M;
+        const float *src = AK ? A + (m0 + mm) * lda + k0 + kk : A + (k0 + kk) * lda + m0 + mm;
+        float *dst = sA + (size_t)st * BM * kTBK +
+                     (AK ? mm * kTBK + (((kk >> 2) ^ ((mm >> 1) & 3)) << 2) + (kk & 3) : e);
+        cp_async4(dst, in ? src : A, in);
+      }
+    }
+    cp_async_arrive(&full[st]);
+  };
+  // every stage starts empty: steps 0 .. kTStages - 1
+  for (int s = 0; s < kTStages && s < nsteps; ++s) {
+    if (tid == 0) fill(s);
+    if (BCP) fill_b(s);
+  }
 
   const int w = tid >> 5, l = tid & 31, tx = l & 7, ty = w * 4 + (l >> 3);
-  float *kc = corr + (size_t)tid * kTLdc;  // Kahan corrections of the 64 sums
+  float *kc = corr + (size_t)tid * T::kLdc;  // Kahan corrections of the sums
+  if (clus == 0) {
 #pragma unroll
-  for (int e = 0; e < 64; e += 4) *reinterpret_cast<float4 *>(kc + e) = make_float4(0.f, 0.f, 0.f, 0.f);
-  float acc[8][8], hi[8][8];
+    for (int e = 0; e < NE; e += 4) *reinterpret_cast<float4 *>(kc + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // slab sums as packed pairs for the two-wide FMA (the same FMAs in half the
+  // issue slots): output (i, j) is half i & 1 of acc[i / 2][j] (!AK: a pair of
+  // rows arrives as one aligned 8-byte half of a fragment) or half j & 1 of
+  // acc[i][j / 2] (AK)
+  f32x2 acc[NE / 2];
+  float hi[NE];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int e = 0; e < NE / 2; ++e) acc[e] = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = hi[i][j] = 0.f;
+  for (int e = 0; e < NE; ++e) hi[e] = 0.f;
   auto fold = [&]() {  // hi += acc with Kahan's compensation; acc = 0
 #pragma unroll
-    for (int e4 = 0; e4 < 64; e4 += 4) {
+    for (int e4 = 0; e4 < NE; e4 += 4) {
       float4 cv = *reinterpret_cast<const float4 *>(kc + e4);
       float *c = &cv.x;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int e = e4 + u, i = e >> 3, j = e & 7;
-        const float y = acc[i][j] - c[u];
-        const float t = hi[i][j] + y;
-        c[u] = (t - hi[i][j]) - y;
-        hi[i][j] = t;
-        acc[i][j] = 0.f;
+        const int e = e4 + u, i = e / TN, j = e % TN;
+        const f32x2 pr = AK ? acc[i * (TN / 2) + j / 2] : acc[(i / 2) * TN + j];
+        const float a = (AK ? (j & 1) : (i & 1)) ? hi32(pr) : lo32(pr);
+        const float y = a - c[u];
+        const float t = hi[e] + y;
+        c[u] = (t - hi[e]) - y;
+        hi[e] = t;
       }
       *reinterpret_cast<float4 *>(kc + e4) = cv;
     }
+#pragma unroll
+    for (int e = 0; e < NE / 2; ++e) acc[e] = 0;
   };
-  // column-major issue order (each b[j] for 8 FFMAs in a row): 2-3 % faster
-  // than row-major at 96000 x 64000 (fewer operand dispatch stalls)
-  auto fma8x8 = [&](const float (&a)[8], const float4 b0, const float4 b1) {
-    const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+  // row i (0 .. RT - 1) of the thread within the tile
+  auto row_of = [&](int i) { return AK ? ty + 32 * i : (i < 4 ? ty * 4 + i : 128 + ty * 4 + i - 4); };
+  auto keep = [&](int sl) {  // the slab's sums into shared memory; acc = 0
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int e = 0; e < NE; ++e) {
+      const int i = e / TN, j = e % TN;
+      const f32x2 pr = AK ? acc[i * (TN / 2) + j / 2] : acc[(i / 2) * TN + j];
+      corr[(sl * BM + row_of(i)) * BN + simt_col<TN>(tx, j)] =
+          (AK ? (j & 1) : (i & 1)) ? hi32(pr) : lo32(pr);
+    }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int e = 0; e < NE / 2; ++e) acc[e] = 0;
+  };
+  // the thread's TN columns of factor row br
+  auto load_b = [&](const float *br, float (&b)[TN]) {
+    if constexpr (TN == 2) {
+      const float2 v = *reinterpret_cast<const float2 *>(br);
+      b[0] = v.x;
+      b[1] = v.y;
+    } else {
+#pragma unroll
+      for (int q = 0; q < TN / 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4 *>(br + 32 * q);
+        b[4 * q] = v.x;
+        b[4 * q + 1] = v.y;
+        b[4 * q + 2] = v.z;
+        b[4 * q + 3] = v.w;
+      }
+    }
   };
   // AK: rows ty + 32 i share their swizzle (r >> 1) & 3 (32 i leaves those bits alone)
   const int sw = (ty >> 1) & 3;
@@ -842,7 +1013,17 @@ __global__ void __launch_bounds__(kTThreads, 1)
   int slab = 0;
   for (int s = 0; s < nsteps; ++s) {
     const int st = s % kTStages;
-    if (producer && s >= 1 && s - 1 + kTStages < nsteps) {
+    if (BCP && s >= 1 && s - 1 + kTStages < nsteps) {
+      // refill the stage read at step s - 1: every thread waits and copies
+      const int sp = s - 1;
+      if (!mbar_wait(&empty[sp % kTStages], (uint32_t)(sp / kTStages) & 1u, err, limit)) {
+        ok = false;
+        break;
+      }
+      if (tid == 0) fill(sp + kTStages);
+      fill_b(sp + kTStages);
+    }
+    if (!BCP && producer && s >= 1 && s - 1 + kTStages < nsteps) {
       // refill the stage read at step s - 1 (use (s - 1) / kTStages of it)
       const int sp = s - 1;
       int okp = 1;
@@ -858,44 +1039,62 @@ __global__ void __launch_bounds__(kTThreads, 1)
       ok = false;
       break;
     }
-    const float *a = sA + (size_t)st * kTBM * kTBK;
-    const float *b = sB + (size_t)st * kTBK * kTBN + tx * 4;
-    if (AK) {  // a: [256 rows][16 K], 64-byte swizzle
+    const float *a = sA + (size_t)st * BM * kTBK;
+    const float *b = sB + (size_t)st * kTBK * BN + (TN == 2 ? tx * 2 : tx * 4);
+    if constexpr (AK) {  // a: [BM rows][16 K], 64-byte swizzle
 #pragma unroll
       for (int kq = 0; kq < kTBK / 4; ++kq) {
-        float4 av[8];
+        float4 av[RT];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < RT; ++i)
           av[i] = *reinterpret_cast<const float4 *>(a + (ty + 32 * i) * kTBK + ((kq ^ sw) << 2));
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const float *br = b + (kq * 4 + u) * kTBN;
-          const float4 b0 = *reinterpret_cast<const float4 *>(br);
-          const float4 b1 = *reinterpret_cast<const float4 *>(br + 32);
-          float af[8];
+          float bf[TN];
+          load_b(b + (kq * 4 + u) * BN, bf);
+          f32x2 bp[TN / 2];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) af[i] = (&av[i].x)[u];
-          fma8x8(af, b0, b1);
+          for (int j = 0; j < TN / 2; ++j) bp[j] = pack2(bf[2 * j], bf[2 * j + 1]);
+#pragma unroll
+          for (int i = 0; i < RT; ++i) {
+            const float x = (&av[i].x)[u];
+            const f32x2 xx = pack2(x, x);
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j)
+              acc[i * (TN / 2) + j] = fma2(xx, bp[j], acc[i * (TN / 2) + j]);
+          }
         }
       }
-    } else {  // a: [16 K][256 rows]
+    } else {  // a: [16 K][BM rows]
 #pragma unroll
       for (int kk = 0; kk < kTBK; ++kk) {
-        const float4 a0 = *reinterpret_cast<const float4 *>(a + kk * kTBM + ty * 4);
-        const float4 a1 = *reinterpret_cast<const float4 *>(a + kk * kTBM + 128 + ty * 4);
-        const float *br = b + kk * kTBN;
-        const float4 b0 = *reinterpret_cast<const float4 *>(br);
-        const float4 b1 = *reinterpret_cast<const float4 *>(br + 32);
-        const float af[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        fma8x8(af, b0, b1);
+        f32x2 ap[RT / 2];
+#pragma unroll
+        for (int q = 0; q < RT / 4; ++q) {
+          const float4 v = *reinterpret_cast<const float4 *>(a + kk * BM + 128 * q + ty * 4);
+          ap[2 * q] = pack2(v.x, v.y);
+          ap[2 * q + 1] = pack2(v.z, v.w);
+        }
+        float bf[TN];
+        load_b(b + kk * BN, bf);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          const f32x2 bb = pack2(bf[j], bf[j]);
+#pragma unroll
+          for (int i = 0; i < RT / 2; ++i) acc[i * TN + j] = fma2(ap[i], bb, acc[i * TN + j]);
+        }
       }
     }
     mbar_arrive(&empty[st]);
     if (++slab == kTSlabSteps || s + 1 == nsteps) {
-      fold();
+      if (clus > 0)
+        keep(s / kTSlabSteps);
+      else
+        fold();
       slab = 0;
     }
   }
+  if (BCP) cp_async_wait_all();
   if (tid == 0) {
     // the copies thread 0 has put in flight land before the block exits
     for (int st = 0; st < kTStages && st < issued; ++st) {
@@ -903,43 +1102,87 @@ __global__ void __launch_bounds__(kTThreads, 1)
       mbar_wait_drain(&full[st], (uint32_t)(cnt - 1) & 1u, limit);
     }
   }
+  if (clus > 0) {
+    // every block of the cluster takes part in both cluster barriers, also
+    // after a wait ran out; the tile is written only if all of them finished
+    if (!ok) *flag = 0;
+    cluster_sync();
+    bool all = true;
+    for (int z = 0; z < clus; ++z) all = all && ld_cluster_u32(su32(flag), z) == 1u;
+    if (all) {
+      const int per = (BM + clus - 1) / clus;
+      const int ra = (int)blockIdx.z * per, rb = min(BM, ra + per);
+      const int total = (int)((K + kTBK * kTSlabSteps - 1) / (kTBK * kTSlabSteps));
+      for (int e = ra * BN + tid; e < rb * BN; e += kTThreads) {
+        const int64_t gm = m0 + e / BN;
+        const int gn = n0 + e % BN;
+        if (gm >= M || gn >= N) continue;
+        float out = 0.f, h = 0.f, c = 0.f;
+        int in_group = 0;
+        for (int g0 = 0; g0 < total; g0 += 8) {  // eight remote loads in flight
+          float v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int g = g0 + u < total ? g0 + u : total - 1, z = g / nslab;
+            v[u] = __uint_as_float(ld_cluster_u32(su32(corr + (g - z * nslab) * BM * BN + e), z));
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (g0 + u >= total) break;
+            const float y = v[u] - c, t = h + y;
+            c = (t - h) - y;
+            h = t;
+            if (++in_group == group || g0 + u + 1 == total) {
+              out = group < total ? out + (h - c) : h - c;
+              h = c = 0.f;
+              in_group = 0;
+            }
+          }
+        }
+        C[gm * ldc + gn] = out;
+      }
+    }
+    cluster_sync();  // no block's shared memory goes away while a peer reads it
+    return;
+  }
   if (!ok) return;
   C += (int64_t)blockIdx.z * M * ldc;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t gm = m0 + (AK ? ty + 32 * i : (i < 4 ? ty * 4 + i : 128 + ty * 4 + i - 4));
+  for (int i = 0; i < RT; ++i) {
+    const int64_t gm = m0 + row_of(i);
     if (gm >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int gn = n0 + (j < 4 ? tx * 4 + j : 32 + tx * 4 + j - 4);
-      if (gn < N) C[gm * ldc + gn] = hi[i][j] - kc[i * 8 + j];
+    for (int j = 0; j < TN; ++j) {
+      const int gn = n0 + simt_col<TN>(tx, j);
+      if (gn < N) C[gm * ldc + gn] = hi[i * TN + j] - kc[i * TN + j];
     }
   }
 }
 
-// Tensor map of A's tiles for k_gemm_simt_tma: AK, a box of 16 K x 256 rows
-// over A (M x K, ld lda), 64-byte swizzle; !AK, 256 rows x 16 K over A
+// Tensor map of A's tiles for k_gemm_simt_tma: AK, a box of 16 K x bm rows
+// over A (M x K, ld lda), 64-byte swizzle; !AK, bm rows x 16 K over A
 // stored K x M, no swizzle.  FP32, zero fill outside the matrix.
-// Tensor map of the factor's tiles: 64 columns x 16 K rows over the padded
+// Tensor map of the factor's tiles: bn columns x 16 K rows over the padded
 // copy (K x N, ld ldp), no swizzle, zero fill past N and K.
-bool simt_factor_map(CUtensorMap *map, const float *Bp, int64_t K, int N, int ldp) {
+bool simt_factor_map(CUtensorMap *map, const float *Bp, int64_t K, int N, int ldp, int bn) {
   ptx::EncodeTiledFn fn = ptx::encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)K};
   cuuint64_t strides[1] = {(cuuint64_t)ldp * 4};
-  cuuint32_t box[2] = {(cuuint32_t)kTBN, (cuuint32_t)kTBK};
+  cuuint32_t box[2] = {(cuuint32_t)bn, (cuuint32_t)kTBK};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(Bp), dims, strides, box,
             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool simt_map(CUtensorMap *map, const float *A, int64_t lda, int64_t M, int64_t K, bool AK) {
+bool simt_map(CUtensorMap *map, const float *A, int64_t lda, int64_t M, int64_t K, bool AK,
+              int bm) {
   ptx::EncodeTiledFn fn = ptx::encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)(AK ? K : M), (cuuint64_t)(AK ? M : K)};
   cuuint64_t strides[1] = {(cuuint64_t)(lda * 4)};
-  cuuint32_t box[2] = {(cuuint32_t)(AK ? kTBK : kTBM), (cuuint32_t)(AK ? kTBM : kTBK)};
+  cuuint32_t box[2] = {(cuuint32_t)(AK ? kTBK : bm), (cuuint32_t)(AK ? bm : kTBK)};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(A), dims, strides, box,
             estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -952,13 +1195,16 @@ constexpr size_t simt_kahan_bytes() {
   return sizeof(float) * 256 * 2 * ((BM / 16) * (BN / 16) + 1);
 }
 
-// K splits: the smallest S in 1..4 whose block count fills the resident
-// slots (`per_sm` blocks per SM) most evenly, each split at least 8 slabs long.
-int simt_splits(int64_t tiles, int64_t K, int per_sm) {
+int simt_sms() {
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t slots = (int64_t)per_sm * (sms > 0 ? sms : 148);
+  return sms > 0 ? sms : 148;
+}
+
+// K splits: the smallest S in 1..4 whose block count fills the resident
+// slots most evenly, each split at least 8 slabs long.
+int simt_wave_splits(int64_t tiles, int64_t K, int64_t slots) {
   int best = 1;
   double best_eff = 0.0;
   for (int S = 1; S <= 4; ++S) {
@@ -970,14 +1216,77 @@ int simt_splits(int64_t tiles, int64_t K, int per_sm) {
   return best;
 }
 
+// The same, and for few tiles as many splits (of at least a slab) as fill the
+// slots once, up to 16.
+int simt_splits(int64_t tiles, int64_t K, int per_sm) {
+  const int64_t slots = (int64_t)per_sm * simt_sms();
+  if (tiles * 4 > slots) return simt_wave_splits(tiles, K, slots);
+  int64_t S = slots / tiles;
+  if (S > 16) S = 16;
+  if (S > (K + 127) / 128) S = (K + 127) / 128;
+  return S > 1 ? (int)S : 1;
+}
+
 __global__ void k_sum_parts(const float *__restrict__ parts, int S, int64_t len,
                             float *__restrict__ C) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len;
        e += (int64_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < S; ++z) s += parts[z * len + e];
-    C[e] = s;
+    float s = 0.f, r = 0.f;  // r: the additions' errors, kept for many parts
+    for (int z = 0; z < S; ++z) {
+      const float v = parts[z * len + e], t = __fadd_rn(s, v), d = __fsub_rn(t, s);
+      if (S > 4) r += __fadd_rn(__fsub_rn(s, __fsub_rn(t, d)), __fsub_rn(v, d));
+      s = t;
+    }
+    C[e] = s + r;
   }
+}
+
+// One launch of a k_gemm_simt_tma form: grid (gx, gy, S), a cluster per tile
+// when group > 0 (see the kernel).
+template <bool AK, int RT, int BN, bool VEC>
+cudaError_t launch_simt_tma(const CUtensorMap &mapA, const CUtensorMap &mapB, const float *A,
+                            int64_t lda, const float *B, int64_t M, int64_t K, int N, float *C, int ldc, int64_t kchunk, int S,
+                            int group, int *err, cudaStream_t s) {
+  using T = SimtTile<RT, BN>;
+  auto kern = k_gemm_simt_tma<AK, RT, BN, VEC>;
+  const bool clus = group > 0;
+  const size_t smem = T::smem(clus ? (int)(kchunk / (kTBK * kTSlabSteps)) : 0);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((M + T::BM - 1) / T::BM), (unsigned)((N + BN - 1) / BN), (unsigned)S);
+  cfg.blockDim = dim3(kTThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = (unsigned)S;
+  cfg.attrs = at;
+  cfg.numAttrs = clus ? 1 : 0;
+  g_launches += 1;
+  return cudaLaunchKernelEx(&cfg, kern, mapA, mapB, A, lda, B, M, K, N, C, ldc, kchunk, clus ? S : 0, group, err,
+                            fault::wait_cycles(), fault::site() == AUNMF_INJECT_SIMT_WAIT ? 1 : 0);
+}
+
+template <bool AK, int RT, bool VEC>
+cudaError_t launch_simt_tma_n(int BN, const CUtensorMap &mapA, const CUtensorMap &mapB,
+                              const float *A, int64_t lda, const float *B, int64_t M, int64_t K,
+                              int N, float *C, int64_t kchunk, int S, int group, int *err,
+                              cudaStream_t s) {
+  if (BN == 16)
+    return launch_simt_tma<AK, RT, 16, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+  if (BN == 32)
+    return launch_simt_tma<AK, RT, 32, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+  return launch_simt_tma<AK, RT, 64, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+}
+
+cudaError_t sum_parts(const float *parts, int S, int64_t len, float *C, cudaStream_t s) {
+  int64_t nb = (len + 255) / 256;
+  if (nb > 152 * 16) nb = 152 * 16;
+  k_sum_parts<<<(unsigned)nb, 256, 0, s>>>(parts, S, len, C);
+  g_launches += 1;
+  return cudaGetLastError();
 }
 
 template <bool AK>
@@ -985,37 +1294,55 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
                       float *C, float *parts, int *err, cudaStream_t s) {
   constexpr int BM = AUNMF_SIMT_BM, BK = 16, SLAB = 128;
   const int vec = (reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 4 == 0) ? 1 : 0;
-  // TMA-fed form: N > 32, 16-byte aligned rows, coordinates within int32
-  // (parts holds the split partials, then the factor's padded copy)
-  CUtensorMap mapA, mapB;
-  const int ldp = (N + 3) & ~3;
-  float *Bp = parts ? parts + ((4 * M * (int64_t)N + 63) & ~63LL) : nullptr;
-  if (N > 32 && vec && err && parts && M < (1LL << 31) && K < (1LL << 31) &&
-      simt_map(&mapA, A, lda, M, K, AK) && simt_factor_map(&mapB, Bp, K, N, ldp)) {
-    const unsigned gx = (unsigned)((M + kTBM - 1) / kTBM), gy = (unsigned)((N + kTBN - 1) / kTBN);
-    const int S = simt_splits((int64_t)gx * gy, K, 1);
-    const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
-    cudaError_t e = launch_copy2d(B, N, Bp, ldp, K, N, s);
-    if (e != cudaSuccess) return e;
-    auto kern = k_gemm_simt_tma<AK>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTSmem);
-    kern<<<dim3(gx, gy, (unsigned)S), kTThreads, kTSmem, s>>>(
-        mapA, mapB, M, K, N, S > 1 ? parts : C, N, kchunk, err, fault::wait_cycles(),
-        fault::site() == AUNMF_INJECT_SIMT_WAIT ? 1 : 0);
-    g_launches += 1;
-    if (S > 1) {
-      const int64_t len = M * (int64_t)N;
-      int64_t nb = (len + 255) / 256;
-      if (nb > 152 * 16) nb = 152 * 16;
-      k_sum_parts<<<(unsigned)nb, 256, 0, s>>>(parts, S, len, C);
-      g_launches += 1;
-    }
-    return cudaGetLastError();
-  }
-  const unsigned gx = (unsigned)((M + BM - 1) / BM);
   const int BN = N <= 16 ? 16 : (N <= 32 ? 32 : 64);
   const unsigned gy = (unsigned)((N + BN - 1) / BN);
-  const int S = parts ? simt_splits((int64_t)gx * gy, K, 2) : 1;
+  // TMA-fed forms: 16-byte aligned rows, coordinates within int32
+  // (parts holds the split partials, then the factor's padded copy)
+  CUtensorMap mapA, mapB;
+  const int sms = simt_sms();
+  const int64_t tiles4 = (M + 127) / 128 * gy;
+  if (err && parts && M < (1LL << 31) && K < (1LL << 31) && tiles4 * 2 <= sms) {
+    // few output tiles: 128-row tiles, K cut over a cluster of up to 8 blocks
+    // (one block per tile walked all of K, at 77-87 us for 2000 x 1500, k =
+    // 10, on 12-16 of the SMs; the cluster takes 13-15).  The line on K: a
+    // block's slab sums fit beside its ring in shared memory.
+    int64_t S = sms / tiles4;
+    if (S > 8) S = 8;
+    const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
+    S = (K + kchunk - 1) / kchunk;
+    if (kchunk / SLAB * 128 * BN * 4 <= 128 * 1024) {
+      // slabs per K group: where the unclustered forms would split K
+      const int bm = vec && N > 32 ? 256 : BM;
+      const int S0 = simt_wave_splits((M + bm - 1) / bm * gy, K, (vec && N > 32 ? 1 : 2) * (int64_t)sms);
+      const int group = (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB);
+      if (vec && simt_map(&mapA, A, lda, M, K, AK, 128))
+        return launch_simt_tma_n<AK, 4, true>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
+                                              group, err, s);
+      memset(&mapA, 0, sizeof(mapA));
+      return launch_simt_tma_n<AK, 4, false>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
+                                             group, err, s);
+    }
+  }
+  if (vec && err && parts && M < (1LL << 31) && K < (1LL << 31) &&
+      simt_map(&mapA, A, lda, M, K, AK, 256)) {
+    const int ldp = (N + 3) & ~3;
+    const bool direct = ldp == N && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+    const unsigned gx = (unsigned)((M + 255) / 256);
+    const int S = simt_splits((int64_t)gx * gy, K, 1);
+    float *Bp = parts + (((S > 4 ? S : 4) * M * (int64_t)N + 63) & ~63LL);
+    const float *Bs = direct ? B : Bp;
+    if (simt_factor_map(&mapB, Bs, K, N, ldp, BN)) {
+      const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
+      cudaError_t e = direct ? cudaSuccess : launch_copy2d(B, N, Bp, ldp, K, N, s);
+      if (e == cudaSuccess)
+        e = launch_simt_tma_n<AK, 8, true>(BN, mapA, mapB, A, lda, B, M, K, N, S > 1 ? parts : C,
+                                           kchunk, S, 0, err, s);
+      if (e != cudaSuccess || S == 1) return e;
+      return sum_parts(parts, S, M * (int64_t)N, C, s);
+    }
+  }
+  const unsigned gx = (unsigned)((M + BM - 1) / BM);
+  const int S = parts ? simt_wave_splits((int64_t)gx * gy, K, 2 * (int64_t)sms) : 1;
   const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
   float *out = S > 1 ? parts : C;
   const dim3 grid(gx, gy, (unsigned)S);
@@ -1029,13 +1356,7 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
     default: go(k_gemm_simt<BM, 64, BK, AK>, simt_kahan_bytes<BM, 64>()); break;
   }
   g_launches += 1;
-  if (S > 1) {
-    const int64_t len = M * (int64_t)N;
-    int64_t nb = (len + 255) / 256;
-    if (nb > 152 * 16) nb = 152 * 16;
-    k_sum_parts<<<(unsigned)nb, 256, 0, s>>>(parts, S, len, C);
-    g_launches += 1;
-  }
+  if (S > 1) return sum_parts(parts, S, M * (int64_t)N, C, s);
   return cudaGetLastError();
 }
 // G = X^T X for X (rows x k, contiguous rows, k >= 96 and a multiple of 4,
@@ -1053,25 +1374,24 @@ bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partial
       rows >= (1LL << 31))
     return false;
   CUtensorMap mapA, mapB;
-  if (!simt_map(&mapA, X, k, k, rows, false) || !simt_factor_map(&mapB, X, rows, k, k)) return false;
+  using T = SimtTile<8, 64>;
+  if (!simt_map(&mapA, X, k, k, rows, false, T::BM) || !simt_factor_map(&mapB, X, rows, k, k, 64))
+    return false;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms <= 0) sms = 148;
-  const unsigned gx = (unsigned)((k + kTBM - 1) / kTBM), gy = (unsigned)((k + kTBN - 1) / kTBN);
+  const unsigned gx = (unsigned)((k + T::BM - 1) / T::BM), gy = (unsigned)((k + 63) / 64);
   int64_t S = (sms + (int64_t)gx * gy - 1) / ((int64_t)gx * gy);
   S = min(S, (int64_t)max_blocks);
   S = min(S, rows / 512);
   if (S < 1) S = 1;
   const int64_t kchunk = ((rows + S - 1) / S + 127) / 128 * 128;
   S = (rows + kchunk - 1) / kchunk;
-  auto kern = k_gemm_simt_tma<false>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTSmem);
-  kern<<<dim3(gx, gy, (unsigned)S), kTThreads, kTSmem, s>>>(
-      mapA, mapB, k, rows, k, partials, k, kchunk, err, fault::wait_cycles(),
-      fault::site() == AUNMF_INJECT_SIMT_WAIT ? 1 : 0);
-  k_gram_reduce<<<(k * k + 31) / 32, 256, 0, s>>>(partials, (int)S, k, G);
-  g_launches += 2;
+  *status = launch_simt_tma<false, 8, 64, true>(mapA, mapB, X, k, X, k, rows, k, partials, k, kchunk, (int)S, 0, err, s);
+  if (*status != cudaSuccess) return true;
+  k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads((int)S), 0, s>>>(partials, (int)S, k, G);
+  g_launches += 1;
   *status = cudaGetLastError();
   return true;
 }
@@ -1088,7 +1408,11 @@ cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, c
 }
 
 size_t simt_parts_bytes(int64_t rows, int k) {
-  return sizeof(float) * (((4 * (size_t)rows * k + 63) & ~(size_t)63) + (size_t)rows * ((k + 3) & ~3));
+  // four partials of `rows` rows, or 16 of the few tiles that are split further
+  // (then tiles x splits is at most the SM count), and the padded factor
+  const size_t few = (size_t)simt_sms() * 256 + 16 * 256;
+  const size_t most = 4 * (size_t)rows > few ? 4 * (size_t)rows : few;
+  return sizeof(float) * (((most * k + 63) & ~(size_t)63) + (size_t)rows * ((k + 3) & ~3));
 }
 
 // ------------------------------------------------------------------ transpose
@@ -1167,94 +1491,90 @@ __device__ double block_sum_d(double v) {
   return r;
 }
 
-// partials[b] = sum of squares over rows r = b, b + nb, ... of A (m x n, lda)
-__global__ void k_norm2_partial(const float *__restrict__ A, int64_t m, int64_t n, int64_t lda,
-                                double *__restrict__ partials) {
-  // squares of one row are summed in FP32 by each thread (<= n/256 terms),
-  // then added in FP64: FP64 adds at every element would bound the pass by
-  // the FP64 rate instead of HBM
-  // With 16-byte aligned rows the row is read as float4 groups, four groups
-  // in flight per thread (scalar loads left the pass at ~1/3 of HBM speed).
-  double s = 0.0;
-  const bool vec = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (lda & 3) == 0;
-  for (int64_t r = blockIdx.x; r < m; r += gridDim.x) {
-    const float *row = A + r * lda;
-    float sr = 0.f;
-    int64_t c0 = 0;
-    if (vec) {
-      const float4 *row4 = reinterpret_cast<const float4 *>(row);
-      const int64_t n4 = n >> 2;
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
-      int64_t g = threadIdx.x;
-      for (; g + 3 * (int64_t)blockDim.x < n4; g += 4 * (int64_t)blockDim.x) {
-        float4 q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = __ldcs(row4 + g + u * blockDim.x);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          s4[u] = fmaf(q[u].w, q[u].w, fmaf(q[u].z, q[u].z, fmaf(q[u].y, q[u].y, fmaf(q[u].x, q[u].x, s4[u]))));
-      }
-      for (; g < n4; g += blockDim.x) {
-        const float4 q = __ldcs(row4 + g);
-        s4[0] = fmaf(q.w, q.w, fmaf(q.z, q.z, fmaf(q.y, q.y, fmaf(q.x, q.x, s4[0]))));
-      }
-      sr = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-      c0 = n4 << 2;
-    }
-    for (int64_t c = c0 + threadIdx.x; c < n; c += blockDim.x) sr = fmaf(row[c], row[c], sr);
-    s += (double)sr;
+// The same for two sums at once (256 threads).
+__device__ void block_sum_d2(double &a, double &b) {
+  __shared__ double sw[2][8];
+  a = warp_sum_d(a);
+  b = warp_sum_d(b);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __syncthreads();
+  if (lane == 0) {
+    sw[0][w] = a;
+    sw[1][w] = b;
   }
-  s = block_sum_d(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void k_norm2_vec_partial(const float *__restrict__ v, int64_t len,
-                                    double *__restrict__ partials) {
-  double s = 0.0;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const double x = (double)v[e];
-    s = fma(x, x, s);
-  }
-  s = block_sum_d(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// out[0] = ||A||^2 from the partials; out[1] = 0: the products read A itself.
-__global__ void k_sum_partials(const double *__restrict__ partials, int nparts,
-                               double *__restrict__ out) {
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += partials[b];
-  s = block_sum_d(s);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    out[0] = s;
+    a = b = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      a += sw[0][i];
+      b += sw[1][i];
+    }
+  }
+}
+
+// out[0] = ||A||^2 (m x n, lda) from per-block FP64 partials, out[1] = 0 (the
+// products read A itself); the last block adds the partials.  Rows without
+// padding are one vector of m n entries.  Each thread squares 16 entries at a
+// time (four 16-byte loads in flight) in FP32 and adds the 16-term sums in
+// FP64 (an FP64 add per entry would bound the pass); EXACT: the squares of a
+// group are summed as an FP32 pair (~2^-48) instead.  Bound by HBM at large
+// sizes; a block per row with one FP32 chain per thread left 4.6 TB/s.
+template <bool EXACT>
+__global__ void __launch_bounds__(256)
+    k_norm2(const float *__restrict__ A, int64_t m, int64_t n, int64_t lda,
+            double *__restrict__ partials, double *__restrict__ out, unsigned *ticket) {
+  double s = 0.0;
+  const bool flat = lda == n || m == 1;
+  const int64_t rows = flat ? 1 : m, len = flat ? m * n : n;
+  // units of 1024 float4 groups (4096 entries) of a row, block-strided
+  const int64_t per_row = (len + 4095) / 4096, units = rows * per_row;
+  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+    const int64_t r = flat ? 0 : u / per_row, c0 = (flat ? u : u % per_row) * 4096;
+    const float *p = A + r * lda + c0;
+    const int64_t left = len - c0;
+    float v[16];
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0 && left >= 4096) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 x = __ldcs(reinterpret_cast<const float4 *>(p) + threadIdx.x + 256 * q);
+        v[4 * q] = x.x;
+        v[4 * q + 1] = x.y;
+        v[4 * q + 2] = x.z;
+        v[4 * q + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int c = threadIdx.x + 256 * q;
+        v[q] = c < left ? p[c] : 0.f;
+      }
+    }
+    if constexpr (EXACT) {
+      float hi = 0.f, lo = 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) two_fma_acc(v[q], v[q], hi, lo);
+      s += (double)hi + (double)lo;
+    } else {
+      float a = 0.f, b = 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; q += 2) {
+        a = fmaf(v[q], v[q], a);
+        b = fmaf(v[q + 1], v[q + 1], b);
+      }
+      s += (double)(a + b);
+    }
+  }
+  s = block_sum_d(s);
+  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  if (!last_block(ticket)) return;
+  double t = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(&partials[b]);
+  t = block_sum_d(t);
+  if (threadIdx.x == 0) {
+    out[0] = t;
     out[1] = 0.0;
   }
-}
-
-// <P, Q> partials.  With 16-byte aligned arrays, four products at a time are
-// formed and summed in FP32 (round-to-nearest: unbiased, ~1e-7 relative per
-// group, averaging out over the groups) and the group joins an FP64 sum; an
-// FP64 FMA per element bound the pass by the FP64 rate (0.14 ms on the sparse
-// workload's 2.5e7 entries, ~5x its memory time).
-__global__ void k_dot_partial(const float *__restrict__ P, const float *__restrict__ Q,
-                              int64_t len, double *__restrict__ partials) {
-  double s = 0.0;
-  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nt = (int64_t)gridDim.x * blockDim.x;
-  int64_t tail = 0;
-  if (((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Q)) & 15) == 0) {
-    const float4 *P4 = reinterpret_cast<const float4 *>(P), *Q4 = reinterpret_cast<const float4 *>(Q);
-    const int64_t n4 = len >> 2;
-    for (int64_t g = t0; g < n4; g += nt) {
-      const float4 p = P4[g], q = Q4[g];
-      s += (double)fmaf(p.w, q.w, fmaf(p.z, q.z, fmaf(p.y, q.y, p.x * q.x)));
-    }
-    tail = n4 << 2;
-  }
-  for (int64_t e = tail + t0; e < len; e += nt) s = fma((double)P[e], (double)Q[e], s);
-  s = block_sum_d(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
 // relres = sqrt(max(0, ||A||^2 + d - 2 <P, Ht> + <GW, GH>) / ||A||^2), FP64
@@ -1266,36 +1586,56 @@ __global__ void k_dot_partial(const float *__restrict__ P, const float *__restri
 // with the fit residual.  Without d, the mean of the rounding errors (not
 // zero on real value distributions: -8e-6 relative for BF16 on uniform
 // low-rank data) would bias the reported residual by ~1e-3 at relres ~1e-2.
-// <GW, GH> in FP64 by one block: four interleaved chains per thread keep
-// loads in flight (a single chain waited on L2 for every element: 0.58 ms at
-// k = 512), combined in a fixed order.
-__device__ double gram_dot_block(const float *__restrict__ GW, const float *__restrict__ GH,
-                                 int kk) {
-  double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-  const int step = blockDim.x;
-  int e = threadIdx.x;
-  for (; e + 3 * step < kk; e += 4 * step) {
-    q0 = fma((double)GW[e], (double)GH[e], q0);
-    q1 = fma((double)GW[e + step], (double)GH[e + step], q1);
-    q2 = fma((double)GW[e + 2 * step], (double)GH[e + 2 * step], q2);
-    q3 = fma((double)GW[e + 3 * step], (double)GH[e + 3 * step], q3);
+// One launch forms both inner products, <P, Ht> over len entries and <GW, GH>
+// over k^2, as per-block FP64 partials, and its last block adds them in block
+// order and writes the result (a separate one-block kernel took 8-61 us, most
+// of it the k^2 FP64 products on one SM).  <P, Ht>: with 16-byte aligned
+// arrays, four products at a time are formed and summed in FP32
+// (round-to-nearest: unbiased, ~1e-7 relative per group, averaging out over
+// the groups) and the group joins an FP64 sum; an FP64 FMA per element bound
+// the pass by the FP64 rate.
+// LOSS: *loss = 0.5 (||A||^2 + d - 2 <P, Ht> + <GW, GH>), not clamped.
+template <bool LOSS>
+__global__ void __launch_bounds__(256)
+    k_residual(const float *__restrict__ P, const float *__restrict__ Q, int64_t len,
+               const float *__restrict__ GW, const float *__restrict__ GH, int kk,
+               const double *__restrict__ n2a, double *__restrict__ partials, unsigned *ticket,
+               double *__restrict__ relres, DevCounters *ctr, double *__restrict__ last) {
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t nt = (int64_t)gridDim.x * blockDim.x;
+  double s = 0.0, q = 0.0;
+  int64_t tail = 0;
+  if (((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Q)) & 15) == 0) {
+    const float4 *P4 = reinterpret_cast<const float4 *>(P), *Q4 = reinterpret_cast<const float4 *>(Q);
+    const int64_t n4 = len >> 2;
+#pragma unroll 4
+    for (int64_t g = t0; g < n4; g += nt) {
+      const float4 x = P4[g], y = Q4[g];
+      s += (double)fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, x.x * y.x)));
+    }
+    tail = n4 << 2;
   }
-  for (; e < kk; e += step) q0 = fma((double)GW[e], (double)GH[e], q0);
-  return block_sum_d((q0 + q1) + (q2 + q3));
-}
-
-__global__ void __launch_bounds__(1024) k_relres_final(const double *__restrict__ partials, int nparts,
-                               const float *__restrict__ GW, const float *__restrict__ GH, int k,
-                               const double *__restrict__ n2a, double *__restrict__ relres,
-                               DevCounters *ctr, double *last) {
-  double cross = 0.0;
-  for (int b = threadIdx.x; b < nparts; b += blockDim.x) cross += partials[b];
-  cross = block_sum_d(cross);
-  const double quad = gram_dot_block(GW, GH, k * k);
+  for (int64_t e = tail + t0; e < len; e += nt) s = fma((double)P[e], (double)Q[e], s);
+  for (int64_t e = t0; e < kk; e += nt) q = fma((double)GW[e], (double)GH[e], q);
+  block_sum_d2(s, q);
   if (threadIdx.x == 0) {
-    const double a2 = n2a[0];
-    double r2 = (a2 + n2a[1]) - 2.0 * cross + quad;
-    if (r2 < 0.0) r2 = 0.0;
+    partials[2 * blockIdx.x] = s;
+    partials[2 * blockIdx.x + 1] = q;
+  }
+  if (!last_block(ticket)) return;
+  double cross = 0.0, quad = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+    cross += __ldcg(&partials[2 * b]);
+    quad += __ldcg(&partials[2 * b + 1]);
+  }
+  block_sum_d2(cross, quad);
+  if (threadIdx.x != 0) return;
+  const double a2 = n2a[0];
+  const double f = (a2 + n2a[1]) - 2.0 * cross + quad;
+  if constexpr (LOSS) {
+    *last = 0.5 * f;
+  } else {
+    const double r2 = f < 0.0 ? 0.0 : f;
     const double rr = a2 > 0.0 ? sqrt(r2 / a2) : 0.0;
     if (!isfinite(rr)) ctr->nonfinite += 1;
     if (relres) relres[ctr->iter] = rr;
@@ -1303,51 +1643,46 @@ __global__ void __launch_bounds__(1024) k_relres_final(const double *__restrict_
     if (last) *last = rr;
   }
 }
-// loss = 0.5 (||A||^2 + d - 2 <P, Ht> + <GW, GH>), FP64 (not clamped); d as
-// for the residual.
-__global__ void __launch_bounds__(1024) k_loss_final(const double *__restrict__ partials, int nparts,
-                             const float *__restrict__ GW, const float *__restrict__ GH, int k,
-                             const double *__restrict__ n2a, double *__restrict__ loss) {
-  double cross = 0.0;
-  for (int b = threadIdx.x; b < nparts; b += blockDim.x) cross += partials[b];
-  cross = block_sum_d(cross);
-  const double quad = gram_dot_block(GW, GH, k * k);
-  if (threadIdx.x == 0) *loss = 0.5 * ((n2a[0] + n2a[1]) - 2.0 * cross + quad);
+
+// Blocks of a residual pass: one per 4096 entries, at most nparts.
+int residual_blocks(int64_t len, int nparts) {
+  const int64_t nb = (len + 4095) / 4096;
+  return (int)(nb < 1 ? 1 : (nb > nparts ? nparts : nb));
 }
 }  // namespace
 
 cudaError_t launch_loss(const float *P, const float *Ht, int64_t len, const float *GW,
                         const float *GH, int k, const double *n2a, double *partials, int nparts,
-                        double *loss, cudaStream_t s) {
-  k_dot_partial<<<nparts, 256, 0, s>>>(P, Ht, len, partials);
-  k_loss_final<<<1, 1024, 0, s>>>(partials, nparts, GW, GH, k, n2a, loss);
-  g_launches += 2;
+                        double *loss, unsigned *ticket, cudaStream_t s) {
+  k_residual<true><<<residual_blocks(len, nparts), 256, 0, s>>>(P, Ht, len, GW, GH, k * k, n2a,
+                                                               partials, ticket, nullptr, nullptr,
+                                                               loss);
+  g_launches += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_norm2(const float *A, int64_t m, int64_t n, int64_t lda, double *partials,
-                         int nparts, double *out, cudaStream_t s) {
-  k_norm2_partial<<<nparts, 256, 0, s>>>(A, m, n, lda, partials);
-  k_sum_partials<<<1, 256, 0, s>>>(partials, nparts, out);
-  g_launches += 2;
+                         int nparts, double *out, unsigned *ticket, cudaStream_t s) {
+  k_norm2<false><<<residual_blocks(m * n, nparts), 256, 0, s>>>(A, m, n, lda, partials, out, ticket);
+  g_launches += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_norm2_vec(const float *v, int64_t len, double *partials, int nparts,
-                             double *out, cudaStream_t s) {
-  k_norm2_vec_partial<<<nparts, 256, 0, s>>>(v, len, partials);
-  k_sum_partials<<<1, 256, 0, s>>>(partials, nparts, out);
-  g_launches += 2;
+                             double *out, unsigned *ticket, cudaStream_t s) {
+  k_norm2<true><<<residual_blocks(len, nparts), 256, 0, s>>>(v, 1, len, len, partials, out, ticket);
+  g_launches += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_relres(const float *P, const float *Ht, int64_t len, const float *GW,
                           const float *GH, int k, const double *n2a, double *partials,
                           int nparts, double *relres_dev, DevCounters *ctr, double *last,
-                          cudaStream_t s) {
-  k_dot_partial<<<nparts, 256, 0, s>>>(P, Ht, len, partials);
-  k_relres_final<<<1, 1024, 0, s>>>(partials, nparts, GW, GH, k, n2a, relres_dev, ctr, last);
-  g_launches += 2;
+                          unsigned *ticket, cudaStream_t s) {
+  k_residual<false><<<residual_blocks(len, nparts), 256, 0, s>>>(P, Ht, len, GW, GH, k * k, n2a,
+                                                                partials, ticket, relres_dev, ctr,
+                                                                last);
+  g_launches += 1;
   return cudaGetLastError();
 }
 

@@ -761,13 +761,32 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// out[0] = sum of the even partials (||A||^2), out[1] = 2 x the odd ones.
-__global__ void k_sum_partials_d(const double *__restrict__ part, int np, double *__restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0, d = 0.0;
-    for (int i = 0; i < np; ++i) {
-      s += part[2 * i];
-      d += part[2 * i + 1];
+// out[0] = sum of the even partials (||A||^2), out[1] = 2 x the odd ones; one
+// block, thread t adding partials t, t + 256, ... and thread 0 the warps' sums
+// (one thread adding all of them took 0.13 ms for 1,216 partials).
+__global__ void __launch_bounds__(256)
+    k_sum_partials_d(const double *__restrict__ part, int np, double *__restrict__ out) {
+  __shared__ double ws[2][8];
+  double s = 0.0, d = 0.0;
+  for (int i = threadIdx.x; i < np; i += 256) {
+    s += part[2 * i];
+    d += part[2 * i + 1];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    d += __shfl_xor_sync(0xffffffffu, d, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    ws[0][threadIdx.x >> 5] = s;
+    ws[1][threadIdx.x >> 5] = d;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s = d = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      s += ws[0][w];
+      d += ws[1][w];
     }
     out[0] = s;
     out[1] = 2.0 * d;
@@ -890,7 +909,7 @@ cudaError_t launch_prepare(const float *A, int64_t m, int64_t n, int64_t lda, vo
       k_prepare<float, false><<<nb, 256, 0, s>>>(A, m, n, lda, (float *)X, ldx, (float *)Xt, ldxt,
                                                  part);
   }
-  k_sum_partials_d<<<1, 32, 0, s>>>(part, nb, norm2);
+  k_sum_partials_d<<<1, 256, 0, s>>>(part, nb, norm2);
   g_launches += 2;
   return cudaGetLastError();
 }

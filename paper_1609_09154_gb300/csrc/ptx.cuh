@@ -94,6 +94,66 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   return p;
 }
 
+// ---- thread-block clusters: barrier over all threads of the cluster (writes
+// before it are visible after it), and a load from the shared memory of the
+// cluster's block `rank` at this block's address `saddr`.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::
+                   : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t saddr, int rank) {
+  uint32_t v;
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %1, %2;\n\t"
+      "ld.shared::cluster.u32 %0, [ra];\n\t}"
+      : "=r"(v)
+      : "r"(saddr), "r"(rank)
+      : "memory");
+  return v;
+}
+
+// 4-byte asynchronous copy into shared memory (zero when !valid: nothing is
+// read), and the arrival on `b` (one of its expected count) once all copies
+// this thread has issued so far have landed.
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(su32(dst)), "l"(src),
+               "r"(valid ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t *b) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// ---- packed FP32 pairs: one instruction does two independent FP32
+// operations, each rounded as the scalar one (half the issue slots; the FMA
+// rate itself is the same: 36.5 against 38.9 T FMA/s measured).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float lo32(f32x2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi32(f32x2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // ---------------------------------------------------------------- host
 // The driver's cuTensorMapEncodeTiled, looked up once through the runtime's
 // entry-point query (no link-time dependency on libcuda); null if absent.
