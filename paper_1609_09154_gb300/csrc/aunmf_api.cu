@@ -174,6 +174,8 @@ struct RunCtx {
   int64_t ldx, ldat;
   void *Hk, *Wt;
   int64_t ldh, ldw;
+  bool direct;       // products round A's tiles themselves (k_direct.cu): no Ax, At
+  bool norm_in_wta;  // direct: the next W^T A product also forms n2a
   float *parts;
   float *tcacc;  // k > 64: the products' per-CTA partial sums (null: added into parts)
   int *err;
@@ -269,8 +271,12 @@ cudaError_t product_aht(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   {
     PhaseTimer t(c, s, kPhAht);
-    e = tc::launch_gemm(c.Ax, A->m, A->n, c.ldx, c.Hk, c.k, c.ldh, split, bf,
-                        S == 1 ? c.PW : c.parts, S, c.tcacc, c.err, s);
+    if (c.direct)
+      e = tc::launch_gemm_direct(true, A->dense, A->m, A->n, A->lda, c.Hk, c.k, c.ldh, bf,
+                                 S == 1 ? c.PW : c.parts, S, nullptr, nullptr, c.err, s);
+    else
+      e = tc::launch_gemm(c.Ax, A->m, A->n, c.ldx, c.Hk, c.k, c.ldh, split, bf,
+                          S == 1 ? c.PW : c.parts, S, c.tcacc, c.err, s);
     if (e != cudaSuccess) return e;
   }
   if (S > 1) {
@@ -304,8 +310,13 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   {
     PhaseTimer t(c, s, kPhWta);
-    e = tc::launch_gemm(c.At, A->n, A->m, c.ldat, c.Wt, c.k, c.ldw, split, bf,
-                        S == 1 ? c.PHt : c.parts, S, c.tcacc, c.err, s);
+    if (c.direct)
+      e = tc::launch_gemm_direct(false, A->dense, A->m, A->n, A->lda, c.Wt, c.k, c.ldw, bf,
+                                 S == 1 ? c.PHt : c.parts, S, c.dpart,
+                                 c.norm_in_wta ? c.n2a : nullptr, c.err, s);
+    else
+      e = tc::launch_gemm(c.At, A->n, A->m, c.ldat, c.Wt, c.k, c.ldw, split, bf,
+                          S == 1 ? c.PHt : c.parts, S, c.tcacc, c.err, s);
     if (e != cudaSuccess) return e;
   }
   if (S > 1) {
@@ -315,10 +326,13 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   return cudaSuccess;
 }
 
-// Workspace and one-off layout copies of A for the tensor-core products:
-// X of A H^T is A and X of W^T A is A^T, both rounded to nearest TF32 (kept
-// in FP32 containers) or BF16, with 16-byte aligned rows.
-int prepare_tc(aunmf_handle *h, RunCtx &c, cudaStream_t s);
+// Workspace of the tensor-core products and, unless c.direct, one-off layout
+// copies of A: X of A H^T is A and X of W^T A is A^T, both rounded to nearest
+// TF32 (kept in FP32 containers) or BF16, with 16-byte aligned rows.  `what`:
+// the products that follow (kPrepAht, kPrepWta), and whether ||A||^2 and the
+// rounding term are wanted now (kPrepNorm).
+enum { kPrepAht = 1, kPrepWta = 2, kPrepNorm = 4 };
+int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s);
 // CSC copy of a sparse A (setup of the W^T A product).
 int prepare_sparse(aunmf_handle *h, RunCtx &c, cudaStream_t s);
 
@@ -423,7 +437,7 @@ int check_run_args(const aunmf_matrix *A, int k, int algo, int iters, const floa
     if (rc_ != AUNMF_OK) return rc_;       \
   } while (0)
 
-int prepare_tc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
+int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s) {
   const aunmf_matrix *A = c.A;
   const int64_t m = A->m, n = A->n;
   const int k = c.k;
@@ -431,10 +445,8 @@ int prepare_tc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   const size_t esz = bf ? 2 : 4;
   c.ldh = tc::copy_ld(n);
   c.ldw = tc::copy_ld(m);
-  c.ldat = tc::copy_ld(m);
-  ENS_TC(h, h->Hk, esz * tc::factor_elems(n, k));
-  ENS_TC(h, h->Wt, esz * tc::factor_elems(m, k));
-  ENS_TC(h, h->At, esz * (size_t)n * c.ldat);
+  if (what & kPrepAht) ENS_TC(h, h->Hk, esz * tc::factor_elems(n, k));
+  if (what & kPrepWta) ENS_TC(h, h->Wt, esz * tc::factor_elems(m, k));
   const size_t parts = tc::parts_elems(m > n ? m : n, k);
   ENS_TC(h, h->parts, sizeof(float) * parts);
   ENS_TC(h, h->err, sizeof(int));
@@ -444,22 +456,32 @@ int prepare_tc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   c.Hk = h->Hk.p;
   c.Wt = h->Wt.p;
-  c.At = h->At.p;
   c.parts = P<float>(h->parts);
   c.err = P<int>(h->err);
   cudaError_t e = cudaMemsetAsync(c.err, 0, sizeof(int), s);
   if (e != cudaSuccess) return fail_cuda(h, e, "cudaMemsetAsync(err)");
-  // X of A H^T: A rounded to nearest TF32 / BF16 with 16-byte aligned rows;
-  // X of W^T A: the same, transposed; and ||A||^2, all in one pass over A
-  c.ldx = tc::copy_ld(n);
-  ENS_TC(h, h->Ax, esz * (size_t)m * c.ldx);
   ENS_TC(h, h->dpart, dpart_bytes(h));
   ENS_TC(h, h->n2a, 2 * sizeof(double));
-  c.Ax = h->Ax.p;
   c.dpart = P<double>(h->dpart);
   if (!c.n2a) c.n2a = P<double>(h->n2a);
-  e = tc::launch_prepare(A->dense, m, n, A->lda, h->Ax.p, c.ldx, h->At.p, c.ldat, bf, c.dpart,
-                         c.n2a, s);
+  if (c.direct) {
+    if (what & kPrepNorm) {  // the layout pass without its outputs: the same sums
+      e = tc::launch_prepare(A->dense, m, n, A->lda, nullptr, n, nullptr, m, bf, c.dpart, c.n2a, s);
+      if (e != cudaSuccess) return fail_cuda(h, e, "norm of A");
+    }
+    return AUNMF_OK;
+  }
+  // A rounded to nearest TF32 / BF16 with 16-byte aligned rows, the same
+  // transposed, and ||A||^2, all in one pass over A
+  c.ldx = tc::copy_ld(n);
+  c.ldat = tc::copy_ld(m);
+  if (what & kPrepAht) ENS_TC(h, h->Ax, esz * (size_t)m * c.ldx);
+  if (what & kPrepWta) ENS_TC(h, h->At, esz * (size_t)n * c.ldat);
+  c.Ax = h->Ax.p;
+  c.At = h->At.p;
+  e = tc::launch_prepare(A->dense, m, n, A->lda, what & kPrepAht ? h->Ax.p : nullptr, c.ldx,
+                         what & kPrepWta ? h->At.p : nullptr, c.ldat, bf, c.dpart,
+                         what & kPrepNorm ? c.n2a : nullptr, s);
   if (e != cudaSuccess) return fail_cuda(h, e, "layout copies of A");
   return AUNMF_OK;
 }
@@ -614,10 +636,11 @@ int aunmf_check_status(int *site) {
   return AUNMF_OK;
 }
 
-int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters,
-              const float *W0, const float *H0, float *W, float *H, double *relres,
-              const aunmf_options *opt, aunmf_info *info) {
-  if (!h) return AUNMF_E_INVAL;
+// aunmf_run; a_host: A->dense is page-locked host memory, read over the host
+// link (once, by the layout pass).
+static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters,
+                    const float *W0, const float *H0, float *W, float *H, double *relres,
+                    const aunmf_options *opt, aunmf_info *info, bool a_host) {
   int rc = check_run_args(A, k, algo, iters, W0, H0, W, H, opt);
   if (rc != AUNMF_OK) return rc;
   aunmf_options o{};
@@ -709,7 +732,15 @@ int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters
     CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (o.prec != AUNMF_FP32) {
-    int prc = prepare_tc(h, c, s);
+    // Short TF32 runs (k <= 64) read A itself and save the layout pass (12 m n
+    // bytes; 14.4 against 3.7 ms for the norm alone at 96000 x 64000), at
+    // products 8 % slower than on the copies there, up to 25 % where the tiles
+    // fill the SMs badly (24000 x 16000, where 10 iterations with the copies
+    // take 7.53 ms, without 7.37): the line is at 12 iterations.  BF16 copies
+    // halve every product's bytes and repay the pass from the second iteration
+    // on.  A in host memory is read once, into copies.
+    c.direct = use_split(k) && !a_host && iters <= (o.prec == AUNMF_TF32 ? 12 : 1);
+    int prc = prepare_tc(h, c, kPrepAht | kPrepWta | kPrepNorm, s);
     if (prc != AUNMF_OK) return prc;
   } else if (A->dense) {
     ENS(h, h->parts, simt_parts_bytes(m > n ? m : n, k));
@@ -807,6 +838,19 @@ int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters
   return AUNMF_OK;
 }
 
+int aunmf_run(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int iters,
+              const float *W0, const float *H0, float *W, float *H, double *relres,
+              const aunmf_options *opt, aunmf_info *info) {
+  if (!h) return AUNMF_E_INVAL;
+  bool a_host = false;
+  if (A && A->dense && opt && opt->prec != AUNMF_FP32) {
+    cudaPointerAttributes at{};
+    a_host = cudaPointerGetAttributes(&at, A->dense) == cudaSuccess && at.type == cudaMemoryTypeHost;
+    cudaGetLastError();
+  }
+  return run_impl(h, A, k, algo, iters, W0, H0, W, H, relres, opt, info, a_host);
+}
+
 int aunmf_run_host(aunmf_handle *h, const float *A, int64_t m, int64_t n, int64_t lda, int k,
                    int algo, int iters, const float *W0, const float *H0, float *W, float *H,
                    double *relres, const aunmf_options *opt, aunmf_info *info) {
@@ -852,7 +896,7 @@ int aunmf_run_host(aunmf_handle *h, const float *A, int64_t m, int64_t n, int64_
   M.n = n;
   M.dense = Ad;
   M.lda = ldd;
-  int rc = aunmf_run(h, &M, k, algo, iters, dW, dH, dW, dH, relres, opt, info);
+  int rc = run_impl(h, &M, k, algo, iters, dW, dH, dW, dH, relres, opt, info, Ad != P<float>(h->hA));
   if (rc != AUNMF_OK && rc != AUNMF_E_NOCONVERGE) return rc;
   CK(h, cudaMemcpyAsync(W, dW, sizeof(float) * m * k, cudaMemcpyDeviceToHost, s));
   CK(h, cudaMemcpyAsync(H, dH, sizeof(float) * k * n, cudaMemcpyDeviceToHost, s));
@@ -903,7 +947,8 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
   c.PW = Pout;
   CK(h, launch_transpose(H, k, n, c.Ht, h->stream));
   if (prec != AUNMF_FP32) {
-    int rc = prepare_tc(h, c, h->stream);
+    c.direct = use_split(k);
+    int rc = prepare_tc(h, c, kPrepAht, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
     ENS(h, h->parts, simt_parts_bytes(A->m > A->n ? A->m : A->n, k));
@@ -933,7 +978,8 @@ int aunmf_wta(aunmf_handle *h, const aunmf_matrix *A, const float *W, int k, int
   c.W = const_cast<float *>(W);
   c.PHt = P<float>(h->PHt);
   if (prec != AUNMF_FP32) {
-    int rc = prepare_tc(h, c, h->stream);
+    c.direct = use_split(k);
+    int rc = prepare_tc(h, c, kPrepWta, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
     ENS(h, h->parts, simt_parts_bytes(A->m > n ? A->m : n, k));
@@ -1114,8 +1160,10 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
 
 // ------------------------------------------------------------ loss / gradient
 namespace {
+// what: the products that follow (kPrepAht, kPrepWta), and kPrepNorm if n2a is
+// wanted (with a W^T A product to follow).
 int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, const float *H,
-               int prec, RunCtx &c) {
+               int prec, int what, RunCtx &c) {
   if (!valid_matrix(A) || !W || !H || k < 1 || k > AUNMF_K_MAX) return AUNMF_E_INVAL;
   if (prec < AUNMF_FP32 || prec > AUNMF_BF16) return AUNMF_E_INVAL;
   if (!A->dense && prec != AUNMF_FP32) return AUNMF_E_UNSUPPORTED;
@@ -1148,16 +1196,19 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
   cudaStream_t s = h->stream;
   CK(h, launch_transpose(H, k, n, c.Ht, s));
   if (prec != AUNMF_FP32) {
-    int rc = prepare_tc(h, c, s);  // also writes ||A||^2
+    c.direct = use_split(k);
+    c.norm_in_wta = c.direct && (what & kPrepNorm);
+    int rc = prepare_tc(h, c, c.norm_in_wta ? what & ~kPrepNorm : what, s);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
+    if (what & kPrepNorm)
+      CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
     ENS(h, h->parts, simt_parts_bytes(m > n ? m : n, k));
     c.parts = P<float>(h->parts);
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));
-  } else {
+  } else if (what & kPrepNorm) {
     CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (!A->dense) {
@@ -1172,7 +1223,7 @@ int aunmf_loss_fwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
                    int prec, double *loss, float *WtA) {
   if (!h || !loss) return AUNMF_E_INVAL;
   RunCtx c{};
-  int rc = loss_setup(h, A, k, W, H, prec, c);
+  int rc = loss_setup(h, A, k, W, H, prec, kPrepWta | kPrepNorm, c);
   if (rc != AUNMF_OK) return rc;
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;
@@ -1189,7 +1240,7 @@ int aunmf_loss_bwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
                    int prec, const float *WtA, const float *grad_out, float *dW, float *dH) {
   if (!h || (!dW && !dH)) return AUNMF_E_INVAL;
   RunCtx c{};
-  int rc = loss_setup(h, A, k, W, H, prec, c);
+  int rc = loss_setup(h, A, k, W, H, prec, (dW ? kPrepAht : 0) | (dH && !WtA ? kPrepWta : 0), c);
   if (rc != AUNMF_OK) return rc;
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;

@@ -1491,7 +1491,7 @@ __device__ double block_sum_d(double v) {
   return r;
 }
 
-// The same for two sums at once (256 threads).
+// Two such sums at once (256 threads).
 __device__ void block_sum_d2(double &a, double &b) {
   __shared__ double sw[2][8];
   a = warp_sum_d(a);
@@ -1513,8 +1513,8 @@ __device__ void block_sum_d2(double &a, double &b) {
   }
 }
 
-// out[0] = ||A||^2 (m x n, lda) from per-block FP64 partials, out[1] = 0 (the
-// products read A itself); the last block adds the partials.  Rows without
+// out[0] = ||A||^2 (m x n, lda) from per-block FP64 partials, out[1] = 0 for
+// products that read A itself; the last block adds the partials.  Rows without
 // padding are one vector of m n entries.  Each thread squares 16 entries at a
 // time (four 16-byte loads in flight) in FP32 and adds the 16-term sums in
 // FP64 (an FP64 add per entry would bound the pass); EXACT: the squares of a

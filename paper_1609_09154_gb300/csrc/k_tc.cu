@@ -51,6 +51,7 @@
 #include "internal.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
+#include "tcgen.cuh"
 
 namespace aunmf {
 namespace tc {
@@ -97,86 +98,6 @@ __device__ __forceinline__ float ld_keep(const float *p, uint64_t pol) {
 __device__ __forceinline__ void st_keep(float *p, float v, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(v), "l"(pol) : "memory");
 }
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(slot)),
-               "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-               : "memory");
-}
-template <bool BF16>
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                    uint32_t acc) {
-  if constexpr (BF16) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-  }
-}
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
-      : "memory");
-}
-// 16 columns of the thread's TMEM lane into r[0..15] without waiting; the
-// values may be read only after tmem_wait_ld().
-__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t *r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-// Waits for the thread's outstanding tcgen05.ld; the empty volatile asm per
-// register orders every later use of r[0..n) after the wait.
-template <int N>
-__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[N]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
-}
-
-// Shared-memory matrix descriptor for a K-major tile in the canonical
-// 128-byte-swizzled layout written by TMA (rows of 128 B, 8-row groups of
-// 1024 B): start address >> 4, leading offset 16 B (unused for this layout),
-// stride offset 1024 B between 8-row groups, descriptor version 1, swizzle
-// mode 2 (128 B).
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(16u >> 4) << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// Instruction descriptor (kind::tf32 / kind::f16): FP32 accumulator, A and
-// B of the same type (TF32 = 2 or BF16 = 1), both K-major, N >> 3 at bit
-// 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t idesc(bool bf16, int M, int N) {
-  return (1u << 4) | ((bf16 ? 1u : 2u) << 7) | ((bf16 ? 1u : 2u) << 10) |
-         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
 // One product C (M x k) = X (M x K) * F (k x K)^T of a launch.  A launch
 // runs one problem (passed by value) or a group of problems (a device array,
 // e.g. all instances of a batch); work units are numbered across the group.
@@ -567,15 +488,7 @@ __global__ void k_sum_splits(const float *__restrict__ parts, int S, int64_t len
   }
 }
 
-// out (cols x ldo) = in (rows x cols, ld ldi)^T, converting to T (float or bf16).
-// FP32 -> TF32 with round-to-nearest (the tensor core would otherwise drop the
-// low 13 mantissa bits, a bias toward zero that does not average out on
-// nonnegative data); the result is an FP32 bit pattern with those bits zero.
-__device__ __forceinline__ float round_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
+// FP32 rounded to T: TF32 in an FP32 container, or BF16.
 template <class T>
 __device__ __forceinline__ T cvt(float x);
 template <>
@@ -644,7 +557,8 @@ __global__ void k_split_transpose(const float *__restrict__ in, int64_t rows, in
 }
 
 // One pass over A (m x n, lda) for the tensor-core runs: writes the rounded
-// copy X (m x n, ld ldx), the rounded transposed copy Xt (n x m, ld ldxt) and
+// copy X (m x n, ld ldx; null: not), the rounded transposed copy Xt (n x m, ld
+// ldxt; null: not) and
 // per-block partial sums of a_ij^2 and of a_ij (round(a_ij) - a_ij) (FP64;
 // each thread first adds the 16 terms it holds in FP32).  64 x 64 tiles: thread (ty, c4) loads the four
 // 16-byte pieces A[r0 + ty + 16 i][c0 + 4 c4 .. +3], i < 4, before storing
@@ -700,6 +614,7 @@ __global__ void __launch_bounds__(256)
       }
     acc += (double)sq;
     acc_d += (double)sd;
+    if (!X && !Xt) continue;
     __syncthreads();  // previous tile's transposed reads are done
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -707,7 +622,7 @@ __global__ void __launch_bounds__(256)
       const int64_t r = r0 + y;
 #pragma unroll
       for (int u = 0; u < 4; ++u) t[y][4 * c4 + u] = v[i][u];
-      if (r < m) {
+      if (X && r < m) {
         T *dst = X + r * ldx + c;
         if (c + 3 < n) {
           store4<T>(dst, v[i][0], v[i][1], v[i][2], v[i][3]);
@@ -718,6 +633,7 @@ __global__ void __launch_bounds__(256)
         }
       }
     }
+    if (!Xt) continue;
     __syncthreads();
     // transposed: thread -> output row cc = c0 + threadIdx.x / 4, 16 entries
     const int oc = threadIdx.x >> 2, seg = (threadIdx.x & 3) * 16;
@@ -868,6 +784,11 @@ int check(int64_t m, int64_t n, int64_t lda, int k, int prec, const float *A) {
   return AUNMF_OK;
 }
 
+bool factor_map(CUtensorMap *map, const void *Y, bool bf16, int64_t rows, int64_t K, int64_t ld,
+                int box_rows) {
+  return make_map(map, Y, bf16, rows, K, ld, box_rows);
+}
+
 size_t factor_elems(int64_t rows, int k) { return (size_t)2 * k * pad_to(rows, 8); }
 int64_t copy_ld(int64_t cols) { return pad_to(cols, 8); }
 size_t parts_elems(int64_t M, int k) { return (size_t)4 * M * k; }
@@ -909,8 +830,13 @@ cudaError_t launch_prepare(const float *A, int64_t m, int64_t n, int64_t lda, vo
       k_prepare<float, false><<<nb, 256, 0, s>>>(A, m, n, lda, (float *)X, ldx, (float *)Xt, ldxt,
                                                  part);
   }
+  g_launches += 1;
+  return norm2 ? launch_sum_norm(part, nb, norm2, s) : cudaGetLastError();
+}
+
+cudaError_t launch_sum_norm(const double *part, int nb, double *norm2, cudaStream_t s) {
   k_sum_partials_d<<<1, 256, 0, s>>>(part, nb, norm2);
-  g_launches += 2;
+  g_launches += 1;
   return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
 // tc.cuh -- tensor-core (tcgen05) products with A: host-side launchers.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -26,8 +27,11 @@ cudaError_t launch_transpose_to(const float *in, int64_t rows, int64_t cols, int
                                 int64_t ldo, bool bf16, cudaStream_t s);
 // One pass over A: X = round(A) (m x n, ldx), Xt = round(A)^T (n x m, ldxt),
 // norm2[0] = sum a_ij^2 and norm2[1] = 2 sum a_ij (round(a_ij) - a_ij) (FP64),
-// via 2 x prepare_blocks() partials in part.
+// via 2 x prepare_blocks() partials in part.  X, Xt or norm2 may be null: that
+// output is left out.
 int prepare_blocks();
+// norm2[0], norm2[1] = the sums of nb pairs of partials, the second doubled.
+cudaError_t launch_sum_norm(const double *part, int nb, double *norm2, cudaStream_t s);
 cudaError_t launch_prepare(const float *A, int64_t m, int64_t n, int64_t lda, void *X, int64_t ldx,
                            void *Xt, int64_t ldxt, bool bf16, double *part, double *norm2,
                            cudaStream_t s);
@@ -54,6 +58,17 @@ cudaError_t launch_split_transpose(const float *in, int64_t rows, int k, int64_t
 // problem_bytes()-sized slot (64-byte aligned) of a host array that the
 // caller copies to device memory; unit0 numbers the problems' work units
 // consecutively (no K splits: each problem writes C directly).
+// Tensor map of a K-major factor copy (rows x K, ld elements): boxes of 128
+// bytes by box_rows, 128-byte swizzle.
+bool factor_map(CUtensorMap *map, const void *Y, bool bf16, int64_t rows, int64_t K, int64_t ld,
+                int box_rows);
+// The same product straight from the FP32 A (m x n, lda, in device memory),
+// k <= 64: aht, C = A Ht (m x k); else C = A^T W (n x k).  Y: the factor's
+// hi/lo split.  norm2 (!aht only, may be null): also the sums of
+// launch_prepare, via 2 x (SM count) partials in part.
+cudaError_t launch_gemm_direct(bool aht, const float *A, int64_t m, int64_t n, int64_t lda,
+                               const void *Y, int k, int64_t ldy, bool bf16, float *parts, int S,
+                               double *part, double *norm2, int *err, cudaStream_t s);
 size_t problem_bytes();
 bool fill_group_problem(void *host_dst, const void *X, int64_t M, int64_t K, int64_t ldx,
                         const void *Y, int k, int64_t ldy, bool split, bool bf16, float *C,
