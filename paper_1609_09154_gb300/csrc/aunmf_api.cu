@@ -61,7 +61,7 @@ struct aunmf_handle {
   Buf Ht, PW, PHt, GH, GW, G64, gpart, dpart, n2a, ctr, relres, last;
   Buf Ax, At, Hk, Wt, parts, err;  // tensor-core path: layout copies, split partials, error flag
   Buf tcacc;                       // tensor-core path, k > 64: partial sums of wide products
-  Buf colptr, rowidx, cval, cscratch;  // sparse path: CSC copy of A
+  Buf colptr, cnz, cscratch;  // sparse path: CSC copy of A
   Buf bppq;                            // BPP: G^{-1} in FP64
   Buf dHt;                             // loss backward: (dL/dH)^T
   Buf batch, batch_meta;               // batched runs: arena, descriptors
@@ -72,7 +72,7 @@ struct aunmf_handle {
   std::map<std::tuple<int, int64_t, int64_t, int, int>, std::pair<int, int>> gemm_tuned;
   Buf hA, hW, hH;  // device copies for aunmf_run_host
   Buf aux;         // printed HALS sweep / projected gradient: partials, barrier, values
-  Buf spl, splpart;  // sparse: long-row lists of the CSR and the CSC; their chunk partials
+  Buf splr, splc;  // sparse: long rows of the CSR and of the CSC, with their partial sums
   int max_gram_blocks = 2 * 152;
   int n_dparts = 2 * 152;
 };
@@ -181,8 +181,7 @@ struct RunCtx {
   int *err;
   // sparse path: CSC form of A; the long rows of the CSR and the CSC
   const int64_t *colptr;
-  const int32_t *rowidx;
-  const float *cval;
+  const uint2 *cnz;
   SpLongRows csr_long, csc_long;
   bool profile;
   int hals_variant;     // 1: Eq. halsupdate as printed
@@ -253,7 +252,7 @@ cudaError_t product_aht(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   if (!A->dense) {
     PhaseTimer t(c, s, kPhAht);
     return launch_aht_csr(A->rowptr, A->colidx, A->val, A->m, A->n, A->nnz, c.Ht, c.k, c.PW,
-                          &c.csr_long, s);
+                          c.csr_long, s);
   }
   if (c.prec == AUNMF_FP32) {
     PhaseTimer t(c, s, kPhAht);
@@ -291,8 +290,7 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   (void)h;
   if (!A->dense) {
     PhaseTimer t(c, s, kPhWta);
-    return launch_wta_csc(c.colptr, c.rowidx, c.cval, A->n, A->m, A->nnz, c.W, c.k, c.PHt,
-                          &c.csc_long, s);
+    return launch_wta_csc(c.colptr, c.cnz, A->n, A->m, A->nnz, c.W, c.k, c.PHt, c.csc_long, s);
   }
   if (c.prec == AUNMF_FP32) {
     PhaseTimer t(c, s, kPhWta);
@@ -333,8 +331,10 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
 // rounding term are wanted now (kPrepNorm).
 enum { kPrepAht = 1, kPrepWta = 2, kPrepNorm = 4 };
 int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s);
-// CSC copy of a sparse A (setup of the W^T A product).
-int prepare_sparse(aunmf_handle *h, RunCtx &c, cudaStream_t s);
+// Setup of the sparse products: the long rows of the CSR (A H^T); the CSC copy
+// of A and its long rows (W^T A).
+int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s);
+int prepare_csc(aunmf_handle *h, RunCtx &c, cudaStream_t s);
 
 cudaError_t update(RunCtx &c, float *X, const float *Pm, const float *G, const double *G64,
                    int64_t rows, cudaStream_t s) {
@@ -486,36 +486,26 @@ int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s) {
   return AUNMF_OK;
 }
 
-int prepare_sparse(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
+int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
+  const aunmf_matrix *A = c.A;
+  ENS_TC(h, h->splr, long_rows_bytes(A->nnz, c.k));
+  cudaError_t e = list_long_rows(A->rowptr, A->m, A->nnz, c.k, h->splr.p, &c.csr_long, s);
+  return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
+}
+
+int prepare_csc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   const aunmf_matrix *A = c.A;
   ENS_TC(h, h->colptr, sizeof(int64_t) * (size_t)(A->n + 1));
-  ENS_TC(h, h->rowidx, sizeof(int32_t) * (size_t)(A->nnz > 0 ? A->nnz : 1));
-  ENS_TC(h, h->cval, sizeof(float) * (size_t)(A->nnz > 0 ? A->nnz : 1));
+  ENS_TC(h, h->cnz, sizeof(uint2) * (size_t)(A->nnz > 0 ? A->nnz : 1));
   ENS_TC(h, h->cscratch, csc_scratch_bytes(A->n, A->nnz));
+  ENS_TC(h, h->splc, long_rows_bytes(A->nnz, c.k));
   cudaError_t e = launch_csr_to_csc(A->rowptr, A->colidx, A->val, A->m, A->n, A->nnz,
-                                    P<int64_t>(h->colptr), P<int32_t>(h->rowidx), P<float>(h->cval),
-                                    h->cscratch.p, s);
+                                    P<int64_t>(h->colptr), P<uint2>(h->cnz), h->cscratch.p, s);
   if (e != cudaSuccess) return fail_cuda(h, e, "csr_to_csc");
   c.colptr = P<int64_t>(h->colptr);
-  c.rowidx = P<int32_t>(h->rowidx);
-  c.cval = P<float>(h->cval);
-  // rows of either form long enough to be split over several warps
-  const int64_t cap = long_rows_capacity(A->nnz);
-  ENS_TC(h, h->spl, sizeof(int64_t) * (size_t)(4 * cap + 2) + 2 * sizeof(unsigned long long));
-  int64_t *L = P<int64_t>(h->spl);
-  unsigned long long *cnt = reinterpret_cast<unsigned long long *>(L + 4 * cap + 2);
-  e = find_long_rows(A->rowptr, A->m, A->nnz, L, L + cap, cnt, &c.csr_long, s);
-  if (e == cudaSuccess)
-    e = find_long_rows(c.colptr, A->n, A->nnz, L + 2 * cap + 1, L + 3 * cap + 1, cnt + 1,
-                       &c.csc_long, s);
-  if (e != cudaSuccess) return fail_cuda(h, e, "find_long_rows");
-  const int64_t parts = c.csr_long.nchunks + c.csc_long.nchunks;
-  if (parts > 0) {
-    ENS_TC(h, h->splpart, sizeof(float) * (size_t)parts * c.k);
-    c.csr_long.part = P<float>(h->splpart);
-    c.csc_long.part = c.csr_long.part + (size_t)c.csr_long.nchunks * c.k;
-  }
-  return AUNMF_OK;
+  c.cnz = P<uint2>(h->cnz);
+  e = list_long_rows(c.colptr, A->n, A->nnz, c.k, h->splc.p, &c.csc_long, s);
+  return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
 }
 
 }  // namespace
@@ -568,7 +558,7 @@ int aunmf_destroy(aunmf_handle *h) {
   cudaStreamSynchronize(h->stream);
   Buf *bufs[] = {&h->tick, &h->GWr, &h->Ht, &h->PW, &h->PHt, &h->GH, &h->GW, &h->G64, &h->gpart, &h->dpart, &h->n2a,
                  &h->ctr, &h->relres, &h->last, &h->Ax, &h->At, &h->Hk, &h->Wt, &h->parts,
-                 &h->err, &h->tcacc, &h->aux, &h->spl, &h->splpart, &h->colptr, &h->rowidx, &h->cval, &h->cscratch, &h->bppq, &h->dHt,
+                 &h->err, &h->tcacc, &h->aux, &h->splr, &h->splc, &h->colptr, &h->cnz, &h->cscratch, &h->bppq, &h->dHt,
                  &h->batch, &h->batch_meta, &h->hA, &h->hW, &h->hH};
   for (Buf *b : bufs)
     if (b->p) cudaFree(b->p);
@@ -750,7 +740,8 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));
   }
   if (!A->dense) {
-    int prc = prepare_sparse(h, c, s);
+    int prc = prepare_csr_rows(h, c, s);
+    if (prc == AUNMF_OK) prc = prepare_csc(h, c, s);
     if (prc != AUNMF_OK) return prc;
   }
   if (!c.err) {  // the bounded waits of the wide-rank Gram report here too
@@ -956,6 +947,9 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), h->stream));
+  } else {
+    int rc = prepare_csr_rows(h, c, h->stream);
+    if (rc != AUNMF_OK) return rc;
   }
   CK(h, product_aht(h, c, h->stream));
   return AUNMF_OK;
@@ -989,7 +983,7 @@ int aunmf_wta(aunmf_handle *h, const aunmf_matrix *A, const float *W, int k, int
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), h->stream));
   }
   if (!A->dense) {
-    int rc = prepare_sparse(h, c, h->stream);
+    int rc = prepare_csc(h, c, h->stream);
     if (rc != AUNMF_OK) return rc;
   }
   CK(h, product_wta(h, c, h->stream));
@@ -1140,9 +1134,10 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
     CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     RunCtx c{};
     c.A = A;
-    int rc = prepare_sparse(h, c, s);
+    c.k = k;
+    int rc = prepare_csc(h, c, s);
     if (rc != AUNMF_OK) return rc;
-    CK(h, launch_wta_csc(c.colptr, c.rowidx, c.cval, n, m, A->nnz, W, k, PHt, &c.csc_long, s));
+    CK(h, launch_wta_csc(c.colptr, c.cnz, n, m, A->nnz, W, k, PHt, c.csc_long, s));
   }
   CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s,
                     P<int>(h->err), gram_tick(h)));
@@ -1212,7 +1207,8 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
     CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (!A->dense) {
-    int rc = prepare_sparse(h, c, s);
+    int rc = what & kPrepAht ? prepare_csr_rows(h, c, s) : AUNMF_OK;
+    if (rc == AUNMF_OK && (what & kPrepWta)) rc = prepare_csc(h, c, s);
     if (rc != AUNMF_OK) return rc;
   }
   return AUNMF_OK;

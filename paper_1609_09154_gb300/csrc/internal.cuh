@@ -133,37 +133,35 @@ cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, c
                             int k, float *P, float *parts, int *err, cudaStream_t s);
 
 // Sparse products (FP32).  P_W (m x k) = A Ht from CSR; P_Ht (n x k) = A^T W
-// from the CSC form (colptr[n+1], rowidx[nnz], cval[nnz]) built by
+// from the CSC form (colptr[n+1], {row, value bits}[nnz]) built by
 // launch_csr_to_csc (scratch: csc_scratch_bytes(n, nnz) bytes).
 // Rows (of the CSR, or of the CSC: columns of A) with more than kLongRowNz
-// nonzeros, which the products split into chunks over many warps: the sorted
-// row list, its chunk prefix, and chunk partial sums (nchunks x k floats);
-// nlong = 0: none (or lr == null).
-constexpr int64_t kLongRowNz = 4096;
-struct SpLongRows {
-  int64_t nlong = 0, nchunks = 0;
-  const int64_t *row = nullptr;
-  const int64_t *chunk0 = nullptr;
-  float *part = nullptr;
+// nonzeros are cut into chunks over many warps.  The line: a warp walks ~50 ns
+// a nonzero, so 512 of them are ~25 us, the tail one row may add to a product.
+constexpr int64_t kLongRowNz = 512;
+struct SpLongRows {               // device memory, filled by list_long_rows
+  unsigned long long *count = nullptr;  // [0]: long rows, [1]: their chunks
+  int64_t *row = nullptr;         // {row, first chunk, chunks} each
+  int64_t *chunk = nullptr;       // {first, end nonzero} each
+  float *part = nullptr;          // partial sums, k per chunk
+  int64_t cap_rows = 0, cap_chunks = 0;
 };
 // (n, m and nnz bound the gathered indices in the checked build.)
 cudaError_t launch_aht_csr(const int64_t *rowptr, const int32_t *colidx, const float *val,
                            int64_t m, int64_t n, int64_t nnz, const float *Ht, int k, float *P,
-                           const SpLongRows *lr, cudaStream_t s);
-cudaError_t launch_wta_csc(const int64_t *colptr, const int32_t *rowidx, const float *cval,
-                           int64_t n, int64_t m, int64_t nnz, const float *W, int k, float *P,
-                           const SpLongRows *lr, cudaStream_t s);
-// list: long_rows_capacity(nnz) int64; chunk0: capacity + 1 int64; count: one
-// counter.  Fills lr (its part stays null: the caller allocates nchunks x k
-// floats).  Synchronises the stream.
-int64_t long_rows_capacity(int64_t nnz);
-cudaError_t find_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int64_t *list,
-                           int64_t *chunk0, unsigned long long *count, SpLongRows *lr,
+                           const SpLongRows &lr, cudaStream_t s);
+cudaError_t launch_wta_csc(const int64_t *colptr, const uint2 *cnz, int64_t n, int64_t m,
+                           int64_t nnz, const float *W, int k, float *P, const SpLongRows &lr,
                            cudaStream_t s);
+// mem: long_rows_bytes(nnz, k) bytes (8-byte aligned), cut up into lr and
+// filled on the device; enqueues only.
+size_t long_rows_bytes(int64_t nnz, int k);
+cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
+                           SpLongRows *lr, cudaStream_t s);
 size_t csc_scratch_bytes(int64_t n, int64_t nnz);
 cudaError_t launch_csr_to_csc(const int64_t *rowptr, const int32_t *colidx, const float *val,
-                              int64_t m, int64_t n, int64_t nnz, int64_t *colptr, int32_t *rowidx,
-                              float *cval, void *scratch, cudaStream_t s);
+                              int64_t m, int64_t n, int64_t nnz, int64_t *colptr, uint2 *cnz,
+                              void *scratch, cudaStream_t s);
 
 // Transpose: out (cols x rows) = in (rows x cols)^T, both row-major, dense ld.
 cudaError_t launch_transpose(const float *in, int64_t rows, int64_t cols, float *out,

@@ -5,10 +5,8 @@
 //                     walks the row's nonzeros and gathers rows of Ht (n x k).
 //   P_Ht = A^T W    : the same kernel over the CSC form of A (the CSR form of
 //                     A^T), gathering rows of W (m x k).
-// The CSC copy is built once per run on the device (k_csc.cu).
-#include <algorithm>
-#include <vector>
-
+// The CSC copy is built once per run on the device (k_csc.cu), each nonzero
+// as an 8-byte {row, value}.
 #include "internal.cuh"
 
 namespace aunmf {
@@ -16,22 +14,44 @@ namespace {
 
 constexpr int kSpThreads = 256;
 constexpr int kSpWarps = kSpThreads / kWarp;
-constexpr int64_t kChunkNz = 2048;  // nonzeros per warp on a long row
+// Nonzeros per chunk of a long row of `len`: one warp's work.  Longer chunks
+// for the longest rows, whose partial sums one block then adds.
+__device__ __forceinline__ int64_t chunk_nz(int64_t len) { return len <= 32768 ? 256 : 512; }
+
+// The nonzeros of a matrix: column (or row) indices and values in two arrays
+// (CSR as given), or index and value bits side by side (the CSC copy: one
+// 8-byte load per nonzero).
+struct NzSplit {
+  const int32_t *__restrict__ idx;
+  const float *__restrict__ val;
+  __device__ __forceinline__ void get(int64_t e, int &c, float &v) const {
+    c = __ldg(idx + e);
+    v = __ldg(val + e);
+  }
+};
+struct NzPacked {
+  const uint2 *__restrict__ nz;
+  __device__ __forceinline__ void get(int64_t e, int &c, float &v) const {
+    const uint2 q = __ldg(nz + e);
+    c = (int)q.x;
+    v = __uint_as_float(q.y);
+  }
+};
 
 // acc[t] (lane's entries j = lane + 32 t) += sum over nonzeros e in [e0, e1)
 // of val[e] X[idx[e], j]: the warp stages 32 nonzeros in registers, then
 // broadcasts them and gathers the k-vectors of X (ncols rows), four at a
 // time.  (ncols is read only by the checked build.)
-template <int KT>
-__device__ __forceinline__ void spmm_range(const int32_t *__restrict__ idx,
-                                           const float *__restrict__ val,
-                                           const float *__restrict__ X, int64_t ncols, int k,
+template <int KT, class NZ>
+__device__ __forceinline__ void spmm_range(const NZ &nz, const float *__restrict__ X, int64_t ncols,
+                                           int k,
                                            int64_t e0, int64_t e1, float (&acc)[KT], int lane) {
   (void)ncols;
   for (int64_t eb = e0; eb < e1; eb += 32) {
     const int64_t e = eb + lane;
-    const int my_c = e < e1 ? __ldg(&idx[e]) : 0;
-    const float my_v = e < e1 ? __ldg(&val[e]) : 0.f;
+    int my_c = 0;
+    float my_v = 0.f;
+    if (e < e1) nz.get(e, my_c, my_v);
     const int cnt = (int)min((int64_t)32, e1 - eb);
     int j = 0;
     for (; j + 4 <= cnt; j += 4) {
@@ -71,26 +91,25 @@ __device__ __forceinline__ void spmm_range(const int32_t *__restrict__ idx,
   }
 }
 
-// Y (rows x k) = S (rows x ncols, CSR ptr/idx/val, nnz nonzeros) * X
-// (ncols x k), a warp per row.  Rows longer than `skip_above` (> 0) are left
-// to the chunked kernels below.
-template <int KT>
+// Y (rows x k) = S (rows x ncols, row pointers and nonzeros, nnz of them) * X
+// (ncols x k), a warp per row.  Rows longer than kLongRowNz are left to the
+// chunked kernels below.
+template <int KT, class NZ>
 __global__ void __launch_bounds__(kSpThreads)
-    k_spmm(const int64_t *__restrict__ ptr, const int32_t *__restrict__ idx,
-           const float *__restrict__ val, int64_t rows, int64_t ncols, int64_t nnz,
-           const float *__restrict__ X, int k, float *__restrict__ Y, int64_t skip_above) {
+    k_spmm(const int64_t *__restrict__ ptr, const NZ nz, int64_t rows, int64_t ncols, int64_t nnz,
+           const float *__restrict__ X, int k, float *__restrict__ Y) {
   (void)nnz;
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + (threadIdx.x >> 5);
   const int64_t ws = (int64_t)gridDim.x * kSpWarps;
   for (int64_t r = w0; r < rows; r += ws) {
     const int64_t e0 = ptr[r], e1 = ptr[r + 1];
-    if (skip_above > 0 && e1 - e0 > skip_above) continue;
+    if (e1 - e0 > kLongRowNz) continue;
     if (!AUNMF_BOUND(e0 >= 0 && e0 <= e1 && e1 <= nnz, AUNMF_CHECK_SPMM_RANGE)) continue;
     float acc[KT];
 #pragma unroll
     for (int t = 0; t < KT; ++t) acc[t] = 0.f;
-    spmm_range<KT>(idx, val, X, ncols, k, e0, e1, acc, lane);
+    spmm_range<KT>(nz, X, ncols, k, e0, e1, acc, lane);
 #pragma unroll
     for (int t = 0; t < KT; ++t) {
       const int col = lane + 32 * t;
@@ -99,91 +118,115 @@ __global__ void __launch_bounds__(kSpThreads)
   }
 }
 
-// Long rows (a power-law hub can hold 10^6 nonzeros, which one warp would
-// walk alone while the rest of the GPU idles): chunk c of the sorted list of
-// long rows covers kChunkNz nonzeros of row lrow[i], chunk0[i] <= c <
-// chunk0[i + 1]; a warp per chunk writes its partial sums, and a warp per
-// long row adds its chunks in chunk order (so results do not depend on
-// scheduling).
-template <int KT>
+// Long rows (a power-law hub can hold 10^6 nonzeros, which one warp would walk
+// alone, ~50 ns a nonzero, while the rest of the GPU idles: 0.9 ms of a 2e7-
+// nonzero product with rows of up to 18,000): cut into chunks, a warp per
+// chunk writes its partial sums, and a block per long row adds its chunks in
+// chunk order (so results do not depend on scheduling).  The list is built on
+// the device (k_list_long) in any order, each row's chunks in consecutive
+// slots; nothing returns to the host.
+template <int KT, class NZ>
 __global__ void __launch_bounds__(kSpThreads)
-    k_spmm_chunks(const int64_t *__restrict__ ptr, const int32_t *__restrict__ idx,
-                  const float *__restrict__ val, int64_t rows, int64_t ncols, int64_t nnz,
-                  const float *__restrict__ X, int k, const int64_t *__restrict__ lrow,
-                  const int64_t *__restrict__ chunk0, int64_t nlong, int64_t nchunks,
-                  float *__restrict__ part) {
-  (void)rows;
+    k_spmm_chunks(const NZ nz, int64_t ncols, int64_t nnz, const float *__restrict__ X, int k,
+                  const SpLongRows lr) {
   (void)nnz;
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + (threadIdx.x >> 5);
   const int64_t ws = (int64_t)gridDim.x * kSpWarps;
+  const int64_t nchunks = min((int64_t)lr.count[1], lr.cap_chunks);
   for (int64_t c = w0; c < nchunks; c += ws) {
-    int64_t lo = 0, hi = nlong - 1;  // last i with chunk0[i] <= c
-    while (lo < hi) {
-      const int64_t mid = (lo + hi + 1) >> 1;
-      if (chunk0[mid] <= c) lo = mid; else hi = mid - 1;
-    }
-    const int64_t r = lrow[lo];
-    if (!AUNMF_BOUND(r >= 0 && r < rows, AUNMF_CHECK_SPMM_RANGE)) continue;
-    const int64_t e0 = ptr[r] + (c - chunk0[lo]) * kChunkNz;
-    const int64_t e1 = min(ptr[r + 1], e0 + kChunkNz);
+    const int64_t e0 = lr.chunk[2 * c], e1 = lr.chunk[2 * c + 1];
     if (!AUNMF_BOUND(e0 >= 0 && e0 <= e1 && e1 <= nnz, AUNMF_CHECK_SPMM_RANGE)) continue;
     float acc[KT];
 #pragma unroll
     for (int t = 0; t < KT; ++t) acc[t] = 0.f;
-    spmm_range<KT>(idx, val, X, ncols, k, e0, e1, acc, lane);
+    spmm_range<KT>(nz, X, ncols, k, e0, e1, acc, lane);
 #pragma unroll
     for (int t = 0; t < KT; ++t) {
       const int col = lane + 32 * t;
-      if (col < k) part[c * k + col] = acc[t];
+      if (col < k) lr.part[c * k + col] = acc[t];
     }
   }
 }
 
+// Y's long rows: warp w of a row's block adds the w-th eighth of its chunks in
+// order, eight loads in flight, and the eighths are added in order.
 template <int KT>
 __global__ void __launch_bounds__(kSpThreads)
-    k_spmm_long_sum(const int64_t *__restrict__ lrow, const int64_t *__restrict__ chunk0,
-                    int64_t nlong, const float *__restrict__ part, int k, float *__restrict__ Y) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + (threadIdx.x >> 5);
-  const int64_t ws = (int64_t)gridDim.x * kSpWarps;
-  for (int64_t i = w0; i < nlong; i += ws) {
+    k_spmm_long_sum(const SpLongRows lr, int64_t rows, int k, float *__restrict__ Y) {
+  (void)rows;
+  __shared__ float sw[kSpWarps][32 * KT];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t nlong = min((int64_t)lr.count[0], lr.cap_rows);
+  for (int64_t i = blockIdx.x; i < nlong; i += gridDim.x) {
+    const int64_t r = lr.row[3 * i], base = lr.row[3 * i + 1], nc = lr.row[3 * i + 2];
+    const int64_t per = (nc + kSpWarps - 1) / kSpWarps;
+    const int64_t c0 = base + w * per, c1 = min(base + nc, c0 + per);
     float acc[KT];
-#pragma unroll
-    for (int t = 0; t < KT; ++t) acc[t] = 0.f;
-    for (int64_t c = chunk0[i]; c < chunk0[i + 1]; ++c)
-#pragma unroll
-      for (int t = 0; t < KT; ++t) {
-        const int col = lane + 32 * t;
-        if (col < k) acc[t] += part[c * k + col];
-      }
-    const int64_t r = lrow[i];
 #pragma unroll
     for (int t = 0; t < KT; ++t) {
       const int col = lane + 32 * t;
-      if (col < k) Y[r * k + col] = acc[t];
+      acc[t] = 0.f;
+      if (col >= k) continue;
+      int64_t c = c0;
+      for (; c + 8 <= c1; c += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = lr.part[(c + u) * k + col];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[t] += v[u];
+      }
+      for (; c < c1; ++c) acc[t] += lr.part[c * k + col];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < KT; ++t) sw[w][32 * t + lane] = acc[t];
+    __syncthreads();
+    if (!AUNMF_BOUND(r >= 0 && r < rows, AUNMF_CHECK_SPMM_RANGE)) continue;
+    for (int col = threadIdx.x; col < k; col += kSpThreads) {
+      float y = sw[0][col];
+#pragma unroll
+      for (int q = 1; q < kSpWarps; ++q) y += sw[q][col];
+      Y[r * k + col] = y;
     }
   }
 }
 
-// len[i] = nonzeros of row list[i].
-__global__ void k_long_lens(const int64_t *__restrict__ ptr, const int64_t *__restrict__ list,
-                            int64_t n, int64_t *__restrict__ len) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    len[i] = ptr[list[i] + 1] - ptr[list[i]];
-}
-
-// Appends the rows longer than thr to list (unordered; the caller sorts).
-__global__ void k_find_long(const int64_t *__restrict__ ptr, int64_t rows, int64_t thr,
-                            int64_t *__restrict__ list, unsigned long long *count,
-                            int64_t capacity) {
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
-       r += (int64_t)gridDim.x * blockDim.x)
-    if (ptr[r + 1] - ptr[r] > thr) {
-      const unsigned long long at = atomicAdd(count, 1ull);
-      if ((int64_t)at < capacity) list[at] = r;
+// The long rows of a row-pointer array: {row, first chunk, chunks} per row and
+// {first, end nonzero} per chunk, a warp per 32 rows.
+__global__ void k_list_long(const int64_t *__restrict__ ptr, int64_t rows, const SpLongRows lr) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t ws = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r0 = w0 * 32; r0 < rows; r0 += ws * 32) {
+    const int64_t r = r0 + lane;
+    const int64_t e0 = r < rows ? ptr[r] : 0, e1 = r < rows ? ptr[r + 1] : 0;
+    unsigned todo = __ballot_sync(0xffffffffu, e1 - e0 > kLongRowNz);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int64_t a = __shfl_sync(0xffffffffu, e0, src), b = __shfl_sync(0xffffffffu, e1, src);
+      const int64_t cz = chunk_nz(b - a), nc = (b - a + cz - 1) / cz;
+      long long i = 0, base = 0;
+      if (lane == 0) {
+        i = (long long)atomicAdd(&lr.count[0], 1ull);
+        base = (long long)atomicAdd(&lr.count[1], (unsigned long long)nc);
+      }
+      i = __shfl_sync(0xffffffffu, i, 0);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      // (always true for a well-formed row-pointer array of nnz nonzeros)
+      if (i >= lr.cap_rows || base + nc > lr.cap_chunks) continue;
+      if (lane == 0) {
+        lr.row[3 * i] = r0 + src;
+        lr.row[3 * i + 1] = base;
+        lr.row[3 * i + 2] = nc;
+      }
+      for (int64_t c = lane; c < nc; c += 32) {
+        lr.chunk[2 * (base + c)] = a + c * cz;
+        lr.chunk[2 * (base + c) + 1] = min(b, a + (c + 1) * cz);
+      }
     }
+  }
 }
 
 int sp_blocks(int64_t warps) {
@@ -203,26 +246,23 @@ int sp_blocks(int64_t warps) {
     default: CALL(16); break;      \
   }
 
-cudaError_t spmm(const int64_t *ptr, const int32_t *idx, const float *val, int64_t rows,
-                 int64_t ncols, int64_t nnz, const float *X, int k, float *Y,
-                 const SpLongRows *lr, cudaStream_t s) {
+template <class NZ>
+cudaError_t spmm(const int64_t *ptr, const NZ nz, int64_t rows, int64_t ncols, int64_t nnz,
+                 const float *X, int k, float *Y, const SpLongRows &lr, cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
   const int kt = (k + 31) / 32;
-  const bool split = lr && lr->nlong > 0;
-  const int64_t skip = split ? kLongRowNz : 0;
   const int nb = sp_blocks(rows);
 #define AUNMF_SP_MAIN(KT) \
-  k_spmm<KT><<<nb, kSpThreads, 0, s>>>(ptr, idx, val, rows, ncols, nnz, X, k, Y, skip)
+  k_spmm<KT, NZ><<<nb, kSpThreads, 0, s>>>(ptr, nz, rows, ncols, nnz, X, k, Y)
   AUNMF_SP_SWITCH(kt, AUNMF_SP_MAIN)
 #undef AUNMF_SP_MAIN
   g_launches += 1;
-  if (split) {
-    const int nbc = sp_blocks(lr->nchunks), nbl = sp_blocks(lr->nlong);
-#define AUNMF_SP_CH(KT)                                                                  \
-  k_spmm_chunks<KT><<<nbc, kSpThreads, 0, s>>>(ptr, idx, val, rows, ncols, nnz, X, k,      \
-                                               lr->row, lr->chunk0, lr->nlong, lr->nchunks, \
-                                               lr->part);                                \
-  k_spmm_long_sum<KT><<<nbl, kSpThreads, 0, s>>>(lr->row, lr->chunk0, lr->nlong, lr->part, k, Y)
+  if (nnz > kLongRowNz) {
+    const int nbc = sp_blocks(lr.cap_chunks);
+    const int nbl = (int)(lr.cap_rows < 152 * 4 ? lr.cap_rows : 152 * 4);
+#define AUNMF_SP_CH(KT)                                                                        \
+  k_spmm_chunks<KT, NZ><<<nbc, kSpThreads, 0, s>>>(nz, ncols, nnz, X, k, lr);                   \
+  k_spmm_long_sum<KT><<<nbl, kSpThreads, 0, s>>>(lr, rows, k, Y)
     AUNMF_SP_SWITCH(kt, AUNMF_SP_CH)
 #undef AUNMF_SP_CH
     g_launches += 2;
@@ -234,60 +274,38 @@ cudaError_t spmm(const int64_t *ptr, const int32_t *idx, const float *val, int64
 
 cudaError_t launch_aht_csr(const int64_t *rowptr, const int32_t *colidx, const float *val,
                            int64_t m, int64_t n, int64_t nnz, const float *Ht, int k, float *P,
-                           const SpLongRows *lr, cudaStream_t s) {
-  return spmm(rowptr, colidx, val, m, n, nnz, Ht, k, P, lr, s);
+                           const SpLongRows &lr, cudaStream_t s) {
+  return spmm(rowptr, NzSplit{colidx, val}, m, n, nnz, Ht, k, P, lr, s);
 }
 
-cudaError_t launch_wta_csc(const int64_t *colptr, const int32_t *rowidx, const float *cval,
-                           int64_t n, int64_t m, int64_t nnz, const float *W, int k, float *P,
-                           const SpLongRows *lr, cudaStream_t s) {
-  return spmm(colptr, rowidx, cval, n, m, nnz, W, k, P, lr, s);
-}
-
-int64_t long_rows_capacity(int64_t nnz) { return nnz / kLongRowNz + 1; }
-
-// The long rows of a CSR (or CSC) row-pointer array, sorted, with their chunk
-// prefix: a device pass finds them (list, count), the host sorts the short
-// list and forms the prefix, which goes back to the device.  Synchronises.
-cudaError_t find_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int64_t *list,
-                           int64_t *chunk0, unsigned long long *count, SpLongRows *lr,
+cudaError_t launch_wta_csc(const int64_t *colptr, const uint2 *cnz, int64_t n, int64_t m,
+                           int64_t nnz, const float *W, int k, float *P, const SpLongRows &lr,
                            cudaStream_t s) {
-  lr->nlong = lr->nchunks = 0;
-  lr->row = list;
-  lr->chunk0 = chunk0;
-  if (rows == 0) return cudaSuccess;
-  const int64_t cap = long_rows_capacity(nnz);
-  cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), s);
+  return spmm(colptr, NzPacked{cnz}, n, m, nnz, W, k, P, lr, s);
+}
+
+size_t long_rows_bytes(int64_t nnz, int k) {
+  const int64_t cr = nnz / kLongRowNz + 1, cc = nnz / 256 + cr + 1;
+  return sizeof(int64_t) * (size_t)(2 + 3 * cr + 2 * cc) + sizeof(float) * (size_t)cc * k;
+}
+
+cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
+                           SpLongRows *lr, cudaStream_t s) {
+  lr->cap_rows = nnz / kLongRowNz + 1;
+  lr->cap_chunks = nnz / 256 + lr->cap_rows + 1;
+  int64_t *p = static_cast<int64_t *>(mem);
+  lr->count = reinterpret_cast<unsigned long long *>(p);
+  lr->row = p + 2;
+  lr->chunk = lr->row + 3 * lr->cap_rows;
+  lr->part = reinterpret_cast<float *>(lr->chunk + 2 * lr->cap_chunks);
+  if (rows == 0 || nnz <= kLongRowNz) return cudaSuccess;  // no long row: spmm skips the pass
+  cudaError_t e = cudaMemsetAsync(lr->count, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   int64_t nb = (rows + 255) / 256;
   if (nb > 152 * 16) nb = 152 * 16;
-  k_find_long<<<(unsigned)nb, 256, 0, s>>>(ptr, rows, kLongRowNz, list, count, cap);
+  k_list_long<<<(unsigned)nb, 256, 0, s>>>(ptr, rows, *lr);
   g_launches += 1;
-  unsigned long long n = 0;
-  if ((e = cudaMemcpyAsync(&n, count, sizeof(n), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-  if (n == 0) return cudaSuccess;
-  if ((int64_t)n > cap) return cudaErrorInvalidValue;  // cannot happen: each has > kLongRowNz
-  std::vector<int64_t> h(n), len(n), c0(n + 1, 0);
-  if ((e = cudaMemcpy(h.data(), list, sizeof(int64_t) * n, cudaMemcpyDeviceToHost)) != cudaSuccess)
-    return e;
-  std::sort(h.begin(), h.end());
-  if ((e = cudaMemcpy(list, h.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess)
-    return e;
-  k_long_lens<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ptr, list, (int64_t)n, chunk0);
-  g_launches += 1;
-  if ((e = cudaMemcpyAsync(len.data(), chunk0, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, s)) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-  for (size_t i = 0; i < n; ++i) c0[i + 1] = c0[i] + (len[i] + kChunkNz - 1) / kChunkNz;
-  if ((e = cudaMemcpy(chunk0, c0.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice)) !=
-      cudaSuccess)
-    return e;
-  lr->nlong = (int64_t)n;
-  lr->nchunks = c0[n];
-  return cudaSuccess;
+  return cudaGetLastError();
 }
-
 
 }  // namespace aunmf
