@@ -173,6 +173,13 @@ cudaError_t launch_mu(float *X, const float *P, const float *G, int64_t rows, in
 // unit: Eq. halsupdate as printed (no division by G_ii).
 cudaError_t launch_hals(float *X, const float *P, const float *G, int64_t rows, int k,
                         cudaStream_t s, bool unit = false);
+// The same for k > 64 (k_wide.cu).  Gradient rows: out = g (X G - P).
+cudaError_t launch_mu_wide(float *X, const float *P, const float *G, int64_t rows, int k, float eps,
+                           cudaStream_t s);
+cudaError_t launch_hals_wide(float *X, const float *P, const float *G, int64_t rows, int k,
+                             bool unit, cudaStream_t s);
+cudaError_t launch_grad_wide(const float *X, const float *P, const float *G, int64_t rows, int k,
+                             const float *gscale, float *out, cudaStream_t s);
 // The W sweep of Eq. halsupdate as printed (no division by (HH^T)_ii, each
 // column normalised before the next is updated), one cooperative launch.
 // part: 2 * printed_sweep_blocks() doubles; bar: one counter (zeroed here);

@@ -2,10 +2,11 @@
 //
 // Both factors are held as row-major "rows x k" matrices (W, and H^T for H),
 // so one kernel serves both updates.  For k <= 64 two threads share one row
-// (k_luc_tpr).  Above, one warp owns one row; lane l holds the entries
-// j = l, l + 32, ... (KT = ceil(k / 32) per lane, rounded up to 12 or 16
-// above 256; k <= 512), and the k x k
-// Gram matrix is staged in shared memory when it fits.
+// (k_luc_tpr).  Wider ranks are in k_wide.cu, but for the HALS sweeps that it does
+// not take (k <= 108, or rows that are not whole 16-byte groups): one warp owns one
+// row, lane l holds the entries j = l, l + 32, ... (KT = ceil(k / 32) per lane,
+// rounded up to 12 or 16 above 256), and the Gram matrix is staged in shared
+// memory when it fits.
 #include <math.h>
 
 #include "internal.cuh"
@@ -32,46 +33,6 @@ __device__ __forceinline__ const float *stage_gram(const float *G, int k, float 
     for (int e = threadIdx.x; e < k * k; e += blockDim.x) sG[e] = G[e];
     __syncthreads();
     return sG;
-  }
-}
-
-// MU (Sec. 4.1, Eq. muupdate) on each row x of X with p the row of P:
-//   x_j <- x_j p_j / ((x G)_j + eps), all j at once (old x on the right).
-template <int KT, bool SMEM>
-__global__ void __launch_bounds__(kLucThreads)
-    k_mu(float *__restrict__ X, const float *__restrict__ P, const float *__restrict__ Gg,
-         int64_t rows, int k, float eps) {
-  extern __shared__ float sG[];
-  const float *G = stage_gram<SMEM>(Gg, k, sG);
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kLucWarps + (threadIdx.x >> 5);
-  const int64_t wstride = (int64_t)gridDim.x * kLucWarps;
-  for (int64_t r = w0; r < rows; r += wstride) {
-    float x[KT], den[KT];
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int j = lane + 32 * t;
-      x[t] = j < k ? X[r * k + j] : 0.f;
-      den[t] = 0.f;
-    }
-#pragma unroll
-    for (int tl = 0; tl < KT; ++tl) {
-      for (int ll = 0; ll < 32; ++ll) {
-        const int l = 32 * tl + ll;
-        if (l >= k) break;
-        const float xl = __shfl_sync(0xffffffffu, x[tl], ll);
-#pragma unroll
-        for (int t = 0; t < KT; ++t) {
-          const int j = lane + 32 * t;
-          if (j < k) den[t] = fmaf(xl, G[l * k + j], den[t]);
-        }
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int j = lane + 32 * t;
-      if (j < k) X[r * k + j] = x[t] * P[r * k + j] / (den[t] + eps);
-    }
   }
 }
 
@@ -120,143 +81,6 @@ __global__ void __launch_bounds__(kLucThreads)
     for (int t = 0; t < KT; ++t) {
       const int j = lane + 32 * t;
       if (j < k) X[r * k + j] = x[t];
-    }
-  }
-}
-
-// The same sweep for wide ranks (k > 108 with k % 4 == 0, the Gram read
-// through L1): lane l holds the entries j = 128 t + 4 l + u (t < KT4, u < 4)
-// of R rows, so a coordinate's row of G arrives as KT4 16-byte loads shared
-// by the R rows, instead of 32 KT4 / 8 scalar loads per row (the scalar form
-// spent ~95 instructions per row and coordinate at k = 512, most of them
-// load issue and 64-bit address arithmetic, at 41 % issue).
-template <int KT4, int R>
-__device__ __forceinline__ void hals4_rows(float *__restrict__ X, const float *__restrict__ P,
-                                           const float *__restrict__ G, int64_t rows, int k,
-                                           int unit) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kLucWarps + (threadIdx.x >> 5);
-  const int64_t wstride = (int64_t)gridDim.x * kLucWarps;
-  const int k4 = k >> 2;
-  const float4 *G4 = reinterpret_cast<const float4 *>(G);
-  for (int64_t rb = w0 * R; rb < rows; rb += wstride * R) {
-    float4 x[R][KT4], p[R][KT4];
-#pragma unroll
-    for (int rho = 0; rho < R; ++rho) {
-      const int64_t r = rb + rho;
-#pragma unroll
-      for (int t = 0; t < KT4; ++t) {
-        const int j4 = 32 * t + lane;  // float4 group of entries 4 j4 .. 4 j4 + 3
-        const bool in = r < rows && j4 < k4;
-        x[rho][t] = in ? reinterpret_cast<const float4 *>(X + r * k)[j4] : make_float4(0.f, 0.f, 0.f, 0.f);
-        p[rho][t] = in ? reinterpret_cast<const float4 *>(P + r * k)[j4] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < KT4; ++t) {
-      for (int l = 0; l < 32; ++l) {
-        const int i0 = 128 * t + 4 * l;
-        if (i0 >= k) break;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + u;
-          const float4 *Gi = G4 + (size_t)i * k4;  // G is symmetric: row i = column i
-          float4 g[KT4];
-#pragma unroll
-          for (int tt = 0; tt < KT4; ++tt) {
-            const int j4 = 32 * tt + lane;
-            g[tt] = j4 < k4 ? Gi[j4] : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-          const float gii = G[(size_t)i * k + i];
-#pragma unroll
-          for (int rho = 0; rho < R; ++rho) {
-            float part = 0.f;
-#pragma unroll
-            for (int tt = 0; tt < KT4; ++tt) {
-              part = fmaf(x[rho][tt].x, g[tt].x, part);
-              part = fmaf(x[rho][tt].y, g[tt].y, part);
-              part = fmaf(x[rho][tt].z, g[tt].z, part);
-              part = fmaf(x[rho][tt].w, g[tt].w, part);
-            }
-            const float dot = warp_sum(part);
-            if (lane == l && (unit || gii > 0.f)) {
-              float *xe = &x[rho][t].x + u;
-              const float pe = (&p[rho][t].x)[u];
-              const float v = *xe + (unit ? pe - dot : (pe - dot) / gii);
-              *xe = v > 0.f ? v : 0.f;
-            }
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int rho = 0; rho < R; ++rho) {
-      const int64_t r = rb + rho;
-#pragma unroll
-      for (int t = 0; t < KT4; ++t) {
-        const int j4 = 32 * t + lane;
-        if (r < rows && j4 < k4) reinterpret_cast<float4 *>(X + r * k)[j4] = x[rho][t];
-      }
-    }
-  }
-}
-
-// The sweep with the compiler's own register choice, and with registers
-// capped at 128 for two blocks per SM (a launch bound with a minimum of one
-// block already changes the choice: 79 against 62 registers at KT4 = 3).
-template <int KT4, int R>
-__global__ void __launch_bounds__(kLucThreads)
-    k_hals4(float *__restrict__ X, const float *__restrict__ P, const float *__restrict__ G,
-            int64_t rows, int k, int unit) {
-  hals4_rows<KT4, R>(X, P, G, rows, k, unit);
-}
-template <int KT4, int R>
-__global__ void __launch_bounds__(kLucThreads, 2)
-    k_hals4_capped(float *__restrict__ X, const float *__restrict__ P, const float *__restrict__ G,
-                   int64_t rows, int k, int unit) {
-  hals4_rows<KT4, R>(X, P, G, rows, k, unit);
-}
-
-// Gradient rows of 0.5 ||A - W H||_F^2: out = g (X G - P) for X rows x k,
-// G k x k, P rows x k (X = W, G = H H^T, P = A H^T gives dL/dW; X = H^T,
-// G = W^T W, P = (W^T A)^T gives (dL/dH)^T).  g is read from device memory
-// (NULL: g = 1).  Same lane layout as k_mu.
-template <int KT, bool SMEM>
-__global__ void __launch_bounds__(kLucThreads)
-    k_xg_minus_p(const float *__restrict__ X, const float *__restrict__ P,
-                 const float *__restrict__ Gg, int64_t rows, int k, const float *__restrict__ gscale,
-                 float *__restrict__ out) {
-  extern __shared__ float sG[];
-  const float *G = stage_gram<SMEM>(Gg, k, sG);
-  const float g = gscale ? *gscale : 1.f;
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kLucWarps + (threadIdx.x >> 5);
-  const int64_t wstride = (int64_t)gridDim.x * kLucWarps;
-  for (int64_t r = w0; r < rows; r += wstride) {
-    float x[KT], acc[KT];
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int j = lane + 32 * t;
-      x[t] = j < k ? X[r * k + j] : 0.f;
-      acc[t] = 0.f;
-    }
-#pragma unroll
-    for (int tl = 0; tl < KT; ++tl) {
-      for (int ll = 0; ll < 32; ++ll) {
-        const int l = 32 * tl + ll;
-        if (l >= k) break;
-        const float xl = __shfl_sync(0xffffffffu, x[tl], ll);
-#pragma unroll
-        for (int t = 0; t < KT; ++t) {
-          const int j = lane + 32 * t;
-          if (j < k) acc[t] = fmaf(xl, G[l * k + j], acc[t]);
-        }
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int j = lane + 32 * t;
-      if (j < k) out[r * k + j] = g * (acc[t] - P[r * k + j]);
     }
   }
 }
@@ -741,16 +565,7 @@ cudaError_t launch_mu(float *X, const float *P, const float *G, int64_t rows, in
                       cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
   if (k <= kTprMaxK) return launch_tpr_k<kOpMu>(X, P, G, rows, k, eps, nullptr, nullptr, s);
-  const int kt = (k + 31) / 32, nb = luc_blocks(rows);
-  const bool sm = k <= kSmemGramMaxK;
-  const size_t smem = sm ? sizeof(float) * k * k : 0;
-#define AUNMF_CALL_MU(KT)                                                          \
-  if (sm) k_mu<KT, true><<<nb, kLucThreads, smem, s>>>(X, P, G, rows, k, eps);     \
-  else k_mu<KT, false><<<nb, kLucThreads, 0, s>>>(X, P, G, rows, k, eps);
-  AUNMF_KT_SWITCH(kt, AUNMF_CALL_MU)
-#undef AUNMF_CALL_MU
-  g_launches += 1;
-  return cudaGetLastError();
+  return launch_mu_wide(X, P, G, rows, k, eps, s);
 }
 
 cudaError_t launch_hals(float *X, const float *P, const float *G, int64_t rows, int k,
@@ -759,29 +574,17 @@ cudaError_t launch_hals(float *X, const float *P, const float *G, int64_t rows, 
   if (k <= kTprMaxK)
     return unit ? launch_tpr_k<kOpHalsUnit>(X, P, G, rows, k, 0.f, nullptr, nullptr, s)
                 : launch_tpr_k<kOpHals>(X, P, G, rows, k, 0.f, nullptr, nullptr, s);
+  // wide ranks with 16-byte rows: blocked over coordinates (k = 256, 12,001 rows:
+  // 327 us with a warp per two rows).  Up to k = 108 the Gram fits in shared memory
+  // and a warp per row sums in 32 chains of stride 32, an order of its own.
+  if (k > kSmemGramMaxK && (k & 3) == 0 &&
+      ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(P) |
+        reinterpret_cast<uintptr_t>(G)) & 15) == 0)
+    return launch_hals_wide(X, P, G, rows, k, unit, s);
   const int kt = (k + 31) / 32, nb = luc_blocks(rows);
   const bool sm = k <= kSmemGramMaxK;
   const size_t smem = sm ? sizeof(float) * k * k : 0;
   const int u = unit ? 1 : 0;
-  if (!sm && (k & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(P) |
-                               reinterpret_cast<uintptr_t>(G)) & 15) == 0) {
-    // rows per warp and the register cap, measured (update phase per
-    // iteration at 96000 x 64000): k <= 256 two rows; 257..384 one row (two
-    // rows: 7.27 against 6.34 ms at k = 384); above, two rows capped at 128
-    // registers for two blocks per SM (10.3 ms at k = 512; one row 12.4 ms;
-    // two rows uncapped took 136 registers, one block per SM: 20.3 ms)
-    const int kt4 = (k + 127) / 128, R = kt4 == 3 ? 1 : 2;
-    int64_t nbw = (rows + kLucWarps * R - 1) / (kLucWarps * R);
-    if (nbw > 152 * 8) nbw = 152 * 8;
-    switch (kt4) {
-      case 1: k_hals4<1, 2><<<(unsigned)nbw, kLucThreads, 0, s>>>(X, P, G, rows, k, u); break;
-      case 2: k_hals4<2, 2><<<(unsigned)nbw, kLucThreads, 0, s>>>(X, P, G, rows, k, u); break;
-      case 3: k_hals4<3, 1><<<(unsigned)nbw, kLucThreads, 0, s>>>(X, P, G, rows, k, u); break;
-      default: k_hals4_capped<4, 2><<<(unsigned)nbw, kLucThreads, 0, s>>>(X, P, G, rows, k, u); break;
-    }
-    g_launches += 1;
-    return cudaGetLastError();
-  }
 #define AUNMF_CALL_HALS(KT)                                                       \
   if (sm) k_hals<KT, true><<<nb, kLucThreads, smem, s>>>(X, P, G, rows, k, u);    \
   else k_hals<KT, false><<<nb, kLucThreads, 0, s>>>(X, P, G, rows, k, u);
@@ -796,16 +599,7 @@ cudaError_t launch_xg_minus_p(const float *X, const float *P, const float *G, in
   if (rows == 0) return cudaSuccess;
   if (k <= kTprMaxK)
     return launch_tpr_k<kOpGrad>(const_cast<float *>(X), P, G, rows, k, 0.f, gscale, out, s);
-  const int kt = (k + 31) / 32, nb = luc_blocks(rows);
-  const bool sm = k <= kSmemGramMaxK;
-  const size_t smem = sm ? sizeof(float) * k * k : 0;
-#define AUNMF_CALL_XG(KT)                                                                  \
-  if (sm) k_xg_minus_p<KT, true><<<nb, kLucThreads, smem, s>>>(X, P, G, rows, k, gscale, out); \
-  else k_xg_minus_p<KT, false><<<nb, kLucThreads, 0, s>>>(X, P, G, rows, k, gscale, out);
-  AUNMF_KT_SWITCH(kt, AUNMF_CALL_XG)
-#undef AUNMF_CALL_XG
-  g_launches += 1;
-  return cudaGetLastError();
+  return launch_grad_wide(X, P, G, rows, k, gscale, out, s);
 }
 
 cudaError_t launch_hals_normalise(float *X, int64_t rows_x, float *Y, int64_t rows_y,
