@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "ptx.cuh"
 
 namespace aunmf {
 namespace bpp {
@@ -40,8 +41,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 
 // Shared memory of the fast kernel: Q = G^{-1} and G as FP32 pairs (k^2
 // doubles each), then per warp: the FP32 Cholesky factor L (kh x ldl floats),
-// a right-hand-side pair (2k floats), corrections (k floats), the index lists
-// (2k ints), |x_F|, r, and a solution pair (k floats each).  Nothing is FP64:
+// a right-hand-side pair (2k floats), the index lists (2k ints), |x_F|, r, and a solution pair (k floats each).  Nothing is FP64:
 // a row whose FP32 solve cannot finish goes to the FP64 fallback kernel.
 struct BppLayout {
   int kh;            // largest factorisation: floor(k / 2)
@@ -56,7 +56,7 @@ __host__ __device__ inline BppLayout bpp_layout(int k) {
   l.ldl = l.kh | 1;
   l.shared_dbl = 2 * (size_t)k * k;
   const size_t kf = 2 * (((size_t)k + 1) / 2);  // k floats, rounded up to whole doubles
-  l.warp_dbl = ((size_t)l.kh * l.ldl + 1) / 2 + kf + kf / 2 + (size_t)k + 4 * (kf / 2);
+  l.warp_dbl = ((size_t)l.kh * l.ldl + 1) / 2 + kf + (size_t)k + 4 * (kf / 2);
   return l;
 }
 
@@ -70,20 +70,28 @@ __host__ __device__ inline BppLayout bpp_layout(int k) {
 // instructions plus ~10 per column, where one lane per row would cost
 // ~n^2 / 2 (each lane running the longest dot product of its column).
 // Returns false (warp-uniform) on a non-positive pivot.
+// tri: (a << 8 | b) of the triangle's e-th entry, a (a + 1) / 2 + b = e, b <= a
+// (tri_table; a square root and its corrections per entry and column took most
+// of the factorisation's instructions).
 __device__ __forceinline__ double rsq(double d) { return rsqrt(d); }
 __device__ __forceinline__ float rsq(float d) { return rsqrtf(d); }
 
-template <class T, class Acc>
-__device__ __forceinline__ bool warp_cholesky(Acc M, const int *I, int n, T *L, int ldl,
-                                              int lane) {
-  // lower triangle of M_FF into L; entry e of the triangle is (a, b) with
-  // a (a + 1) / 2 <= e < (a + 1) (a + 2) / 2
-  const int tri = n * (n + 1) / 2;
-  for (int e = lane; e < tri; e += 32) {
+// Fills tri for n x n triangles (n <= 64), block-wide; the caller synchronises.
+__device__ __forceinline__ void tri_table(uint16_t *tri, int n) {
+  for (int e = threadIdx.x; e < n * (n + 1) / 2; e += blockDim.x) {
     int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
     if ((a + 1) * (a + 2) / 2 <= e) ++a;
     if (a * (a + 1) / 2 > e) --a;
-    const int b = e - a * (a + 1) / 2;
+    tri[e] = (uint16_t)(a << 8 | (e - a * (a + 1) / 2));
+  }
+}
+
+template <class T, class Acc>
+__device__ __forceinline__ bool warp_cholesky(Acc M, const int *I, int n, T *L, int ldl,
+                                              const uint16_t *tri, int lane) {
+  // lower triangle of M_FF into L
+  for (int e = lane; e < n * (n + 1) / 2; e += 32) {
+    const int a = tri[e] >> 8, b = tri[e] & 255;
     L[a * ldl + b] = M(I[b], I[a]);
   }
   __syncwarp();
@@ -95,13 +103,10 @@ __device__ __forceinline__ bool warp_cholesky(Acc M, const int *I, int n, T *L, 
     __syncwarp();
     if (lane == 0) L[c * ldl + c] = r;
     const int w = n - c - 1, tw = w * (w + 1) / 2;
+    T *Lc = L + (c + 1) * ldl + c;  // column c below the diagonal, stride ldl
     for (int e = lane; e < tw; e += 32) {
-      int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-      if ((a + 1) * (a + 2) / 2 <= e) ++a;
-      if (a * (a + 1) / 2 > e) --a;
-      const int b = e - a * (a + 1) / 2;
-      const int ra = c + 1 + a, rb = c + 1 + b;
-      L[ra * ldl + rb] = fma(-L[ra * ldl + c], L[rb * ldl + c], L[ra * ldl + rb]);
+      const int t = tri[e], ra = (t >> 8) * ldl, rb = t & 255;
+      Lc[ra + rb + 1] = fma(-Lc[ra], Lc[rb * ldl], Lc[ra + rb + 1]);
     }
     __syncwarp();
   }
@@ -126,6 +131,27 @@ __device__ __forceinline__ void warp_chol_solve(const T *L, int ldl, int n, T *v
     if (lane == 0) v[c] = vc;
     __syncwarp();
   }
+}
+
+// The same solve for n <= 32 with v in registers, lane a holding v_a: the
+// updates of one column need v_c by a shuffle, and L's columns are loaded ahead
+// (through shared memory each column was two warp barriers and a store-load round
+// trip on the solve's serial chain).
+__device__ __forceinline__ float lane_chol_solve(const float *L, int ldl, int n, float v, int lane) {
+  const float *row = L + (lane < n ? lane : 0) * ldl;
+  for (int c = 0; c < n; ++c) {
+    const float l = row[c];
+    const float vc = __shfl_sync(0xffffffffu, v, c) * L[c * ldl + c];
+    if (lane > c) v = fmaf(-l, vc, v);
+    if (lane == c) v = vc;
+  }
+  for (int c = n - 1; c >= 0; --c) {
+    const float l = L[c * ldl + (lane < c ? lane : c)];
+    const float vc = __shfl_sync(0xffffffffu, v, c) * L[c * ldl + c];
+    if (lane < c) v = fmaf(-l, vc, v);
+    if (lane == c) v = vc;
+  }
+  return v;
 }
 
 // Q = G^{-1} in three steps, spread over the GPU (a single block doing it
@@ -259,9 +285,9 @@ struct BppWarp {
   bool refine;  // solves through G^{-1} take a refinement step
   float *Lf;       // FP32 Cholesky factor (kh x ldl)
   float *bh, *bl;  // right-hand side pair (k each)
-  float *dv;       // corrections (k)
   int *Fl, *Bl;
   float *xa;
+  const uint16_t *tri;  // tri_table of n <= k / 2
   float *rsf;  // r in FP32, by index
   float *vh, *vl;  // solution pairs: x_F in F order or Q_BB^{-1} z_B in B order
   int ldl, kh;
@@ -271,7 +297,7 @@ struct BppWarp {
 // the caller synchronises) and return warp wib's view.
 __device__ __forceinline__ BppWarp bpp_stage(const double *__restrict__ Gd,
                                              const float *__restrict__ Qsg, const int *q_ok, int k,
-                                             double *sm, int wib) {
+                                             double *sm, const uint16_t *tri, int wib) {
   const BppLayout lay = bpp_layout(k);
   float *Qs = reinterpret_cast<float *>(sm);                        // hi (k^2), lo (k^2)
   float *Gp = reinterpret_cast<float *>(sm + (size_t)k * k);        // hi (k^2), lo (k^2)
@@ -305,8 +331,7 @@ __device__ __forceinline__ BppWarp bpp_stage(const double *__restrict__ Gd,
   w.Lf = base;
   w.bh = base + 2 * (((size_t)lay.kh * lay.ldl + 1) / 2);
   w.bl = w.bh + kf;
-  w.dv = w.bl + kf;
-  w.Fl = reinterpret_cast<int *>(w.dv + kf);  // passive indices, ascending (k)
+  w.Fl = reinterpret_cast<int *>(w.bl + kf);  // passive indices, ascending (k)
   w.Bl = w.Fl + k;                            // active indices, ascending (k)
   w.xa = reinterpret_cast<float *>(w.Bl + k);  // |x_F| in FP32, F order
   w.rsf = w.xa + kf;
@@ -314,6 +339,7 @@ __device__ __forceinline__ BppWarp bpp_stage(const double *__restrict__ Gd,
   w.vl = w.vh + kf;
   w.ldl = lay.ldl;
   w.kh = lay.kh;
+  w.tri = tri;
   return w;
 }
 
@@ -349,10 +375,70 @@ __device__ __forceinline__ void pair_dot(const float *Mh, const float *Ml, int k
   l = __fsub_rn(lo, __fsub_rn(h, hi));
 }
 
-__device__ __forceinline__ float warp_max(float v) {
+// Packed FP32 pairs of two columns j at once (the two entries of a lane, k > 32):
+// the same operations in half the issue slots, so the same bits.  sub2(x, y) is
+// one FMA with -1, rounded once like x - y.
+using aunmf::ptx::add2;
+using aunmf::ptx::f32x2;
+using aunmf::ptx::fma2;
+using aunmf::ptx::hi32;
+using aunmf::ptx::lo32;
+using aunmf::ptx::mul2;
+using aunmf::ptx::pack2;
+__device__ __forceinline__ f32x2 sub2(f32x2 x, f32x2 y) { return fma2(y, pack2(-1.f, -1.f), x); }
+// two_fma_acc for both columns: hi + lo += m x (x in both halves, nx = -x)
+__device__ __forceinline__ void two_fma_acc2(f32x2 m, f32x2 x, f32x2 nx, f32x2 &hi, f32x2 &lo) {
+  const f32x2 p = mul2(m, x);
+  const f32x2 ne = fma2(m, nx, p);  // - (m x - p)
+  const f32x2 s = add2(hi, p);
+  const f32x2 z = sub2(s, hi);
+  const f32x2 t = add2(sub2(hi, sub2(s, z)), sub2(p, z));
+  lo = add2(lo, sub2(t, ne));
+  hi = s;
+}
+
+// Lane's columns of a k x k matrix: j_t = lane + 32 t, clamped into the matrix
+// (the values of a column that does not exist are not used).
+template <int KT>
+struct LaneCols {
+  int j[KT];
+  __device__ __forceinline__ LaneCols(int k, int lane) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+    for (int t = 0; t < KT; ++t) j[t] = lane + 32 * t < k ? lane + 32 * t : (lane < k ? lane : 0);
+  }
+};
+
+// pair_dot of all the lane's columns at once: (h[t], l[t]) = sum_b M(I[b], j_t) x_b.
+template <int KT>
+__device__ __forceinline__ void pair_dots(const float *Mh, const float *Ml, int k, const int *I,
+                                          int n, const LaneCols<KT> &J, const float *xh,
+                                          const float *xl, float (&h)[KT], float (&l)[KT]) {
+  if constexpr (KT == 1) {
+    pair_dot(Mh, Ml, k, I, n, J.j[0], xh, xl, h[0], l[0]);
+  } else {
+    f32x2 hi = 0, lo = 0;
+#pragma unroll 2
+    for (int b = 0; b < n; ++b) {
+      const int e = I[b] * k;
+      const f32x2 mh = pack2(Mh[e + J.j[0]], Mh[e + J.j[1]]);
+      const f32x2 ml = pack2(Ml[e + J.j[0]], Ml[e + J.j[1]]);
+      const float p = xh[b], q = xl[b];
+      two_fma_acc2(mh, pack2(p, p), pack2(-p, -p), hi, lo);
+      lo = fma2(mh, pack2(q, q), lo);
+      lo = fma2(ml, pack2(p, p), lo);
+    }
+    const f32x2 hh = add2(hi, lo), ll = sub2(lo, sub2(hh, hi));
+    h[0] = lo32(hh);
+    h[1] = hi32(hh);
+    l[0] = lo32(ll);
+    l[1] = hi32(ll);
+  }
+}
+
+// Maximum over the warp of values >= 0 (their bits order as integers; a NaN
+// counts as 0).
+__device__ __forceinline__ float warp_max(float v) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(v, 0.f))));
 }
 
 constexpr int kRefineSteps = 6;
@@ -369,36 +455,34 @@ constexpr float kRefineTol = 9.31322575e-10f;  // 2^-30
 // ill-conditioned M); the caller then takes the FP64 solve.
 __device__ __forceinline__ bool solve_mixed(const float *Mh, const float *Ml, int k, const int *I,
                                             int n, const float *bh, const float *bl, float *Lf,
-                                            int ldl, float *d, float *xh, float *xl, int lane) {
+                                            int ldl, const uint16_t *tri, float *xh, float *xl,
+                                            int lane) {
   auto Mf = [Mh, k](int a, int b) { return Mh[a * k + b]; };
-  if (!warp_cholesky(Mf, I, n, Lf, ldl, lane)) return false;
-  for (int a = lane; a < n; a += 32) {
-    xh[a] = 0.f;
-    xl[a] = 0.f;
-    d[a] = bh[a];
-  }
-  __syncwarp();
+  if (!warp_cholesky(Mf, I, n, Lf, ldl, tri, lane)) return false;
+  // lane a < n holds x_a, b_a and the correction d_a (n <= k / 2 <= 32); x is also
+  // kept in shared memory for the residual
+  const bool own = lane < n;
+  const float b_h = own ? bh[lane] : 0.f, b_l = own ? bl[lane] : 0.f;
+  float x_h = 0.f, x_l = 0.f, d = b_h;
+  const int row = own ? I[lane] : 0;
   for (int step = 0; step < kRefineSteps; ++step) {
-    warp_chol_solve(Lf, ldl, n, d, lane);
-    float dm = 0.f, xm = 0.f;
-    for (int a = lane; a < n; a += 32) {
-      pair_add(xh[a], xl[a], d[a], 0.f);
-      dm = fmaxf(dm, fabsf(d[a]));
-      xm = fmaxf(xm, fabsf(xh[a]));
+    d = lane_chol_solve(Lf, ldl, n, d, lane);
+    if (own) pair_add(x_h, x_l, d, 0.f);
+    const float dm = warp_max(own ? fabsf(d) : 0.f), xm = warp_max(own ? fabsf(x_h) : 0.f);
+    __syncwarp();
+    if (own) {
+      xh[lane] = x_h;
+      xl[lane] = x_l;
     }
-    dm = warp_max(dm);
-    xm = warp_max(xm);
     if (dm <= kRefineTol * xm) return true;
     if (!(dm < 3.0e38f)) return false;
     __syncwarp();
-    for (int a = lane; a < n; a += 32) {
-      float h, l;
-      pair_dot(Mh, Ml, k, I, n, I[a], xh, xl, h, l);  // (M x)_a
-      float rh = bh[a], rl = bl[a];
+    if (own) {
+      float h, l, rh = b_h, rl = b_l;
+      pair_dot(Mh, Ml, k, I, n, row, xh, xl, h, l);  // (M x)_a
       pair_add(rh, rl, -h, -l);
-      d[a] = __fadd_rn(rh, rl);
+      d = __fadd_rn(rh, rl);
     }
-    __syncwarp();
   }
   return false;
 }
@@ -427,7 +511,6 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
   const bool have_q = w.have_q;
   float *Lf = w.Lf;
   float *bh = w.bh, *bl = w.bl;  // right-hand side pair
-  float *dv = w.dv;              // corrections
   float *vh = w.vh, *vl = w.vl;  // solution pairs: F order (x_F) or B order (Q_BB^-1 z_B)
   int *Fl = w.Fl, *Bl = w.Bl;
   float *xa = w.xa, *rsf = w.rsf;
@@ -454,20 +537,32 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
   // all, for warm 2)
   float zh[KT], zl[KT];
   bool have_z = false;
+  const LaneCols<KT> J(k, lane);
   auto form_z = [&]() {
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      // z_j = sum_l (Qh + Ql)_lj r_l, r_l an FP32 value
-      const int j = lane + 32 * t;
+    // z_j = sum_l (Qh + Ql)_lj r_l, r_l an FP32 value
+    if constexpr (KT == 1) {
       float hi = 0.f, lo = 0.f;
-      if (j < k)
-        for (int l = 0; l < k; ++l) {
-          const float rl = rsf[l];
-          two_fma_acc(Qh[l * k + j], rl, hi, lo);
-          lo = fmaf(Ql[l * k + j], rl, lo);
-        }
-      zh[t] = __fadd_rn(hi, lo);
-      zl[t] = __fsub_rn(lo, __fsub_rn(zh[t], hi));
+      for (int l = 0; l < k; ++l) {
+        const float rl = rsf[l];
+        two_fma_acc(Qh[l * k + J.j[0]], rl, hi, lo);
+        lo = fmaf(Ql[l * k + J.j[0]], rl, lo);
+      }
+      zh[0] = __fadd_rn(hi, lo);
+      zl[0] = __fsub_rn(lo, __fsub_rn(zh[0], hi));
+    } else {
+      f32x2 hi = 0, lo = 0;
+#pragma unroll 2
+      for (int l = 0; l < k; ++l) {
+        const float rl = rsf[l];
+        const f32x2 rr = pack2(rl, rl);
+        two_fma_acc2(pack2(Qh[l * k + J.j[0]], Qh[l * k + J.j[1]]), rr, pack2(-rl, -rl), hi, lo);
+        lo = fma2(pack2(Ql[l * k + J.j[0]], Ql[l * k + J.j[1]]), rr, lo);
+      }
+      const f32x2 h = add2(hi, lo), l = sub2(lo, sub2(h, hi));
+      zh[0] = lo32(h);
+      zh[1] = hi32(h);
+      zl[0] = lo32(l);
+      zl[1] = hi32(l);
     }
     have_z = true;
   };
@@ -520,7 +615,7 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
         __syncwarp();
         // a system the FP32 solve cannot finish (an ill-conditioned G_FF)
         // sends the row to the FP64 fallback kernel
-        if (!solve_mixed(Gh, Gl, k, Fl, nf, bh, bl, Lf, ldl, dv, vh, vl, lane)) {
+        if (!solve_mixed(Gh, Gl, k, Fl, nf, bh, bl, Lf, ldl, w.tri, vh, vl, lane)) {
           failed_numeric = true;
           break;
         }
@@ -542,21 +637,21 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
           }
         __syncwarp();
         // (vh, vl)[0..nb) = Q_BB^{-1} z_B = -y_B
-        if (!solve_mixed(Qh, Ql, k, Bl, nb, bh, bl, Lf, ldl, dv, vh, vl, lane)) {
+        if (!solve_mixed(Qh, Ql, k, Bl, nb, bh, bl, Lf, ldl, w.tri, vh, vl, lane)) {
           failed_numeric = true;
           break;
         }
         __syncwarp();
+        float h[KT], l[KT];
+        pair_dots<KT>(Qh, Ql, k, Bl, nb, J, vh, vl, h, l);
 #pragma unroll
         for (int t = 0; t < KT; ++t) {
           const int j = lane + 32 * t;
           xh[t] = xl[t] = 0.f;
           if (j < k && pas[t]) {
-            float h, l;
-            pair_dot(Qh, Ql, k, Bl, nb, j, vh, vl, h, l);
             xh[t] = zh[t];
             xl[t] = zl[t];
-            pair_add(xh[t], xl[t], -h, -l);
+            pair_add(xh[t], xl[t], -h[t], -l[t]);
           }
           if (j < k && !pas[t]) {
             yh[t] = -vh[posb[t]];
@@ -582,14 +677,14 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
           // on a par with the ~1e-14 to which G itself is formed.  r in FP32
           // (rsf) is no longer needed: z is formed, and a direct solve takes
           // r from the lanes' registers.
+          pair_dots<KT>(Gh, Gl, k, Fl, nf, J, vh, vl, h, l);
 #pragma unroll
           for (int t = 0; t < KT; ++t) {
             const int j = lane + 32 * t;
             float rho = 0.f;
             if (j < k && pas[t]) {
-              float h, l, rh = rf[t], rl = 0.f;
-              pair_dot(Gh, Gl, k, Fl, nf, j, vh, vl, h, l);
-              pair_add(rh, rl, -h, -l);
+              float rh = rf[t], rl = 0.f;
+              pair_add(rh, rl, -h[t], -l[t]);
               rho = __fadd_rn(rh, rl);
             }
             if (j < k) rsf[j] = rho;
@@ -601,13 +696,21 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
           // of the pair form's instructions (the residual rho above is the
           // part that needs the pairs)
           float zrh[KT], zrl[KT];
+          if constexpr (KT == 1) {
+            float hi = 0.f;
+            for (int a = 0; a < k; ++a) hi = fmaf(Qh[a * k + J.j[0]], rsf[a], hi);
+            zrh[0] = hi;
+          } else {
+            f32x2 hi = 0;
+#pragma unroll 4
+            for (int a = 0; a < k; ++a)
+              hi = fma2(pack2(Qh[a * k + J.j[0]], Qh[a * k + J.j[1]]), pack2(rsf[a], rsf[a]), hi);
+            zrh[0] = lo32(hi);
+            zrh[1] = hi32(hi);
+          }
 #pragma unroll
           for (int t = 0; t < KT; ++t) {
-            const int j = lane + 32 * t;
-            float hi = 0.f;
-            if (j < k)
-              for (int l = 0; l < k; ++l) hi = fmaf(Qh[l * k + j], rsf[l], hi);
-            zrh[t] = hi;
+            if (lane + 32 * t >= k) zrh[t] = 0.f;
             zrl[t] = 0.f;
           }
 #pragma unroll
@@ -617,18 +720,18 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
               bl[posb[t]] = zrl[t];
             }
           __syncwarp();
-          if (!solve_mixed(Qh, Ql, k, Bl, nb, bh, bl, Lf, ldl, dv, vh, vl, lane)) {
+          if (!solve_mixed(Qh, Ql, k, Bl, nb, bh, bl, Lf, ldl, w.tri, vh, vl, lane)) {
             failed_numeric = true;
             break;
           }
           __syncwarp();
+          pair_dots<KT>(Qh, Ql, k, Bl, nb, J, vh, vl, h, l);
 #pragma unroll
           for (int t = 0; t < KT; ++t) {
             const int j = lane + 32 * t;
             if (j < k && pas[t]) {
-              float h, l, ch = zrh[t], cl = zrl[t];
-              pair_dot(Qh, Ql, k, Bl, nb, j, vh, vl, h, l);
-              pair_add(ch, cl, -h, -l);
+              float ch = zrh[t], cl = zrl[t];
+              pair_add(ch, cl, -h[t], -l[t]);
               pair_add(xh[t], xl[t], ch, cl);
             }
           }
@@ -640,14 +743,13 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
               vl[posf[t]] = xl[t];
             }
           __syncwarp();
+          pair_dots<KT>(Gh, Gl, k, Fl, nf, J, vh, vl, h, l);
 #pragma unroll
           for (int t = 0; t < KT; ++t) {
             const int j = lane + 32 * t;
             if (j < k && !pas[t]) {
-              float h, l;
-              pair_dot(Gh, Gl, k, Fl, nf, j, vh, vl, h, l);
-              yh[t] = h;
-              yl[t] = l;
+              yh[t] = h[t];
+              yl[t] = l[t];
               pair_add(yh[t], yl[t], -rf[t], 0.f);
             }
           }
@@ -659,6 +761,21 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
       for (int t = 0; t < KT; ++t)
         if (pas[t]) xa[posf[t]] = fabsf(__fadd_rn(xh[t], xl[t]));
       __syncwarp();
+      float mag[KT], h[KT], l[KT];
+      if constexpr (KT == 1) {
+        mag[0] = fabsf(rf[0]);
+        for (int a = 0; a < nf; ++a) mag[0] = fmaf(fabsf(Gh[Fl[a] * k + J.j[0]]), xa[a], mag[0]);
+      } else {
+        f32x2 m = pack2(fabsf(rf[0]), fabsf(rf[1]));
+#pragma unroll 4
+        for (int a = 0; a < nf; ++a) {
+          const float *g = Gh + Fl[a] * k;
+          m = fma2(pack2(fabsf(g[J.j[0]]), fabsf(g[J.j[1]])), pack2(xa[a], xa[a]), m);
+        }
+        mag[0] = lo32(m);
+        mag[1] = hi32(m);
+      }
+      if (direct) pair_dots<KT>(Gh, Gl, k, Fl, nf, J, vh, vl, h, l);
 #pragma unroll
       for (int t = 0; t < KT; ++t) {
         const int j = lane + 32 * t;
@@ -667,14 +784,10 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
           yh[t] = yl[t] = 0.f;
           tauf[t] = 0.f;
         } else {
-          float mag = fabsf(rf[t]);
-          for (int a = 0; a < nf; ++a) mag = fmaf(fabsf(Gh[Fl[a] * k + j]), xa[a], mag);
-          tauf[t] = kBppYTolF * mag;
+          tauf[t] = kBppYTolF * mag[t];
           if (direct) {
-            float h, l;
-            pair_dot(Gh, Gl, k, Fl, nf, j, vh, vl, h, l);
-            yh[t] = h;
-            yl[t] = l;
+            yh[t] = h[t];
+            yl[t] = l[t];
             pair_add(yh[t], yl[t], -rf[t], 0.f);
           }
         }
@@ -734,7 +847,8 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
 // passive system solved by a Cholesky factorisation of G_FF of any size.
 template <int KT>
 __device__ __forceinline__ int bpp_row_direct(const double *__restrict__ G, double *L, double *v,
-                                              double *rs, int *Fl, const float *__restrict__ R,
+                                              double *rs, int *Fl, const uint16_t *tri,
+                                              const float *__restrict__ R,
                                               int64_t row, int k, float *__restrict__ X, int warm,
                                               int max_piv, bool *failed_numeric_out,
                                               bool *failed_cap_out) {
@@ -784,7 +898,7 @@ __device__ __forceinline__ int bpp_row_direct(const double *__restrict__ G, doub
         if (pas[t] && AUNMF_BOUND(pos[t] < k && lane + 32 * t < k, AUNMF_CHECK_BPP_LIST))
           Fl[pos[t]] = lane + 32 * t;
       __syncwarp();
-      if (!warp_cholesky([G, k](int a, int b) { return G[a * k + b]; }, Fl, nf, L, ldl, lane)) {
+      if (!warp_cholesky([G, k](int a, int b) { return G[a * k + b]; }, Fl, nf, L, ldl, tri, lane)) {
         failed_numeric = true;
         break;
       }

@@ -319,6 +319,8 @@ __global__ void __launch_bounds__(32 * bpp::kBppWarps, 1)
     g_bpp(const BInst *__restrict__ P, const Item *__restrict__ items, int nitems, int side,
           int max_piv, int cold, DevCounters *ctr) {
   extern __shared__ double sm[];
+  __shared__ uint16_t tri[32 * 33 / 2];
+  bpp::tri_table(tri, 32);  // (synchronised with the first item's staging)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int nwb = blockDim.x >> 5;
   long long piv_total = 0, nonconv = 0;
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(32 * bpp::kBppWarps, 1)
       continue;
     __syncthreads();
     const bpp::BppWarp w =
-        bpp::bpp_stage(side ? b.GW : b.GH, reinterpret_cast<const float *>(b.Q), b.q_ok, k, sm, wib);
+        bpp::bpp_stage(side ? b.GW : b.GH, reinterpret_cast<const float *>(b.Q), b.q_ok, k, sm, tri, wib);
     __syncthreads();
     const float *R = side ? b.PHt : b.PW;
     float *X = side ? b.Ht : b.W;
@@ -368,6 +370,8 @@ __global__ void __launch_bounds__(256)
     g_bpp_direct(const BInst *__restrict__ P, const Item *__restrict__ items, int nitems,
                  int side, int max_piv, int cold, DevCounters *ctr) {
   extern __shared__ double sm[];
+  __shared__ uint16_t tri[64 * 65 / 2];
+  bpp::tri_table(tri, 64);  // (synchronised with the first flagged item's staging)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int nwb = blockDim.x >> 5;
   long long piv_total = 0, nonconv = 0, numeric = 0, redone = 0;
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(256)
     for (int64_t row = I.r0 + wib; row < I.r1; row += nwb) {
       if (!b.redo[row]) continue;
       bool fnum, fcap;
-      const int n_ex = bpp::bpp_row_direct<KT>(G, L, v, rs, Fl, R, row, k, X, cold ? 0 : 1, max_piv,
+      const int n_ex = bpp::bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X, cold ? 0 : 1, max_piv,
                                                     &fnum, &fcap);
       piv_total += n_ex;
       nonconv += fcap;

@@ -53,7 +53,9 @@ __global__ void __launch_bounds__(32 * kBppWarps, 1)
   extern __shared__ double sm[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int nwb = blockDim.x >> 5;
-  const BppWarp w = bpp_stage(Gd, Qg, q_ok, k, sm, wib);
+  __shared__ uint16_t tri[32 * 33 / 2];
+  tri_table(tri, k / 2 > 0 ? k / 2 : 1);
+  const BppWarp w = bpp_stage(Gd, Qg, q_ok, k, sm, tri, wib);
   __syncthreads();
   // a run's first iteration (no relres written yet): the previous iterate is
   // the random start (or W = 0), so the solves start from the signs of the
@@ -111,6 +113,26 @@ __global__ void __launch_bounds__(256)
                  float *__restrict__ X, int warm, int max_piv, DevCounters *ctr,
                  const uint8_t *__restrict__ redo) {
   extern __shared__ double sm[];
+  __shared__ uint16_t tri[64 * 65 / 2];
+  __shared__ int any;
+  // the block's rows are flagged rarely: look before staging anything
+  if (threadIdx.x == 0) any = 0;
+  __syncthreads();
+  {
+    const int nwb = blockDim.x >> 5;  // the block's rows: groups of nwb, gridDim.x apart
+    const int per = blockDim.x / nwb;
+    int mine = 0;
+    if ((int)threadIdx.x < per * nwb)
+      for (int64_t g = blockIdx.x + (int64_t)gridDim.x * (threadIdx.x / nwb);; g += (int64_t)gridDim.x * per) {
+        const int64_t row = g * nwb + threadIdx.x % nwb;
+        if (g * nwb >= rows) break;
+        if (row < rows) mine |= redo[row];
+      }
+    if (mine) any = 1;
+  }
+  __syncthreads();
+  if (!any) return;
+  tri_table(tri, k);
   const int ldl = k | 1;
   double *G = sm;
   for (int e = threadIdx.x; e < k * k; e += blockDim.x) G[e] = Gd[e];
@@ -126,7 +148,7 @@ __global__ void __launch_bounds__(256)
        row += (int64_t)gridDim.x * nwb) {
     if (!redo[row]) continue;
     bool fnum, fcap;
-    const int it = bpp_row_direct<KT>(G, L, v, rs, Fl, R, row, k, X, warm, max_piv, &fnum, &fcap);
+    const int it = bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X, warm, max_piv, &fnum, &fcap);
     piv_total += it;
     nonconv += fcap;
     numeric += fnum;
