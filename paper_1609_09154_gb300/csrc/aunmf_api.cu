@@ -726,10 +726,14 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
     // bytes; 14.4 against 3.7 ms for the norm alone at 96000 x 64000), at
     // products 8 % slower than on the copies there, up to 25 % where the tiles
     // fill the SMs badly (24000 x 16000, where 10 iterations with the copies
-    // take 7.53 ms, without 7.37): the line is at 12 iterations.  BF16 copies
-    // halve every product's bytes and repay the pass from the second iteration
-    // on.  A in host memory is read once, into copies.
-    c.direct = use_split(k) && !a_host && iters <= (o.prec == AUNMF_TF32 ? 12 : 1);
+    // take 7.53 ms, without 7.37): the line is at 12 iterations; at 3 when A's
+    // rows are not 16-byte aligned, whose direct products take 1.8 times those on
+    // copies (38912 x 8193, k = 50: 0.41 against 0.23 ms).  BF16 copies halve every
+    // product's bytes and repay the pass from the second iteration on.  A in host
+    // memory is read once, into copies.
+    const bool aligned = (reinterpret_cast<uintptr_t>(A->dense) & 15) == 0 && (A->lda & 3) == 0;
+    c.direct = use_split(k) && !a_host &&
+               iters <= (o.prec == AUNMF_BF16 ? 1 : aligned ? 12 : 3);
     int prc = prepare_tc(h, c, kPrepAht | kPrepWta | kPrepNorm, s);
     if (prc != AUNMF_OK) return prc;
   } else if (A->dense) {

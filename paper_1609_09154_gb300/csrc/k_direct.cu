@@ -19,9 +19,16 @@
 //                in turn: read a raw tile, round to nearest TF32 / BF16 and write
 //                the K-major 128-byte-swizzled operand tile; a group's first
 //                thread also issues the copy of the stage's Y tile
-// A raw tile is 32 KB; an operand stage is 32 (TF32) or 64 (BF16) K.  When A's
-// rows are not 16-byte aligned (TMA cannot read them) the converters fill the
-// raw ring themselves with 4-byte asynchronous copies (two slots a group).
+// A raw tile is 32 KB; an operand stage is 32 (TF32) or 64 (BF16) K.
+// When A's rows are not 16-byte aligned (lda % 4 != 0) no tensor map describes A,
+// but the rows r = c (mod 4) are 16 lda bytes apart: four maps, each based on the
+// 16-byte boundary at or before row c, whose rows start sh_c = 0 to 3 floats later.
+// A tile is then four boxes 36 floats wide (AHT), or eight of 132 (!AHT), and the
+// converters read each row at its class's shift.  (Row by row with untiled bulk
+// copies it ran at 0.62 TB/s (AHT, 144-byte copies) and 2.6 TB/s (1,040 bytes);
+// with 4-byte asynchronous copies at 1.6 TB/s; this way at 3.0 (TF32, the converters'
+// scalar reads) and 4.2 (BF16) against 5.5 for aligned rows, whole calls at 38912 x
+// 8192, k = 50.)
 // The operands, MMA order and chain lengths are those of k_gemm_tc, so the
 // products are the same to the bit.
 //
@@ -55,13 +62,24 @@ using namespace aunmf::ptx;
 
 constexpr int kDThreads = 576;       // 18 warps
 constexpr int kDGroup = 128;         // threads of one of the two converter groups
-constexpr int kRaw = 4, kOp = 2;     // ring depths (group g writes operand slot g)
+constexpr int kOp = 2;               // operand slots (group g writes slot g)
+// Raw ring: four tiles of 32 KB; unaligned rows: three of 256 rows of 36 floats
+// (AHT; class c's 64 rows together) or of 4 classes x 2 halves x 8 K-rows x 132.
+template <bool VEC>
+struct Raw {
+  static constexpr int N = VEC ? 4 : 3;
+  static constexpr uint32_t kBytes = VEC ? 32768 : 256 * 36 * 4;
+};
+constexpr int kWAht = 36, kWWta = 132;  // box widths of the unaligned form (floats)
+static_assert(64 * kWWta <= 256 * kWAht, "one slot size for both directions");
+struct MapsA {
+  CUtensorMap m[4];  // VEC: m[0]
+};
 constexpr int kDTileM = 256;
-constexpr uint32_t kRawBytes = 32768;
 constexpr uint32_t kXBytes = 32768;  // operand tile of X: 256 rows x 128 bytes
 
 struct DirectArgs {
-  const float *A;      // m x n, lda (unaligned form)
+  const float *A;      // m x n, lda (for the shifts of unaligned rows)
   int64_t lda;
   int64_t M, K;        // C's rows, the contraction
   int64_t units;       // (tiles of 256 rows) x S
@@ -80,17 +98,6 @@ struct DirectArgs {
 
 // all converters
 __device__ __forceinline__ void conv_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-// the barrier of converter group g with a vote: true if all of it is `ok`
-__device__ __forceinline__ bool group_bar_and(int g, bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, %2, 128, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)ok), "r"(g + 2)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void fence_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -102,13 +109,15 @@ __device__ __forceinline__ void pair_acc(float x, float &h, float &l) {
   h = s;
 }
 
-template <bool AHT, bool BF16, bool TMA, bool NORM>
+template <bool AHT, bool BF16, bool VEC, bool NORM>
 __global__ void __launch_bounds__(kDThreads, 1)
-    k_gemm_direct(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapY,
+    k_gemm_direct(const __grid_constant__ MapsA mapA, const __grid_constant__ CUtensorMap mapY,
                   const DirectArgs L) {
   constexpr int RPS = BF16 ? 2 : 1;   // raw tiles per operand stage
   constexpr int KS = 32 * RPS;        // K per operand stage (128 bytes)
   constexpr int KPM = BF16 ? 16 : 8;  // K per MMA (32 bytes)
+  constexpr int kRaw = Raw<VEC>::N;
+  constexpr uint32_t kRawBytes = Raw<VEC>::kBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023);
   const uint32_t ybytes = (uint32_t)L.BN * 128, opbytes = kXBytes + ybytes;
@@ -141,7 +150,8 @@ __global__ void __launch_bounds__(kDThreads, 1)
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async();
-    if (TMA) asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA) : "memory");
+    for (int c = 0; c < (VEC ? 1 : 4); ++c)
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA.m[c]) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapY) : "memory");
   }
   if (warp == 1) tmem_alloc(tslot, L.tmem_cols);
@@ -158,8 +168,9 @@ __global__ void __launch_bounds__(kDThreads, 1)
   };
 
   if (warp == 0) {
-    if (TMA && lane == 0) {
+    if (lane == 0) {
       const uint64_t pol = policy_evict_first();  // A streams through once
+      constexpr uint32_t kTx = VEC ? 32768 : 4u * (AHT ? 256 * kWAht : 64 * kWWta);
       int r = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -169,15 +180,28 @@ __global__ void __launch_bounds__(kDThreads, 1)
         range(u, tile, s0, s1);
         for (int64_t t = s0 * RPS; t < s1 * RPS; ++t) {
           if (!mbar_wait(&rempty[r], ph ^ 1u, L.err, L.wait_cycles)) { ok = false; break; }
-          mbar_expect_tx(&rfull[r], kRawBytes);
+          mbar_expect_tx(&rfull[r], kTx);
+          uint8_t *dst = raw + (size_t)r * kRawBytes;
           const int kc = (int)(t * 32), mc = (int)(tile * kDTileM);
-          // (checked build: a bad coordinate skips the copy; the stage then
+          // (checked build: a bad coordinate skips the copies; the stage then
           // never fills and the bounded waits end the launch)
           if (AUNMF_BOUND(kc >= 0 && mc >= 0 && t * 32 <= 0x7fffffffLL, AUNMF_CHECK_TMA_COORD)) {
-            if (AHT)
-              tma_load_2d(raw + (size_t)r * kRawBytes, &mapA, &rfull[r], kc, mc, pol);
-            else
-              tma_load_2d(raw + (size_t)r * kRawBytes, &mapA, &rfull[r], mc, kc, pol);
+            if constexpr (VEC) {
+              if (AHT)
+                tma_load_2d(dst, &mapA.m[0], &rfull[r], kc, mc, pol);
+              else
+                tma_load_2d(dst, &mapA.m[0], &rfull[r], mc, kc, pol);
+            } else {
+              for (int c = 0; c < 4; ++c) {  // (tiles start at multiples of 4 rows)
+                if (AHT) {
+                  tma_load_2d(dst + c * 64 * kWAht * 4, &mapA.m[c], &rfull[r], kc, mc >> 2, pol);
+                } else {
+                  uint8_t *d = dst + c * 16 * kWWta * 4;
+                  tma_load_2d(d, &mapA.m[c], &rfull[r], mc, kc >> 2, pol);
+                  tma_load_2d(d + 8 * kWWta * 4, &mapA.m[c], &rfull[r], mc + kWWta, kc >> 2, pol);
+                }
+              }
+            }
           }
           ++issued;
           if (++r == kRaw) { r = 0; ph ^= 1u; }
@@ -290,27 +314,6 @@ __global__ void __launch_bounds__(kDThreads, 1)
     auto pack_bf = [&](float a, float b) {  // (values already BF16-valued) -> bf16x2
       return (__float_as_uint(a) >> 16) | (__float_as_uint(b) & 0xffff0000u);
     };
-    // unaligned form: raw tile tr of `tile` into slot `slot` of the group, 4-byte
-    // copies (AHT: a warp per row, a lane per K; !AHT: a thread per column)
-    auto fetch = [&](int64_t tile, int64_t tr, int slot) {
-      float *dst = reinterpret_cast<float *>(raw + (size_t)slot * kRawBytes);
-      const int64_t k0 = tr * 32, m0 = tile * kDTileM;
-      if constexpr (AHT) {
-        const int64_t kk = k0 + lane;
-        for (int i = 0; i < 64; ++i) {
-          const int row = (t >> 5) * 64 + i;
-          const bool in = kk < L.K && m0 + row < L.M;
-          cp_async4(dst + row * 32 + (((lane >> 2) ^ (row & 7)) << 2) + (lane & 3),
-                    in ? L.A + (m0 + row) * L.lda + kk : L.A, in);
-        }
-      } else {
-        for (int i = 0; i < 64; ++i) {
-          const int kk = i >> 1, col = t + 128 * (i & 1);
-          const bool in = m0 + col < L.M && k0 + kk < L.K;
-          cp_async4(dst + kk * 256 + col, in ? L.A + (k0 + kk) * L.lda + m0 + col : L.A, in);
-        }
-      }
-    };
     // The CTA's operand stages are numbered q = 0, 1, ... over its units; group
     // g takes q = g, g + 2, ...  Walks them: unit u, stage s of it.
     struct Walk {
@@ -331,58 +334,60 @@ __global__ void __launch_bounds__(kDThreads, 1)
     Walk w{(int64_t)blockIdx.x, 0, 0, 0, 0};
     enter(w);
     step(w, grp);
-    // unaligned form: the group's raw tiles are fetched one ahead into its two
-    // slots, 2 g and 2 g + 1
-    Walk f = w;
-    int fh = 0;
-    int64_t fn = 0, rn = 0;  // raw tiles fetched / converted by the group
-    auto fetch_next = [&]() {
-      if (f.u < L.units) {
-        fetch(f.tile, f.s * RPS + fh, 2 * grp + (int)(fn & 1));
-        ++fn;
-        if (++fh == RPS) {
-          fh = 0;
-          step(f, 2);
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    if constexpr (!TMA) fetch_next();
-    bool go = true;  // (without TMA the group leaves the loop as one, by its vote)
-    for (; w.u < L.units && go; step(w, 2)) {
+    // unaligned form: the shift of class c, and (!AHT) the place of this thread's
+    // rows t and t + 128 in class c's first K-row
+    int sh[4], o0[4], o1[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sh[c] = VEC ? 0 : (int)(((reinterpret_cast<uintptr_t>(L.A) >> 2) + c * (L.lda & 3)) & 3);
+      const int f0 = sh[c] + t, f1 = f0 + 128;
+      o0[c] = c * 16 * kWWta + f0 + (f0 < kWWta ? 0 : 7 * kWWta);
+      o1[c] = c * 16 * kWWta + f1 + (f1 < kWWta ? 0 : 7 * kWWta);
+    }
+    for (; w.u < L.units && ok; step(w, 2)) {
       const uint32_t use_no = (uint32_t)(w.q >> 1);  // uses of operand slot grp so far
-      if (!mbar_wait(&oempty[grp], (use_no & 1u) ^ 1u, L.err, L.wait_cycles)) ok = false;
-      if (TMA && !ok) break;
+      if (!mbar_wait(&oempty[grp], (use_no & 1u) ^ 1u, L.err, L.wait_cycles)) break;
       uint8_t *xo = op + (size_t)grp * opbytes;
-      if (t == 0 && ok) {
+      if (t == 0) {
         mbar_expect_tx(&yfull[grp], ybytes);
         tma_load_2d(xo + kXBytes, &mapY, &yfull[grp], (int)(w.s * KS), 0, pol_y);
         ++yissued;
       }
 #pragma unroll
       for (int h = 0; h < RPS; ++h) {
-        int r;
-        if constexpr (TMA) {
-          const int64_t tr = w.q * RPS + h;  // raw tile number
-          r = (int)(tr % kRaw);
-          if (!mbar_wait(&rfull[r], (uint32_t)(tr / kRaw) & 1u, L.err, L.wait_cycles)) {
-            ok = go = false;
-            break;
-          }
-        } else {
-          // the group's tile has landed; after the barrier all of it is
-          // visible, and its other slot has been read
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-          if (!group_bar_and(grp, ok)) {
-            ok = go = false;
-            break;
-          }
-          fetch_next();
-          r = 2 * grp + (int)(rn++ & 1);
+        const int64_t tr = w.q * RPS + h;  // raw tile number
+        const int r = (int)(tr % kRaw);
+        if (!mbar_wait(&rfull[r], (uint32_t)(tr / kRaw) & 1u, L.err, L.wait_cycles)) {
+          ok = false;
+          break;
         }
         const float *rw = reinterpret_cast<const float *>(raw + (size_t)r * kRawBytes);
         sq = sd = 0.f;
-        if constexpr (AHT && !BF16) {
+        // (unaligned form: K past the end, which a class without rows does not
+        // zero-fill)
+        const int kv = VEC ? 32 : (int)min((int64_t)32, L.K - (w.s * RPS + h) * 32);
+        auto at = [&](int kk, int i) {  // !AHT: entry (kk, t + 128 i) of the raw tile
+          if constexpr (VEC) return rw[kk * 256 + t + 128 * i];
+          return kk < kv ? rw[(i ? o1 : o0)[kk & 3] + (kk >> 2) * kWWta] : 0.f;
+        };
+        if constexpr (AHT && !VEC) {
+          // a warp per row (TF32) or two (BF16), lanes along K
+          constexpr int LPR = BF16 ? 16 : 32;
+          const int l = lane & (LPR - 1);
+#pragma unroll 8
+          for (int row = (t >> 5) * (32 / LPR) + lane / LPR; row < 256; row += 4 * (32 / LPR)) {
+            const float *src = rw + ((row & 3) * 64 + (row >> 2)) * kWAht + sh[row & 3];
+            const int x = row & 7;
+            if constexpr (BF16) {
+              const float a = 2 * l < kv ? src[2 * l] : 0.f, b = 2 * l + 1 < kv ? src[2 * l + 1] : 0.f;
+              reinterpret_cast<uint32_t *>(xo)[row * 32 + (((4 * h + (l >> 2)) ^ x) << 2) + (l & 3)] =
+                  pack_bf(use(a), use(b));
+            } else {
+              reinterpret_cast<float *>(xo)[row * 32 + (((l >> 2) ^ x) << 2) + (l & 3)] =
+                  use(l < kv ? src[l] : 0.f);
+            }
+          }
+        } else if constexpr (AHT && !BF16) {
           // same swizzled place in the operand tile
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
@@ -408,8 +413,8 @@ __global__ void __launch_bounds__(kDThreads, 1)
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const int c = i >> 1, row = t + 128 * (i & 1);
-            const float a0 = rw[(4 * c) * 256 + row], a1 = rw[(4 * c + 1) * 256 + row];
-            const float a2 = rw[(4 * c + 2) * 256 + row], a3 = rw[(4 * c + 3) * 256 + row];
+            const float a0 = at(4 * c, i & 1), a1 = at(4 * c + 1, i & 1);
+            const float a2 = at(4 * c + 2, i & 1), a3 = at(4 * c + 3, i & 1);
             reinterpret_cast<float4 *>(xo)[row * 8 + (c ^ (row & 7))] =
                 make_float4(use(a0), use(a1), use(a2), use(a3));
           }
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
             const int c = i >> 1, row = t + 128 * (i & 1);
             float a[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) a[e] = rw[(8 * c + e) * 256 + row];
+            for (int e = 0; e < 8; ++e) a[e] = at(8 * c + e, i & 1);
             uint4 o;
             o.x = pack_bf(use(a[0]), use(a[1]));
             o.y = pack_bf(use(a[2]), use(a[3]));
@@ -436,14 +441,12 @@ __global__ void __launch_bounds__(kDThreads, 1)
         // arrival right behind the loads may be performed while they still queue
         // for shared memory, and a tile that hits L2 then overwrites the slot
         // under them (seen as values of the tile after next).
-        if constexpr (TMA) mbar_arrive(&rempty[r]);
+        mbar_arrive(&rempty[r]);
       }
-      if (!go) break;
-      if (!ok) continue;  // (without TMA: the vote at the next tile)
+      if (!ok) break;
       fence_async();
       mbar_arrive(&ofull[grp]);
     }
-    if constexpr (!TMA) cp_async_wait_all();
     if (t == 0 && yissued > 0)  // the Y copies issued land before the CTA exits
       mbar_wait_drain(&yfull[grp], (uint32_t)((yissued - 1) & 1), L.wait_cycles);
     if constexpr (NORM) {
@@ -525,14 +528,27 @@ cudaError_t launch_gemm_direct(bool aht, const float *A, int64_t m, int64_t n, i
   L.err = err;
   L.wait_cycles = fault::wait_cycles();
   L.inject = fault::site() == AUNMF_INJECT_TC_WAIT ? 1 : 0;
-  CUtensorMap mapA, mapY;
+  MapsA mapA;
+  CUtensorMap mapY;
   if (!factor_map(&mapY, Y, bf16, 2 * k, K, ldy, L.BN)) return cudaErrorInvalidValue;
-  bool tma = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (lda & 3) == 0;
-  if (tma)
-    tma = aht ? map_f32(&mapA, A, m, n, lda, 32, 256, true)
-              : map_f32(&mapA, A, m, n, lda, 256, 32, false);
-  if (!tma) mapA = mapY;  // not read
-  const size_t smem = 1024 + (size_t)kRaw * kRawBytes +
+  const bool vec = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (lda & 3) == 0;
+  for (int c = 0; c < 4; ++c) {
+    bool ok;
+    if (vec) {
+      ok = aht ? map_f32(&mapA.m[c], A, m, n, lda, 32, 256, true)
+               : map_f32(&mapA.m[c], A, m, n, lda, 256, 32, false);
+    } else {
+      // rows c, c + 4, ...; a class without rows is never used unmasked: class 0's
+      const int cc = c < m ? c : 0;
+      const uintptr_t a = reinterpret_cast<uintptr_t>(A + cc * lda), b = a & ~(uintptr_t)15;
+      ok = map_f32(&mapA.m[c], reinterpret_cast<const float *>(b), (m - cc + 3) / 4,
+                   n + (int64_t)((a - b) >> 2), 4 * lda, aht ? kWAht : kWWta, aht ? 64 : 8, false);
+    }
+    if (!ok) return cudaErrorInvalidValue;
+  }
+  const size_t raw = vec ? (size_t)Raw<true>::N * Raw<true>::kBytes
+                         : (size_t)Raw<false>::N * Raw<false>::kBytes;
+  const size_t smem = 1024 + raw +
                       (size_t)kOp * (kXBytes + (size_t)L.BN * 128) + 256;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
@@ -547,11 +563,11 @@ cudaError_t launch_gemm_direct(bool aht, const float *A, int64_t m, int64_t n, i
   };
   using Y1 = std::true_type;
   using N0 = std::false_type;
-  auto by_tma = [&](auto a, auto b, auto nm) {
-    if (tma) pick(a, b, Y1{}, nm); else pick(a, b, N0{}, nm);
+  auto by_vec = [&](auto a, auto b, auto nm) {
+    if (vec) pick(a, b, Y1{}, nm); else pick(a, b, N0{}, nm);
   };
   auto by_prec = [&](auto a, auto nm) {
-    if (bf16) by_tma(a, Y1{}, nm); else by_tma(a, N0{}, nm);
+    if (bf16) by_vec(a, Y1{}, nm); else by_vec(a, N0{}, nm);
   };
   if (aht) by_prec(Y1{}, N0{});
   else if (norm2) by_prec(N0{}, Y1{});

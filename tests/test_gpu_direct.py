@@ -57,33 +57,48 @@ def test_products(ax, m, n, k, prec):
     check(ax.wta(At, H.T.contiguous(), prec).T, A, H.T, Ar, n, prec)
 
 
-def test_repeated_products_are_equal(ax):
+@pytest.mark.parametrize("n", [1600, 1601])
+def test_repeated_products_are_equal(ax, n):
     """Many units per CTA, tiles that hit L2: the ring slots are refilled while
     the warps are far apart, and every call gives the same bits."""
     g = torch.Generator(device="cuda")
     g.manual_seed(5)
-    A = torch.rand((40000, 1600), generator=g, device="cuda")
-    H, W = torch.rand((50, 1600), generator=g, device="cuda"), torch.rand((40000, 50), generator=g, device="cuda")
+    A = torch.rand((40000, n), generator=g, device="cuda")
+    H, W = torch.rand((50, n), generator=g, device="cuda"), torch.rand((40000, 50), generator=g, device="cuda")
     for prec in ("tf32", "bf16"):
         P, Q = ax.aht(A, H, prec), ax.wta(A, W, prec)
-        check(P, A, H.T, rounded(A, prec), 1600, prec)
+        check(P, A, H.T, rounded(A, prec), n, prec)
         for _ in range(10):
             assert torch.equal(P, ax.aht(A, H, prec)) and torch.equal(Q, ax.wta(A, W, prec))
 
 
-@pytest.mark.parametrize("m,n,k", [(700, 512, 20), (611, 503, 64)])
-def test_run_equals_the_form_with_copies(ax, m, n, k):
-    """A run of up to 12 TF32 iterations reads A directly, a longer one keeps
-    rounded copies: the same factors and residuals to the bit."""
+def test_unaligned_base(ax):
+    """A starts 4 bytes past a 16-byte boundary, rows of 16-byte multiples."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(6)
+    m, n, k = 515, 260, 24
+    A = torch.rand(m * n + 1, generator=g, device="cuda")[1:].view(m, n)
+    H, W = torch.rand((k, n), generator=g, device="cuda"), torch.rand((m, k), generator=g, device="cuda")
+    for prec in ("tf32", "bf16"):
+        Ar = rounded(A.clone(), prec)
+        check(ax.aht(A, H, prec), A, H.T, Ar, n, prec)
+        check(ax.wta(A, W, prec).T, A.T, W, Ar.T, m, prec)
+
+
+@pytest.mark.parametrize("m,n,k,last", [(700, 512, 20, 12), (611, 503, 64, 3)])
+def test_run_equals_the_form_with_copies(ax, m, n, k, last):
+    """A run of up to 12 TF32 iterations (3 when A's rows are not 16-byte aligned)
+    reads A directly, a longer one keeps rounded copies: the same factors and
+    residuals to the bit."""
     from paper_1609_09154_gb300 import synth
 
     A, _, _ = synth.dense_lowrank_torch(m, n, k, 3, "cuda")
     W0, H0 = synth.init_factors_torch(m, n, k, 3, "cuda")
-    W, H, rel, _ = ax.run(A, k, "hals", 12, W0, H0, prec="tf32")
-    W1, H1, rel1, _ = ax.run(A, k, "hals", 13, W0, H0, prec="tf32")
-    np.testing.assert_array_equal(rel, rel1[:12])
+    W, H, rel, _ = ax.run(A, k, "hals", last, W0, H0, prec="tf32")
+    W1, H1, rel1, _ = ax.run(A, k, "hals", last + 1, W0, H0, prec="tf32")
+    np.testing.assert_array_equal(rel, rel1[:last])
     W2, H2, rel2, _ = ax.run(A, k, "hals", 1, W, H, prec="tf32")
-    assert torch.equal(W2, W1) and torch.equal(H2, H1) and rel2[0] == rel1[12]
+    assert torch.equal(W2, W1) and torch.equal(H2, H1) and rel2[0] == rel1[last]
     # BF16: one iteration reads A directly, more keep copies
     _, _, r1, _ = ax.run(A, k, "mu", 1, W0, H0, prec="bf16")
     _, _, r2, _ = ax.run(A, k, "mu", 2, W0, H0, prec="bf16")
