@@ -777,30 +777,33 @@ __global__ void __launch_bounds__(256, AUNMF_SIMT_MINB)
 
 // ---------------------------------------------------------------- TMA-fed form
 // k_gemm_simt_tma: the same product and the same compensated summation as
-// k_gemm_simt, for N > 32 (column tiles of 64) when A's rows are 16-byte
-// aligned.  A's tiles and the fixed factor's 16 x 64 tiles arrive by TMA in
-// a seven-stage shared-memory ring with mbarriers (full: one arrival + the
-// copies' bytes; empty: all 256 threads).  The factor is read from a copy
-// whose rows are padded to a multiple of 4 floats (TMA needs 16-byte row
-// strides; N = 50 floats is not one); staging its tiles with 4-byte
-// asynchronous copies instead measured 3x slower than the whole product
-// should take (11.5 ms for the copies alone at 96,000 x 64,000).  Eight warps compute, 8 x 8 outputs per thread (256 x 64 per
-// block, one block per SM), four 16-byte fragment loads per 64 FFMAs, with
-// the running sums in registers (two warps per SM sub-partition may hold
-// up to 255 registers each; a ninth, producer-only warp would cap them at
-// 168).  Thread 0 also fills the ring: steps 0 .. 6 first, then at the top
-// of step s it waits until every thread has released the stage read at
-// step s - 1 (warp 0 trails the others, so the wait is short) and issues
-// the two copies of step s + 6 into it.
+// k_gemm_simt, when A's rows are 16-byte aligned; and, in its short form, for
+// few output tiles whatever the alignment.  FP32 issue bounds it (k = 50,
+// W^T A at 32,000 x 24,000: 46 TFLOP/s of useful FMAs against the 73 a loop
+// of packed FMAs reaches).  A's tiles and the fixed factor's 16 x BN tiles
+// arrive by TMA in a seven-stage shared-memory ring with mbarriers (full:
+// one arrival + the copies' bytes; empty: all 256 threads).  The factor is
+// read from a copy whose rows are padded to a multiple of 4 floats (TMA needs
+// 16-byte row strides; N = 50 floats is not one), or in place where they are;
+// staging its tiles with 4-byte asynchronous copies instead measured 3x
+// slower than the whole product should take (11.5 ms for the copies alone at
+// 96,000 x 64,000).  Eight warps compute, 8 x BN / 8 outputs per thread (256
+// x BN per block, one block per SM), four 16-byte fragment loads per 32
+// two-wide FMAs, with the running sums in registers (two warps per SM
+// sub-partition may hold up to 255 registers each; a ninth, producer-only
+// warp would cap them at 168).  Thread 0 also fills the ring: steps 0 .. 6
+// first, then at the top of step s it waits until every thread has released
+// the stage read at step s - 1 (warp 0 trails the others, so the wait is
+// short) and issues the two copies of step s + 6 into it.
 //   Thread (ty, tx), ty = 0..31, tx = 0..7 (a warp: 4 ty x 8 tx): columns
-//   tx*4 + {0..3} and 32 + tx*4 + {0..3}; rows ty + 32 i (AK) or
-//   ty*4 + {0..3} and 128 + ty*4 + {0..3} (!AK).
+//   simt_col(tx, j); rows ty + 32 i (AK) or ty*4 + {0..3} and 128 + ty*4 +
+//   {0..3} (!AK).
 // AK (A K-contiguous): the tile is 256 rows of 16 K (64 bytes), copied with
 // the 64-byte swizzle (16-byte chunk c of row r lands at chunk
 // c ^ ((r >> 1) & 3)), so the four rows a warp reads at once (ty .. ty+3)
 // sit in four different bank groups.  !AK: 16 K-rows of 256 (one kilobyte):
-// a warp's four row fragments are consecutive.  Either way a warp's 16-byte
-// loads of the factor tile read 8 consecutive chunks, with no bank conflict.
+// a warp's four row fragments are consecutive.  Either way a warp's loads of
+// the factor tile read consecutive words, with no bank conflict.
 // Slab sums are folded every 128 K into the running sums with Kahan's
 // corrections, which sit in shared memory (one row per thread).  Every wait
 // is bounded; on expiry the kernel raises *err, writes nothing and returns
@@ -827,8 +830,8 @@ struct SimtTile {
 // Column j (0 .. TN - 1) of thread column tx within the tile.
 template <int TN>
 __device__ __forceinline__ int simt_col(int tx, int j) {
-  if constexpr (TN == 8)
-    return j < 4 ? tx * 4 + j : 32 + tx * 4 + j - 4;
+  if constexpr (TN >= 4)  // 32 columns by fours, then 32 by fours, 16 by twos, 8 by ones
+    return j < 4 ? tx * 4 + j : TN == 8 ? 32 + tx * 4 + j - 4 : j < 6 ? 32 + tx * 2 + j - 4 : 48 + tx;
   else
     return tx * TN + j;
 }
@@ -949,7 +952,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   // slab sums as packed pairs for the two-wide FMA (the same FMAs in half the
   // issue slots): output (i, j) is half i & 1 of acc[i / 2][j] (!AK: a pair of
   // rows arrives as one aligned 8-byte half of a fragment) or half j & 1 of
-  // acc[i][j / 2] (AK)
+  // acc[i][j / 2] (AK: TN is even)
   f32x2 acc[NE / 2];
   float hi[NE];
 #pragma unroll
@@ -989,21 +992,27 @@ __global__ void __launch_bounds__(kTThreads, 1)
 #pragma unroll
     for (int e = 0; e < NE / 2; ++e) acc[e] = 0;
   };
-  // the thread's TN columns of factor row br
+  // the thread's TN columns (simt_col) of factor row br
   auto load_b = [&](const float *br, float (&b)[TN]) {
     if constexpr (TN == 2) {
-      const float2 v = *reinterpret_cast<const float2 *>(br);
+      const float2 v = *reinterpret_cast<const float2 *>(br + tx * 2);
       b[0] = v.x;
       b[1] = v.y;
     } else {
 #pragma unroll
       for (int q = 0; q < TN / 4; ++q) {
-        const float4 v = *reinterpret_cast<const float4 *>(br + 32 * q);
+        const float4 v = *reinterpret_cast<const float4 *>(br + 32 * q + tx * 4);
         b[4 * q] = v.x;
         b[4 * q + 1] = v.y;
         b[4 * q + 2] = v.z;
         b[4 * q + 3] = v.w;
       }
+      if constexpr (TN == 6 || TN == 7) {
+        const float2 v = *reinterpret_cast<const float2 *>(br + 32 + tx * 2);
+        b[4] = v.x;
+        b[5] = v.y;
+      }
+      if constexpr (TN == 7) b[6] = br[48 + tx];
     }
   };
   // AK: rows ty + 32 i share their swizzle (r >> 1) & 3 (32 i leaves those bits alone)
@@ -1040,7 +1049,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
       break;
     }
     const float *a = sA + (size_t)st * BM * kTBK;
-    const float *b = sB + (size_t)st * kTBK * BN + (TN == 2 ? tx * 2 : tx * 4);
+    const float *b = sB + (size_t)st * kTBK * BN;
     if constexpr (AK) {  // a: [BM rows][16 K], 64-byte swizzle
 #pragma unroll
       for (int kq = 0; kq < kTBK / 4; ++kq) {
@@ -1278,6 +1287,13 @@ cudaError_t launch_simt_tma_n(int BN, const CUtensorMap &mapA, const CUtensorMap
     return launch_simt_tma<AK, RT, 16, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
   if (BN == 32)
     return launch_simt_tma<AK, RT, 32, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+  if constexpr (RT == 8) {
+    if (BN == 48)
+      return launch_simt_tma<AK, RT, 48, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+    if constexpr (!AK)
+      if (BN == 56)
+        return launch_simt_tma<AK, RT, 56, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+  }
   return launch_simt_tma<AK, RT, 64, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
 }
 
@@ -1329,13 +1345,22 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
     const bool direct = ldp == N && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
     const unsigned gx = (unsigned)((M + 255) / 256);
     const int S = simt_splits((int64_t)gx * gy, K, 1);
+    // Column tiles of 48 or 56 where these take no more of them: padding columns
+    // cost FMAs like any other.  W^T A at k = 50 (56 for 64), 32,000 x 24,000:
+    // 1775 -> 1657 us.  AK keeps 64 for 56: its row fragments hold four K of one
+    // row, so the odd column would be packed from two rows with moves (A H^T and
+    // W^T A at k = 100, 20,000 x 10,000, both with 56: 2983 us, so 2753).
+    const int bn = BN < 64                           ? BN
+                   : (N + 47) / 48 == (int)gy        ? 48
+                   : !AK && (N + 55) / 56 == (int)gy ? 56
+                                                     : 64;
     float *Bp = parts + (((S > 4 ? S : 4) * M * (int64_t)N + 63) & ~63LL);
     const float *Bs = direct ? B : Bp;
-    if (simt_factor_map(&mapB, Bs, K, N, ldp, BN)) {
+    if (simt_factor_map(&mapB, Bs, K, N, ldp, bn)) {
       const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
       cudaError_t e = direct ? cudaSuccess : launch_copy2d(B, N, Bp, ldp, K, N, s);
       if (e == cudaSuccess)
-        e = launch_simt_tma_n<AK, 8, true>(BN, mapA, mapB, A, lda, B, M, K, N, S > 1 ? parts : C,
+        e = launch_simt_tma_n<AK, 8, true>(bn, mapA, mapB, A, lda, B, M, K, N, S > 1 ? parts : C,
                                            kchunk, S, 0, err, s);
       if (e != cudaSuccess || S == 1) return e;
       return sum_parts(parts, S, M * (int64_t)N, C, s);
