@@ -175,6 +175,7 @@ struct RunCtx {
   void *Hk, *Wt;
   int64_t ldh, ldw;
   bool direct;       // products round A's tiles themselves (k_direct.cu): no Ax, At
+  bool even;         // FP32 products: equal runs of slabs instead of whole K splits
   bool norm_in_wta;  // direct: the next W^T A product also forms n2a
   float *parts;
   float *tcacc;  // k > 64: the products' per-CTA partial sums (null: added into parts)
@@ -256,7 +257,8 @@ cudaError_t product_aht(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   if (c.prec == AUNMF_FP32) {
     PhaseTimer t(c, s, kPhAht);
-    return launch_aht_simt(A->dense, A->m, A->n, A->lda, c.Ht, c.k, c.PW, c.parts, c.err, s);
+    return launch_aht_simt(A->dense, A->m, A->n, A->lda, c.Ht, c.k, c.PW, c.parts, c.even, c.err,
+                           s);
   }
   const bool bf = c.prec == AUNMF_BF16;
   const bool split = use_split(c.k);
@@ -294,7 +296,8 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   }
   if (c.prec == AUNMF_FP32) {
     PhaseTimer t(c, s, kPhWta);
-    return launch_wta_simt(A->dense, A->m, A->n, A->lda, c.W, c.k, c.PHt, c.parts, c.err, s);
+    return launch_wta_simt(A->dense, A->m, A->n, A->lda, c.W, c.k, c.PHt, c.parts, c.even, c.err,
+                           s);
   }
   const bool bf = c.prec == AUNMF_BF16;
   const bool split = use_split(c.k);
@@ -737,7 +740,7 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
     int prc = prepare_tc(h, c, kPrepAht | kPrepWta | kPrepNorm, s);
     if (prc != AUNMF_OK) return prc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(m > n ? m : n, k));
+    ENS(h, h->parts, simt_parts_bytes(m, n, k, false));
     c.parts = P<float>(h->parts);
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
@@ -946,8 +949,9 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
     int rc = prepare_tc(h, c, kPrepAht, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(A->m > A->n ? A->m : A->n, k));
+    ENS(h, h->parts, simt_parts_bytes(A->m, A->n, k, true));
     c.parts = P<float>(h->parts);
+    c.even = true;
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), h->stream));
@@ -980,8 +984,9 @@ int aunmf_wta(aunmf_handle *h, const aunmf_matrix *A, const float *W, int k, int
     int rc = prepare_tc(h, c, kPrepWta, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(A->m > n ? A->m : n, k));
+    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, true));
     c.parts = P<float>(h->parts);
+    c.even = true;
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), h->stream));
@@ -1131,9 +1136,9 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
   CK(h, launch_transpose(H, k, n, Ht, s));
   if (A->dense) {
     CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
-    ENS(h, h->parts, simt_parts_bytes(A->m > n ? A->m : n, k));
-    CK(h, launch_wta_simt(A->dense, m, n, A->lda, W, k, PHt, P<float>(h->parts), P<int>(h->err),
-                          s));
+    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, false));
+    CK(h, launch_wta_simt(A->dense, m, n, A->lda, W, k, PHt, P<float>(h->parts), false,
+                          P<int>(h->err), s));
   } else {
     CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     RunCtx c{};
@@ -1202,8 +1207,9 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
   } else if (A->dense) {
     if (what & kPrepNorm)
       CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
-    ENS(h, h->parts, simt_parts_bytes(m > n ? m : n, k));
+    ENS(h, h->parts, simt_parts_bytes(m, n, k, true));
     c.parts = P<float>(h->parts);
+    c.even = true;
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));

@@ -9,6 +9,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.cuh"
@@ -827,6 +828,23 @@ struct SimtTile {
   }
 };
 
+// The runs of slabs of a launch of `blocks` blocks (at most one per slab):
+// slab u of the product is slab u % nsl of tile u / nsl, and block b has slabs
+// first(b) .. first(b + 1) - 1.  A split into whole tiles and whole K splits
+// left part of the last wave idle (125 row tiles on 152 SMs: 18 %).
+struct SimtRuns {
+  int64_t nsl, per, rem;  // slabs per tile; slabs per block, one more in the first rem
+  __host__ __device__ int64_t first(int64_t b) const { return b * per + (b < rem ? b : rem); }
+  __host__ __device__ int64_t owner(int64_t u) const {
+    return u < rem * (per + 1) ? u / (per + 1) : rem + (u - rem * (per + 1)) / per;
+  }
+};
+__host__ __device__ inline SimtRuns simt_runs(int64_t M, int64_t K, int gy, int64_t blocks) {
+  const int64_t nsl = (K + kTBK * kTSlabSteps - 1) / (kTBK * kTSlabSteps);
+  const int64_t u = (M + 255) / 256 * gy * nsl;
+  return {nsl, u / blocks, u % blocks};
+}
+
 // Column j (0 .. TN - 1) of thread column tx within the tile.
 template <int TN>
 __device__ __forceinline__ int simt_col(int tx, int j) {
@@ -841,8 +859,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
     k_gemm_simt_tma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const float *__restrict__ A, int64_t lda, const float *__restrict__ B,
                     int64_t M, int64_t K, int N, float *__restrict__ C,
-                    int ldc, int64_t kchunk, int clus, int group, int *err, long long limit,
-                    int inject) {
+                    int ldc, int64_t kchunk, int clus, int group, float *__restrict__ parts,
+                    int *err, long long limit, int inject) {
   // The short form (RT = 4, few tiles) stages the factor's tile with 4-byte
   // asynchronous copies straight from B (K x N, contiguous): it spares the
   // launch that pads B's rows to 16 bytes for TMA (mapB is not used).  VEC
@@ -855,6 +873,12 @@ __global__ void __launch_bounds__(kTThreads, 1)
   // compensation within each `group` slabs, the groups' sums added plainly --
   // the additions of an unclustered pass over K split every `group` slabs, so
   // both give the same bits.  clus == 0: split z writes its partial at C + z M ldc.
+  // parts (RT = 8): the grid is one block per SM and the tiles' slabs, tile
+  // after tile, are cut into equal runs, one per block (SimtRuns).  A block
+  // writes a tile it has all of to C, another one's part to its first (the
+  // run's first tile) or second (its last) slot of parts, for k_simt_join.
+  // parts and group > 0: every slab's sums go to parts, slab after slab, for
+  // k_simt_fold, which adds them as a cluster does.
   // inject (test hook): thread 0 never arrives on the first stage's barrier,
   // so every thread's bounded wait runs out
   using namespace aunmf::ptx;
@@ -875,7 +899,22 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int64_t m0 = (int64_t)blockIdx.x * BM;
   const int n0 = blockIdx.y * BN;
   const int64_t kz0 = (int64_t)blockIdx.z * kchunk, kz1 = min(K, kz0 + kchunk);
-  const int nsteps = kz1 > kz0 ? (int)((kz1 - kz0 + kTBK - 1) / kTBK) : 0;
+  int nsteps = kz1 > kz0 ? (int)((kz1 - kz0 + kTBK - 1) / kTBK) : 0;
+  // RT = 8: the tile (row tile * gy + column tile) and the K step within it that
+  // the copies and the sums have reached; a tile ends after nst steps
+  const int nst = (int)((K + kTBK - 1) / kTBK);
+  const int gy = RT == 8 && parts ? (N + BN - 1) / BN : gridDim.y;
+  int64_t tile0 = (int64_t)blockIdx.x * gy + blockIdx.y;
+  int step0 = (int)(kz0 / kTBK);
+  int64_t u0 = 0;
+  if (RT == 8 && parts) {
+    const SimtRuns r = simt_runs(M, K, gy, gridDim.x);
+    const int64_t u1 = r.first(blockIdx.x + 1);
+    u0 = r.first(blockIdx.x);
+    tile0 = u0 / r.nsl;
+    step0 = (int)(u0 % r.nsl) * kTSlabSteps;
+    nsteps = (int)((u1 / r.nsl - tile0) * nst + u1 % r.nsl * kTSlabSteps - step0);
+  }
   const bool producer = tid < 32;
   if (tid == 0) {
     for (int st = 0; st < kTStages; ++st) {
@@ -890,9 +929,22 @@ __global__ void __launch_bounds__(kTThreads, 1)
   // thread 0: fill stage st with step s
   const uint64_t pol_a = policy_evict_first(), pol_b = policy_evict_last();  // A streams once
   int issued = 0;
+  int64_t ft = tile0;
+  int fk = step0;
   auto fill = [&](int s) {
     const int st = s % kTStages;
-    const int k0 = (int)(kz0 + (int64_t)s * kTBK);
+    int k0 = (int)(kz0 + (int64_t)s * kTBK);
+    int64_t fm = m0;
+    int fn = n0;
+    if constexpr (RT == 8) {
+      k0 = fk * kTBK;
+      fm = ft / gy * BM;
+      fn = (int)(ft % gy) * BN;
+      if (++fk == nst) {
+        fk = 0;
+        ++ft;
+      }
+    }
     const uint32_t bytes = (uint32_t)(!VEC ? 0 : BCP ? T::kA : T::kA + T::kB);
     if (!VEC) {
       if (!(inject && s == 0)) mbar_arrive(&full[st]);
@@ -904,14 +956,14 @@ __global__ void __launch_bounds__(kTThreads, 1)
       mbar_expect_tx(&full[st], bytes);
     // x coordinates (k0 for AK and the factor, m0 otherwise) are multiples
     // of 16 floats; the checked build tests it and skips bad copies
-    if (!AUNMF_BOUND(k0 >= 0 && (k0 & 3) == 0 && (m0 & 3) == 0 && (n0 & 3) == 0,
+    if (!AUNMF_BOUND(k0 >= 0 && (k0 & 3) == 0 && (fm & 3) == 0 && (fn & 3) == 0,
                      AUNMF_CHECK_TMA_COORD))
       return;
     if (AK)
-      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], k0, (int)m0, pol_a);
+      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], k0, (int)fm, pol_a);
     else
-      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], (int)m0, k0, pol_a);
-    if (!BCP) tma_load_2d(sB + (size_t)st * kTBK * BN, &mapB, &full[st], n0, k0, pol_b);
+      tma_load_2d(sA + (size_t)st * BM * kTBK, &mapA, &full[st], (int)fm, k0, pol_a);
+    if (!BCP) tma_load_2d(sB + (size_t)st * kTBK * BN, &mapB, &full[st], fn, k0, pol_b);
     ++issued;
   };
   auto fill_b = [&](int s) {  // every thread's share of the factor's tile
@@ -981,17 +1033,18 @@ __global__ void __launch_bounds__(kTThreads, 1)
   };
   // row i (0 .. RT - 1) of the thread within the tile
   auto row_of = [&](int i) { return AK ? ty + 32 * i : (i < 4 ? ty * 4 + i : 128 + ty * 4 + i - 4); };
-  auto keep = [&](int sl) {  // the slab's sums into shared memory; acc = 0
+  auto keep_at = [&](float *p) {  // the slab's sums into a tile at p; acc = 0
 #pragma unroll
     for (int e = 0; e < NE; ++e) {
       const int i = e / TN, j = e % TN;
       const f32x2 pr = AK ? acc[i * (TN / 2) + j / 2] : acc[(i / 2) * TN + j];
-      corr[(sl * BM + row_of(i)) * BN + simt_col<TN>(tx, j)] =
+      p[row_of(i) * BN + simt_col<TN>(tx, j)] =
           (AK ? (j & 1) : (i & 1)) ? hi32(pr) : lo32(pr);
     }
 #pragma unroll
     for (int e = 0; e < NE / 2; ++e) acc[e] = 0;
   };
+  auto keep = [&](int sl) { keep_at(corr + sl * BM * BN); };
   // the thread's TN columns (simt_col) of factor row br
   auto load_b = [&](const float *br, float (&b)[TN]) {
     if constexpr (TN == 2) {
@@ -1019,7 +1072,9 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int sw = (ty >> 1) & 3;
 
   bool ok = true;
-  int slab = 0;
+  int slab = 0, kept = 0, ck = step0;
+  bool from0 = step0 == 0;  // the sums began with the tile's first K step
+  int64_t ct = tile0;
   for (int s = 0; s < nsteps; ++s) {
     const int st = s % kTStages;
     if (BCP && s >= 1 && s - 1 + kTStages < nsteps) {
@@ -1095,12 +1150,48 @@ __global__ void __launch_bounds__(kTThreads, 1)
       }
     }
     mbar_arrive(&empty[st]);
-    if (++slab == kTSlabSteps || s + 1 == nsteps) {
-      if (clus > 0)
+    const bool last = s + 1 == nsteps || (RT == 8 && ck + 1 == nst);
+    if (++slab == kTSlabSteps || last) {
+      if (clus > 0) {
         keep(s / kTSlabSteps);
-      else
+      } else if (RT == 8 && group > 0) {
+        keep_at(parts + (u0 + kept++) * BM * BN);
+      } else {
         fold();
+      }
       slab = 0;
+    }
+    if constexpr (RT == 8) {
+      ++ck;
+      if (last && group > 0) {
+        ck = 0;
+      } else if (parts && last) {
+        const int64_t tm = ct / gy * BM;
+        const int tn = (int)(ct % gy) * BN;
+        float *slot = parts + (2 * (int64_t)blockIdx.x + (ct != tile0)) * 2 * BM * BN;
+        const bool whole = from0 && ck == nst;
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          const int64_t gm = tm + row_of(i);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) {
+            const int e = i * TN + j, c = simt_col<TN>(tx, j);
+            const float v = hi[e] - kc[e];
+            if (!whole) {
+              slot[row_of(i) * BN + c] = v;
+              slot[(BM + row_of(i)) * BN + c] = (hi[e] - v) - kc[e];  // what v rounded off
+            } else if (gm < M && tn + c < N) {
+              C[gm * ldc + tn + c] = v;
+            }
+            hi[e] = 0.f;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < NE; e += 4) *reinterpret_cast<float4 *>(kc + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+        ck = 0;
+        from0 = true;
+        ++ct;
+      }
     }
   }
   if (BCP) cp_async_wait_all();
@@ -1154,7 +1245,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     cluster_sync();  // no block's shared memory goes away while a peer reads it
     return;
   }
-  if (!ok) return;
+  if (!ok || (RT == 8 && parts)) return;
   C += (int64_t)blockIdx.z * M * ldc;
 #pragma unroll
   for (int i = 0; i < RT; ++i) {
@@ -1225,44 +1316,101 @@ int simt_wave_splits(int64_t tiles, int64_t K, int64_t slots) {
   return best;
 }
 
-// The same, and for few tiles as many splits (of at least a slab) as fill the
-// slots once, up to 16.
-int simt_splits(int64_t tiles, int64_t K, int per_sm) {
-  const int64_t slots = (int64_t)per_sm * simt_sms();
-  if (tiles * 4 > slots) return simt_wave_splits(tiles, K, slots);
-  int64_t S = slots / tiles;
-  if (S > 16) S = 16;
-  if (S > (K + 127) / 128) S = (K + 127) / 128;
-  return S > 1 ? (int)S : 1;
-}
-
 __global__ void k_sum_parts(const float *__restrict__ parts, int S, int64_t len,
                             float *__restrict__ C) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len;
        e += (int64_t)gridDim.x * blockDim.x) {
-    float s = 0.f, r = 0.f;  // r: the additions' errors, kept for many parts
-    for (int z = 0; z < S; ++z) {
-      const float v = parts[z * len + e], t = __fadd_rn(s, v), d = __fsub_rn(t, s);
-      if (S > 4) r += __fadd_rn(__fsub_rn(s, __fsub_rn(t, d)), __fsub_rn(v, d));
-      s = t;
-    }
-    C[e] = s + r;
+    float s = 0.f;
+    for (int z = 0; z < S; ++z) s += parts[z * len + e];
+    C[e] = s;
   }
 }
 
+// The tiles that runs of k_gemm_simt_tma cut: block x takes the tile that the
+// boundary of runs x and x + 1 cuts, unless an earlier boundary cuts it too,
+// and adds its parts (a sum and what it rounded off) in K order, with the
+// additions' errors carried along.
+template <int BN>
+__global__ void k_simt_join(const float *__restrict__ parts, int64_t M, int64_t K, int N,
+                            float *__restrict__ C, int ldc) {
+  constexpr int BM = 256;
+  const int gy = (N + BN - 1) / BN;
+  const SimtRuns r = simt_runs(M, K, gy, gridDim.x + 1);
+  const int64_t cut = r.first(blockIdx.x + 1), t = cut / r.nsl;
+  const int64_t b0 = r.owner(t * r.nsl), b1 = r.owner((t + 1) * r.nsl - 1);
+  if (cut == t * r.nsl || b0 != blockIdx.x) return;
+  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < BM * BN; e += gridDim.y * blockDim.x) {
+    const int64_t gm = t / gy * BM + e / BN;
+    const int gn = (int)(t % gy) * BN + e % BN;
+    if (gm >= M || gn >= N) continue;
+    // tile t is the last of run b0 (its first slot if also the first) and the
+    // first of the others
+    const float *p = parts + (2 * b0 + (r.first(b0) / r.nsl != t)) * 2 * BM * BN + e;
+    float s = p[0], c = p[BM * BN];
+#pragma unroll 4
+    for (int64_t b = b0 + 1; b <= b1; ++b) {
+      const float *q = parts + 4 * b * BM * BN + e;
+      const float v = q[0], u = __fadd_rn(s, v), d = __fsub_rn(u, s);
+      c += __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(u, d)), __fsub_rn(v, d)), q[BM * BN]);
+      s = u;
+    }
+    C[gm * ldc + gn] = s + c;
+  }
+}
+
+// The slab sums that k_gemm_simt_tma left for every tile, folded in K order:
+// Kahan's compensation within each `group` slabs (a thread each, at most four),
+// the groups' sums added plainly.
+template <int BN>
+__global__ void k_simt_fold(const float *__restrict__ parts, int64_t M, int64_t K, int N, int group,
+                            float *__restrict__ C, int ldc) {
+  constexpr int BM = 256;
+  __shared__ float part[4][64];
+  const int gy = (N + BN - 1) / BN;
+  const int64_t nsl = simt_runs(M, K, gy, 1).nsl;
+  const int64_t x = (int64_t)blockIdx.x * 64 + threadIdx.x, t = x / (BM * BN);
+  const int e = (int)(x % (BM * BN));
+  const int64_t gm = t / gy * BM + e / BN, a = (int64_t)threadIdx.y * group;
+  const int gn = (int)(t % gy) * BN + e % BN;
+  const bool in = gm < M && gn < N;
+  const int64_t len = in ? min((int64_t)group, nsl - a) : 0;
+  const float *p = parts + (t * nsl + a) * BM * BN + e;
+  float h = 0.f, c = 0.f;
+  for (int64_t g0 = 0; g0 < len; g0 += 16) {  // sixteen loads in flight
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = p[min(g0 + u, len - 1) * BM * BN];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      if (g0 + u >= len) break;
+      const float y = v[u] - c, w = h + y;
+      c = (w - h) - y;
+      h = w;
+    }
+  }
+  part[threadIdx.y][threadIdx.x] = h - c;
+  __syncthreads();
+  if (!in || threadIdx.y) return;
+  float out = h - c;
+  for (int z = 1; z < (int)blockDim.y; ++z) out += part[z][threadIdx.x];
+  C[gm * ldc + gn] = out;
+}
+
 // One launch of a k_gemm_simt_tma form: grid (gx, gy, S), a cluster per tile
-// when group > 0 (see the kernel).
+// when group > 0, S blocks with equal runs when parts is given (see the
+// kernel), and then the launch that joins the cut tiles or folds the slabs.
 template <bool AK, int RT, int BN, bool VEC>
 cudaError_t launch_simt_tma(const CUtensorMap &mapA, const CUtensorMap &mapB, const float *A,
                             int64_t lda, const float *B, int64_t M, int64_t K, int N, float *C, int ldc, int64_t kchunk, int S,
-                            int group, int *err, cudaStream_t s) {
+                            int group, float *parts, int *err, cudaStream_t s) {
   using T = SimtTile<RT, BN>;
   auto kern = k_gemm_simt_tma<AK, RT, BN, VEC>;
-  const bool clus = group > 0;
+  const bool clus = group > 0 && !parts;
   const size_t smem = T::smem(clus ? (int)(kchunk / (kTBK * kTSlabSteps)) : 0);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((M + T::BM - 1) / T::BM), (unsigned)((N + BN - 1) / BN), (unsigned)S);
+  const unsigned gx = (unsigned)((M + T::BM - 1) / T::BM), gy = (unsigned)((N + BN - 1) / BN);
+  cfg.gridDim = parts ? dim3((unsigned)S) : dim3(gx, gy, (unsigned)S);
   cfg.blockDim = dim3(kTThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -1274,27 +1422,39 @@ cudaError_t launch_simt_tma(const CUtensorMap &mapA, const CUtensorMap &mapB, co
   cfg.attrs = at;
   cfg.numAttrs = clus ? 1 : 0;
   g_launches += 1;
-  return cudaLaunchKernelEx(&cfg, kern, mapA, mapB, A, lda, B, M, K, N, C, ldc, kchunk, clus ? S : 0, group, err,
-                            fault::wait_cycles(), fault::site() == AUNMF_INJECT_SIMT_WAIT ? 1 : 0);
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, kern, mapA, mapB, A, lda, B, M, K, N, C, ldc, kchunk, clus ? S : 0, group, parts, err,
+                         fault::wait_cycles(), fault::site() == AUNMF_INJECT_SIMT_WAIT ? 1 : 0);
+  if (e != cudaSuccess || !parts) return e;
+  if (group > 0) {
+    const int64_t nsl = simt_runs(M, K, gy, 1).nsl;
+    k_simt_fold<BN><<<gx * gy * (T::BM * BN / 64), dim3(64, (unsigned)((nsl + group - 1) / group)), 0, s>>>(
+        parts, M, K, N, group, C, ldc);
+  } else {
+    if ((int64_t)gx * gy % S == 0) return e;  // no tile is cut
+    k_simt_join<BN><<<dim3((unsigned)S - 1, 16), 256, 0, s>>>(parts, M, K, N, C, ldc);
+  }
+  g_launches += 1;
+  return cudaGetLastError();
 }
 
 template <bool AK, int RT, bool VEC>
 cudaError_t launch_simt_tma_n(int BN, const CUtensorMap &mapA, const CUtensorMap &mapB,
                               const float *A, int64_t lda, const float *B, int64_t M, int64_t K,
-                              int N, float *C, int64_t kchunk, int S, int group, int *err,
-                              cudaStream_t s) {
+                              int N, float *C, int64_t kchunk, int S, int group, float *parts,
+                              int *err, cudaStream_t s) {
   if (BN == 16)
-    return launch_simt_tma<AK, RT, 16, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+    return launch_simt_tma<AK, RT, 16, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, parts, err, s);
   if (BN == 32)
-    return launch_simt_tma<AK, RT, 32, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+    return launch_simt_tma<AK, RT, 32, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, parts, err, s);
   if constexpr (RT == 8) {
     if (BN == 48)
-      return launch_simt_tma<AK, RT, 48, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+      return launch_simt_tma<AK, RT, 48, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, parts, err, s);
     if constexpr (!AK)
       if (BN == 56)
-        return launch_simt_tma<AK, RT, 56, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+        return launch_simt_tma<AK, RT, 56, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, parts, err, s);
   }
-  return launch_simt_tma<AK, RT, 64, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, err, s);
+  return launch_simt_tma<AK, RT, 64, VEC>(mapA, mapB, A, lda, B, M, K, N, C, N, kchunk, S, group, parts, err, s);
 }
 
 cudaError_t sum_parts(const float *parts, int S, int64_t len, float *C, cudaStream_t s) {
@@ -1305,9 +1465,28 @@ cudaError_t sum_parts(const float *parts, int S, int64_t len, float *C, cudaStre
   return cudaGetLastError();
 }
 
+// Whether a product with whole K splits keeps its slab sums in memory: few
+// tiles, and at most a quarter gigabyte of them.
+bool simt_keep_slabs(int64_t M, int64_t K, int bn, int gy) {
+  const int64_t tiles = (M + 255) / 256 * gy;
+  return tiles * 4 <= simt_sms() && tiles * ((K + 127) / 128) * 256 * bn <= (1LL << 26);
+}
+
+// Floats of `parts` that the product's parts take before the factor's copy.
+int64_t simt_parts_floats(int64_t M, int64_t K, int N, bool even) {
+  const int bn = N <= 16 ? 16 : N <= 32 ? 32 : 64;
+  const int gy = (N + bn - 1) / bn;
+  const int64_t slabs = (M + 255) / 256 * gy * ((K + 127) / 128);
+  const int64_t splits = 4 * M * N;
+  const int64_t other = even                               ? 4 * std::min<int64_t>(slabs, simt_sms()) * 256 * bn
+                        : simt_keep_slabs(M, K, bn, gy) ? slabs * 256 * bn
+                                                          : 0;
+  return (std::max(other, splits) + 63) & ~63LL;
+}
+
 template <bool AK>
 cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const float *B, int N,
-                      float *C, float *parts, int *err, cudaStream_t s) {
+                      float *C, float *parts, bool even, int *err, cudaStream_t s) {
   constexpr int BM = AUNMF_SIMT_BM, BK = 16, SLAB = 128;
   const int vec = (reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 4 == 0) ? 1 : 0;
   const int BN = N <= 16 ? 16 : (N <= 32 ? 32 : 64);
@@ -1316,6 +1495,12 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
   // (parts holds the split partials, then the factor's padded copy)
   CUtensorMap mapA, mapB;
   const int sms = simt_sms();
+  // K splits: of 256-row tiles on the SMs where N > 32, else of BM-row tiles,
+  // two to an SM.  Each form sums the same splits, so a call's bits do not
+  // depend on which one it takes; `even` alone cuts K elsewhere.
+  const int S0 = !parts           ? 1
+                 : vec && N > 32 ? simt_wave_splits((M + 255) / 256 * gy, K, sms)
+                                 : simt_wave_splits((M + BM - 1) / BM * gy, K, 2 * (int64_t)sms);
   const int64_t tiles4 = (M + 127) / 128 * gy;
   if (err && parts && M < (1LL << 31) && K < (1LL << 31) && tiles4 * 2 <= sms) {
     // few output tiles: 128-row tiles, K cut over a cluster of up to 8 blocks
@@ -1327,16 +1512,14 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
     const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
     S = (K + kchunk - 1) / kchunk;
     if (kchunk / SLAB * 128 * BN * 4 <= 128 * 1024) {
-      // slabs per K group: where the unclustered forms would split K
-      const int bm = vec && N > 32 ? 256 : BM;
-      const int S0 = simt_wave_splits((M + bm - 1) / bm * gy, K, (vec && N > 32 ? 1 : 2) * (int64_t)sms);
+      // slabs per K group
       const int group = (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB);
       if (vec && simt_map(&mapA, A, lda, M, K, AK, 128))
         return launch_simt_tma_n<AK, 4, true>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
-                                              group, err, s);
+                                              group, nullptr, err, s);
       memset(&mapA, 0, sizeof(mapA));
       return launch_simt_tma_n<AK, 4, false>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
-                                             group, err, s);
+                                             group, nullptr, err, s);
     }
   }
   if (vec && err && parts && M < (1LL << 31) && K < (1LL << 31) &&
@@ -1344,7 +1527,21 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
     const int ldp = (N + 3) & ~3;
     const bool direct = ldp == N && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
     const unsigned gx = (unsigned)((M + 255) / 256);
-    const int S = simt_splits((int64_t)gx * gy, K, 1);
+    // Equal runs of slabs, one block per SM, for single products and losses
+    // (whole tiles left up to half of the last wave idle: W^T A 32,000 x 24,000,
+    // k = 50, 1659 -> 1613 us; A H^T at k = 64 2263 -> 1898; loss and gradients
+    // 20,000 x 10,000, k = 100, 2753 -> 2429).  Whole K splits (S0) in a
+    // factorisation: its sweeps amplify the sums' last bits (1e-5 in a trace-form
+    // residual after eight sweeps).  Where those splits leave a quarter of the SMs
+    // without a block, equal runs whose slab sums are folded as the splits would
+    // be (8 HALS iterations, 15,000 x 1200, k = 20: 3100 -> 1612 us; at 12,000 x
+    // 8000, k = 64, 128 blocks, the kept slabs cost 4 %).
+    int64_t S = S0;
+    even = even && K > 0;
+    const bool keep = !even && K > 0 && simt_keep_slabs(M, K, BN, (int)gy) &&
+                      (int64_t)gx * gy * S0 * 4 <= (int64_t)sms * 3;
+    const int group = keep ? (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB) : 0;
+    if (even || keep) S = std::min<int64_t>(sms, (int64_t)gx * gy * ((K + SLAB - 1) / SLAB));
     // Column tiles of 48 or 56 where these take no more of them: padding columns
     // cost FMAs like any other.  W^T A at k = 50 (56 for 64), 32,000 x 24,000:
     // 1775 -> 1657 us.  AK keeps 64 for 56: its row fragments hold four K of one
@@ -1354,20 +1551,21 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
                    : (N + 47) / 48 == (int)gy        ? 48
                    : !AK && (N + 55) / 56 == (int)gy ? 56
                                                      : 64;
-    float *Bp = parts + (((S > 4 ? S : 4) * M * (int64_t)N + 63) & ~63LL);
+    float *Bp = parts + simt_parts_floats(M, K, N, even);
     const float *Bs = direct ? B : Bp;
     if (simt_factor_map(&mapB, Bs, K, N, ldp, bn)) {
       const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
       cudaError_t e = direct ? cudaSuccess : launch_copy2d(B, N, Bp, ldp, K, N, s);
       if (e == cudaSuccess)
-        e = launch_simt_tma_n<AK, 8, true>(bn, mapA, mapB, A, lda, B, M, K, N, S > 1 ? parts : C,
-                                           kchunk, S, 0, err, s);
-      if (e != cudaSuccess || S == 1) return e;
-      return sum_parts(parts, S, M * (int64_t)N, C, s);
+        e = launch_simt_tma_n<AK, 8, true>(bn, mapA, mapB, A, lda, B, M, K, N,
+                                           !even && !keep && S > 1 ? parts : C, kchunk, (int)S, group,
+                                           even || keep ? parts : nullptr, err, s);
+      if (e != cudaSuccess || even || keep || S == 1) return e;
+      return sum_parts(parts, (int)S, M * (int64_t)N, C, s);
     }
   }
   const unsigned gx = (unsigned)((M + BM - 1) / BM);
-  const int S = parts ? simt_wave_splits((int64_t)gx * gy, K, 2 * (int64_t)sms) : 1;
+  const int S = S0;
   const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
   float *out = S > 1 ? parts : C;
   const dim3 grid(gx, gy, (unsigned)S);
@@ -1413,7 +1611,7 @@ bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partial
   if (S < 1) S = 1;
   const int64_t kchunk = ((rows + S - 1) / S + 127) / 128 * 128;
   S = (rows + kchunk - 1) / kchunk;
-  *status = launch_simt_tma<false, 8, 64, true>(mapA, mapB, X, k, X, k, rows, k, partials, k, kchunk, (int)S, 0, err, s);
+  *status = launch_simt_tma<false, 8, 64, true>(mapA, mapB, X, k, X, k, rows, k, partials, k, kchunk, (int)S, 0, nullptr, err, s);
   if (*status != cudaSuccess) return true;
   k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads((int)S), 0, s>>>(partials, (int)S, k, G);
   g_launches += 1;
@@ -1423,21 +1621,18 @@ bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partial
 }  // namespace
 
 cudaError_t launch_aht_simt(const float *A, int64_t m, int64_t n, int64_t lda, const float *Ht,
-                            int k, float *P, float *parts, int *err, cudaStream_t s) {
-  return gemm_simt<true>(A, lda, m, n, Ht, k, P, parts, err, s);
+                            int k, float *P, float *parts, bool even, int *err, cudaStream_t s) {
+  return gemm_simt<true>(A, lda, m, n, Ht, k, P, parts, even, err, s);
 }
 
 cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, const float *W,
-                            int k, float *P, float *parts, int *err, cudaStream_t s) {
-  return gemm_simt<false>(A, lda, n, m, W, k, P, parts, err, s);
+                            int k, float *P, float *parts, bool even, int *err, cudaStream_t s) {
+  return gemm_simt<false>(A, lda, n, m, W, k, P, parts, even, err, s);
 }
 
-size_t simt_parts_bytes(int64_t rows, int k) {
-  // four partials of `rows` rows, or 16 of the few tiles that are split further
-  // (then tiles x splits is at most the SM count), and the padded factor
-  const size_t few = (size_t)simt_sms() * 256 + 16 * 256;
-  const size_t most = 4 * (size_t)rows > few ? 4 * (size_t)rows : few;
-  return sizeof(float) * (((most * k + 63) & ~(size_t)63) + (size_t)rows * ((k + 3) & ~3));
+size_t simt_parts_bytes(int64_t m, int64_t n, int k, bool even) {
+  const int64_t parts = std::max(simt_parts_floats(m, n, k, even), simt_parts_floats(n, m, k, even));
+  return sizeof(float) * (size_t)(parts + std::max(m, n) * ((k + 3) & ~3));
 }
 
 // ------------------------------------------------------------------ transpose
