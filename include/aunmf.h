@@ -323,8 +323,8 @@ int aunmf_check_status(int *site);
  *              AUNMF_E_NOMEM (cudaMalloc is not called); buffers a handle
  *              already holds stay usable
  *            AUNMF_INJECT_SIMT_WAIT     the TMA-fed FP32 kernel: dense FP32
- *              products with k > 32 (aunmf_run, aunmf_relres, aunmf_aht /
- *              aunmf_wta in FP32) and the Gram matrices at k >= 96 (a
+ *              products of 16-byte aligned rows or few output tiles
+ *              (aunmf_run, aunmf_relres, aunmf_aht / aunmf_wta in FP32) and the Gram matrices at k >= 96 (a
  *              multiple of 4, >= 1024 rows) in every precision: thread 0
  *              never arrives on the first stage's barrier, so every thread's
  *              wait for that stage runs out
