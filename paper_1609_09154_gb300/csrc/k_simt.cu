@@ -865,7 +865,7 @@ __device__ __forceinline__ int simt_col(int tx, int j) {
     return tx * TN + j;
 }
 
-template <bool AK, int RT, int BN, bool VEC>
+template <bool AK, int RT, int BN, bool VEC, bool RUNS>
 __global__ void __launch_bounds__(kTThreads, 1)
     k_gemm_simt_tma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const float *__restrict__ A, int64_t lda, const float *__restrict__ B,
@@ -877,19 +877,21 @@ __global__ void __launch_bounds__(kTThreads, 1)
   // launch that pads B's rows to 16 bytes for TMA (mapB is not used).  VEC
   // false (short form only): A's rows are not 16-byte aligned, and its tile is
   // copied the same way into the same places (mapA is not used).
-  static_assert(VEC || RT == 4, "unaligned rows: short form");
+  static_assert((VEC || RT == 4) && !(RUNS && RT == 4), "unaligned rows: short form");
   // clus > 0: the grid's clus K splits of a tile form one cluster (1, 1, clus):
   // every block keeps its slab sums in shared memory, and the cluster folds all
   // of them, in K order, through distributed shared memory: with Kahan's
   // compensation within each `group` slabs, the groups' sums added plainly --
   // the additions of an unclustered pass over K split every `group` slabs, so
   // both give the same bits.  clus == 0: split z writes its partial at C + z M ldc.
-  // parts (RT = 8): the grid is one block per SM and the tiles' slabs, tile
+  // RUNS (parts given): the grid is one block per SM and the tiles' slabs, tile
   // after tile, are cut into equal runs, one per block (SimtRuns).  A block
   // writes a tile it has all of to C, another one's part to its first (the
   // run's first tile) or second (its last) slot of parts, for k_simt_join.
   // parts and group > 0: every slab's sums go to parts, slab after slab, for
-  // k_simt_fold, which adds them as a cluster does.
+  // k_simt_fold, which adds them as a cluster does.  (A form of its own: the
+  // runs' bookkeeping in the slab loop cost a grid of whole tiles 2-4 %: five HALS
+  // iterations at 24,000 x 16,000, k = 50, 10,860 -> 10,480 us without it.)
   // inject (test hook): thread 0 never arrives on the first stage's barrier,
   // so every thread's bounded wait runs out
   using namespace aunmf::ptx;
@@ -911,14 +913,14 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int n0 = blockIdx.y * BN;
   const int64_t kz0 = (int64_t)blockIdx.z * kchunk, kz1 = min(K, kz0 + kchunk);
   int nsteps = kz1 > kz0 ? (int)((kz1 - kz0 + kTBK - 1) / kTBK) : 0;
-  // RT = 8: the tile (row tile * gy + column tile) and the K step within it that
+  // RUNS: the tile (row tile * gy + column tile) and the K step within it that
   // the copies and the sums have reached; a tile ends after nst steps
   const int nst = (int)((K + kTBK - 1) / kTBK);
-  const int gy = RT == 8 && parts ? (N + BN - 1) / BN : gridDim.y;
-  int64_t tile0 = (int64_t)blockIdx.x * gy + blockIdx.y;
-  int step0 = (int)(kz0 / kTBK);
+  const int gy = (N + BN - 1) / BN;
+  int64_t tile0 = 0;
+  int step0 = 0;
   int64_t u0 = 0;
-  if (RT == 8 && parts) {
+  if (RUNS) {
     const SimtRuns r = simt_runs(M, K, gy, gridDim.x);
     const int64_t u1 = r.first(blockIdx.x + 1);
     u0 = r.first(blockIdx.x);
@@ -947,7 +949,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     int k0 = (int)(kz0 + (int64_t)s * kTBK);
     int64_t fm = m0;
     int fn = n0;
-    if constexpr (RT == 8) {
+    if constexpr (RUNS) {
       k0 = fk * kTBK;
       fm = ft / gy * BM;
       fn = (int)(ft % gy) * BN;
@@ -1161,22 +1163,22 @@ __global__ void __launch_bounds__(kTThreads, 1)
       }
     }
     mbar_arrive(&empty[st]);
-    const bool last = s + 1 == nsteps || (RT == 8 && ck + 1 == nst);
+    const bool last = s + 1 == nsteps || (RUNS && ck + 1 == nst);
     if (++slab == kTSlabSteps || last) {
       if (clus > 0) {
         keep(s / kTSlabSteps);
-      } else if (RT == 8 && group > 0) {
+      } else if (RUNS && group > 0) {
         keep_at(parts + (u0 + kept++) * BM * BN);
       } else {
         fold();
       }
       slab = 0;
     }
-    if constexpr (RT == 8) {
+    if constexpr (RUNS) {
       ++ck;
       if (last && group > 0) {
         ck = 0;
-      } else if (parts && last) {
+      } else if (last) {
         const int64_t tm = ct / gy * BM;
         const int tn = (int)(ct % gy) * BN;
         float *slot = parts + (2 * (int64_t)blockIdx.x + (ct != tile0)) * 2 * BM * BN;
@@ -1256,7 +1258,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     cluster_sync();  // no block's shared memory goes away while a peer reads it
     return;
   }
-  if (!ok || (RT == 8 && parts)) return;
+  if (!ok || RUNS) return;
   C += (int64_t)blockIdx.z * M * ldc;
 #pragma unroll
   for (int i = 0; i < RT; ++i) {
@@ -1415,7 +1417,9 @@ cudaError_t launch_simt_tma(const CUtensorMap &mapA, const CUtensorMap &mapB, co
                             int64_t lda, const float *B, int64_t M, int64_t K, int N, float *C, int ldc, int64_t kchunk, int S,
                             int group, float *parts, int *err, cudaStream_t s) {
   using T = SimtTile<RT, BN>;
-  auto kern = k_gemm_simt_tma<AK, RT, BN, VEC>;
+  auto kern = k_gemm_simt_tma<AK, RT, BN, VEC, false>;
+  if constexpr (RT == 8)
+    if (parts) kern = k_gemm_simt_tma<AK, RT, BN, VEC, true>;
   const bool clus = group > 0 && !parts;
   const size_t smem = T::smem(clus ? (int)(kchunk / (kTBK * kTSlabSteps)) : 0);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1540,12 +1544,12 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
     const unsigned gx = (unsigned)((M + 255) / 256);
     // Equal runs of slabs, one block per SM, for single products and losses
     // (whole tiles left up to half of the last wave idle: W^T A 32,000 x 24,000,
-    // k = 50, 1659 -> 1613 us; A H^T at k = 64 2263 -> 1898; loss and gradients
-    // 20,000 x 10,000, k = 100, 2753 -> 2429).  Whole K splits (S0) in a
+    // k = 50, 1659 -> 1594 us; A H^T at k = 64 2263 -> 1898; loss and gradients
+    // 20,000 x 10,000, k = 100, 2753 -> 2377).  Whole K splits (S0) in a
     // factorisation: its sweeps amplify the sums' last bits (1e-5 in a trace-form
     // residual after eight sweeps).  Where those splits leave a quarter of the SMs
     // without a block, equal runs whose slab sums are folded as the splits would
-    // be (8 HALS iterations, 15,000 x 1200, k = 20: 3100 -> 1612 us; at 12,000 x
+    // be (8 HALS iterations, 15,000 x 1200, k = 20: 3100 -> 1543 us; at 12,000 x
     // 8000, k = 64, 128 blocks, the kept slabs cost 4 %).
     int64_t S = S0;
     even = even && K > 0;
