@@ -98,9 +98,6 @@ struct DirectArgs {
 
 // all converters
 __device__ __forceinline__ void conv_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ void fence_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 
 // (h, l) += x, exact to ~2^-48 (FP32 pair)
 __device__ __forceinline__ void pair_acc(float x, float &h, float &l) {
@@ -437,14 +434,15 @@ __global__ void __launch_bounds__(kDThreads, 1)
           pair_acc(sq, nh, nl);
           pair_acc(sd, dh, dl);
         }
-        // The slot is released only after the stores that consume the loads: an
-        // arrival right behind the loads may be performed while they still queue
-        // for shared memory, and a tile that hits L2 then overwrites the slot
-        // under them (seen as values of the tile after next).
+        // Both proxies meet here: the raw tile has been read and the next copy
+        // overwrites it, the operand tile has been written and the MMAs read it.
+        // (An arrival right behind the loads, without the fence, was seen to let a
+        // tile that hits L2 overwrite the slot under them: values of the tile after
+        // next.)
+        fence_async();
         mbar_arrive(&rempty[r]);
       }
       if (!ok) break;
-      fence_async();
       mbar_arrive(&ofull[grp]);
     }
     if (t == 0 && yissued > 0)  // the Y copies issued land before the CTA exits

@@ -1162,6 +1162,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
         }
       }
     }
+    // (cp.async, which fills unaligned rows' stages, is of the same proxy as the loads)
+    if constexpr (VEC) fence_async();
     mbar_arrive(&empty[st]);
     const bool last = s + 1 == nsteps || (RUNS && ck + 1 == nst);
     if (++slab == kTSlabSteps || last) {

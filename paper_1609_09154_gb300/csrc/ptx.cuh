@@ -30,6 +30,15 @@ __device__ __forceinline__ void mbar_expect_tx_only(uint64_t *b, uint32_t bytes)
 __device__ __forceinline__ void mbar_arrive(uint64_t *b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
 }
+// Orders this thread's shared-memory accesses so far before later ones of the
+// asynchronous proxy (TMA copies, tensor-core operand reads) that a barrier
+// puts behind them: after writing an operand tile, and also after reading a tile
+// that a TMA copy will overwrite.  An arrival alone orders only this proxy's
+// accesses: without the fence, or a wait for the loaded values, it can be performed
+// while the loads still queue, and the next copy lands under them.
+__device__ __forceinline__ void fence_async() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 __device__ __forceinline__ bool mbar_try(uint64_t *b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
