@@ -1754,9 +1754,11 @@ __device__ void block_sum_d2(double &a, double &b) {
 // products that read A itself; the last block adds the partials.  Rows without
 // padding are one vector of m n entries.  Each thread squares 16 entries at a
 // time (four 16-byte loads in flight) in FP32 and adds the 16-term sums in
-// FP64 (an FP64 add per entry would bound the pass); EXACT: the squares of a
-// group are summed as an FP32 pair (~2^-48) instead.  Bound by HBM at large
-// sizes; a block per row with one FP32 chain per thread left 4.6 TB/s.
+// FP64 (an FP64 add per entry would bound the pass).  EXACT (sparse A, far fewer
+// entries): every square in FP64, which no finite entry overflows or loses; in FP32
+// pairs an entry above 1.8e19 makes the sum a NaN and one below 1e-23 nothing.
+// Bound by HBM at large sizes (a block per row with one FP32 chain per thread left
+// 4.6 TB/s), EXACT by the FP64 rate (5e7 entries: 162 us more than the pairs).
 template <bool EXACT>
 __global__ void __launch_bounds__(256)
     k_norm2(const float *__restrict__ A, int64_t m, int64_t n, int64_t lda,
@@ -1788,10 +1790,10 @@ __global__ void __launch_bounds__(256)
       }
     }
     if constexpr (EXACT) {
-      float hi = 0.f, lo = 0.f;
+      double d[4] = {};
 #pragma unroll
-      for (int q = 0; q < 16; ++q) two_fma_acc(v[q], v[q], hi, lo);
-      s += (double)hi + (double)lo;
+      for (int q = 0; q < 16; ++q) d[q & 3] = fma((double)v[q], (double)v[q], d[q & 3]);
+      s += (d[0] + d[1]) + (d[2] + d[3]);
     } else {
       float a = 0.f, b = 0.f;
 #pragma unroll
@@ -1873,7 +1875,8 @@ __global__ void __launch_bounds__(256)
     *last = 0.5 * f;
   } else {
     const double r2 = f < 0.0 ? 0.0 : f;
-    const double rr = a2 > 0.0 ? sqrt(r2 / a2) : 0.0;
+    // (a NaN in ||A||^2 has to reach nonfinite: 0 only for A = 0)
+    const double rr = a2 == 0.0 ? 0.0 : sqrt(r2 / a2);
     if (!isfinite(rr)) ctr->nonfinite += 1;
     if (relres) relres[ctr->iter] = rr;
     ctr->iter += 1;
