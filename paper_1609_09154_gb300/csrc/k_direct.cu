@@ -294,8 +294,22 @@ __global__ void __launch_bounds__(kDThreads, 1)
     const uint64_t pol_y = policy_evict_last();
     int64_t yissued = 0;
     bool ok = true;
-    float nh = 0.f, nl = 0.f, dh = 0.f, dl = 0.f;  // NORM: FP32 pairs
-    float sq, sd;
+    // NORM: chains of 16 terms, as launch_prepare sums them, joined in FP32 pairs
+    // (a chain over the thread's whole 64 terms of a tile errs four times as much on
+    // entries of few values; every chain into FP64, as there, took 524 us for the
+    // loss of 20,000 x 24,000, k = 50, TF32, and 500 BF16, this way 495 and 416, the
+    // chain of 64 480 and 409).  The pairs hold a quarter of the sums, so that a
+    // tile's four chains fit wherever one does, and go to FP64 before they are large.
+    float nh = 0.f, nl = 0.f, dh = 0.f, dl = 0.f;
+    double na = 0.0, nd = 0.0;
+    float sq = 0.f, sd = 0.f;
+    auto join = [&]() {
+      if constexpr (NORM) {
+        pair_acc(0.25f * sq, nh, nl);
+        pair_acc(0.25f * sd, dh, dl);
+        sq = sd = 0.f;
+      }
+    };
     auto use = [&](float a) {  // rounded value, and the two sums of it
       float v;
       if constexpr (BF16)
@@ -359,7 +373,6 @@ __global__ void __launch_bounds__(kDThreads, 1)
           break;
         }
         const float *rw = reinterpret_cast<const float *>(raw + (size_t)r * kRawBytes);
-        sq = sd = 0.f;
         // (unaligned form: K past the end, which a class without rows does not
         // zero-fill)
         const int kv = VEC ? 32 : (int)min((int64_t)32, L.K - (w.s * RPS + h) * 32);
@@ -414,6 +427,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
             const float a2 = at(4 * c + 2, i & 1), a3 = at(4 * c + 3, i & 1);
             reinterpret_cast<float4 *>(xo)[row * 8 + (c ^ (row & 7))] =
                 make_float4(use(a0), use(a1), use(a2), use(a3));
+            if ((i & 3) == 3) join();
           }
         } else {
 #pragma unroll
@@ -428,12 +442,16 @@ __global__ void __launch_bounds__(kDThreads, 1)
             o.z = pack_bf(use(a[4]), use(a[5]));
             o.w = pack_bf(use(a[6]), use(a[7]));
             reinterpret_cast<uint4 *>(xo)[row * 8 + ((4 * h + c) ^ (row & 7))] = o;
+            if (i & 1) join();
           }
         }
-        if constexpr (NORM) {
-          pair_acc(sq, nh, nl);
-          pair_acc(sd, dh, dl);
-        }
+        if constexpr (NORM)
+          if (nh > 1e30f) {  // (|dh| is smaller)
+            na += (double)nh;
+            nd += (double)dh;
+            if (isinf(nh)) nl = 0.f;  // (inf - inf in the pair's sum)
+            nh = dh = 0.f;
+          }
         // Both proxies meet here: the raw tile has been read and the next copy
         // overwrites it, the operand tile has been written and the MMAs read it.
         // (An arrival right behind the loads, without the fence, was seen to let a
@@ -449,7 +467,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
       mbar_wait_drain(&yfull[grp], (uint32_t)((yissued - 1) & 1), L.wait_cycles);
     if constexpr (NORM) {
       // fixed order: lanes by butterfly, then the eight warps
-      double a = (double)nh + (double)nl, d = (double)dh + (double)dl;
+      double a = 4.0 * (na + ((double)nh + (double)nl)), d = 4.0 * (nd + ((double)dh + (double)dl));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, o);
