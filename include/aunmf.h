@@ -123,7 +123,12 @@ typedef struct {
 /* Creates a handle bound to the current CUDA device and `stream` (a
  * cudaStream_t; NULL = the legacy default stream).  *h receives the handle. */
 int aunmf_create(aunmf_handle **h, void *stream);
-/* Rebinds the handle to another stream of the same device. */
+/* Rebinds the handle to another stream of the same device.  What the handle has
+ * enqueued on the stream bound so far (which still exists) comes before what it
+ * enqueues on the new one, by an event; the call does not synchronise, unless the
+ * new stream is being captured (then the host waits for the old one's work).
+ * Graphs that the caller captures from a handle's calls use its workspace: order
+ * their launches with the handle's other work. */
 int aunmf_set_stream(aunmf_handle *h, void *stream);
 /* Frees the workspace and the handle (synchronises its stream first). */
 int aunmf_destroy(aunmf_handle *h);
