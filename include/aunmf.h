@@ -77,7 +77,11 @@ typedef struct {
 typedef struct {
   int prec;           /* AUNMF_FP32 (default) / AUNMF_TF32 / AUNMF_BF16 */
   double mu_eps;      /* MU: added to the denominator of Eq. muupdate; 0 -> 1e-16 */
-  int bpp_max_pivots; /* ABPP: exchange cap per right-hand side; 0 -> 10*k */
+  int bpp_max_pivots; /* ABPP: exchange cap per right-hand side and solver; 0 -> 10*k.  A
+                         right-hand side that the fast solver hands to the FP64 fallback (see
+                         bpp_redone) has the cap's exchanges there again: one whose FP32 solve
+                         broke down, or one that reached a cap of at least 10*k on a Gram of
+                         condition >= 1e8 (a smaller cap ends it). */
   int use_graph;      /* 1: capture one iteration as a CUDA graph and replay it */
   int profile;        /* 1: time product / update / Gram phases with CUDA events */
   int hals_variant;   /* HALS: 0 = exact coordinate steps, normalisation compensated in H;
@@ -100,7 +104,8 @@ typedef struct {
 /* Per-call report, filled when the pointer is non-NULL. */
 typedef struct {
   int64_t bpp_pivots;       /* total BPP exchanges over all right-hand sides and iterations */
-  int64_t bpp_nonconverged; /* right-hand sides that hit the pivot cap */
+                            /*   (not those before an FP32 solve broke down)                */
+  int64_t bpp_nonconverged; /* right-hand sides that ended at the pivot cap */
   int64_t bpp_numeric;      /* right-hand sides with a non-positive Cholesky pivot */
   int iters_done;
   float ms_total;           /* device time of the whole call (CUDA events) */
@@ -111,7 +116,7 @@ typedef struct {
   int tuned_bpp_warps;      /* aunmf_run_batched: autotuned BPP work tile (warps per block, */
   int tuned_bpp_rows;       /*   rows per warp per item)                                    */
   int64_t bpp_redone;       /* right-hand sides the fast BPP solver handed to the direct    */
-                            /*   (cold-start, full-size Cholesky) fallback                  */
+                            /*   (FP64, full-size Cholesky) fallback                        */
   double pgrad_first;       /* stop_tol > 0: projected-gradient norm of (W0, H0) ...        */
   double pgrad_last;        /*   ... and of the state the last iteration started from       */
   int tuned_gemm_stages_aht; /* aunmf_run_batched: autotuned pipeline stages of the grouped */
@@ -232,8 +237,8 @@ int aunmf_update_h(aunmf_handle *h, int algo, float *H, const float *PH, const f
  * G = C^T C (k x k float32 [device]) and r = C^T b, to FP64 accuracy (FP32
  * solves refined with FP32-pair residuals, FP64 where they cannot finish); writes x as row r
  * of X (nrhs x k float32 [device]).  pivots/nonconv (may be NULL) [host]
- * receive the total exchanges and the number of right-hand sides that hit
- * max_pivots (0 -> 10*k).  Returns AUNMF_E_NOCONVERGE / AUNMF_E_NUMERIC if
+ * receive the total exchanges and the number of right-hand sides that ended at
+ * max_pivots (0 -> 10*k; the cap is as aunmf_options.bpp_max_pivots).  Returns AUNMF_E_NOCONVERGE / AUNMF_E_NUMERIC if
  * any right-hand side failed (X still written).  Synchronises. */
 int aunmf_nls_bpp(aunmf_handle *h, const float *G, const float *R, int64_t nrhs, int k, float *X,
                   int max_pivots, int64_t *pivots, int64_t *nonconv);

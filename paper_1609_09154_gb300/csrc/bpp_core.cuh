@@ -491,18 +491,27 @@ __device__ __forceinline__ bool solve_mixed(const float *Mh, const float *Ml, in
 // X's row; warm 2: from the positive entries of the unconstrained solution
 // z = G^{-1} r when G^{-1} is usable (else as warm 1) -- for a first update,
 // whose X (zero, or a random start) says nothing about the solution; warm 0:
-// from the empty passive set); returns the exchanges, *failed_numeric /
-// *failed_cap.  Each
+// from the empty passive set); returns the exchanges, *redo (what the fallback
+// kernel does with the row) and *failed_cap (the cap ended it, in X as it was).
+// Each
 // lane keeps its entries of r (FP32), x and y (FP32 pairs) and the
 // tolerances (FP32): the exchange rule needs only their signs and
 // magnitudes, and FP64 instructions -- conversions and compares included --
 // run at ~1/60 of the FP32 rate.  The passive-set systems are solved by
 // solve_mixed; a system it cannot finish sends the row to the FP64 fallback
 // kernel (k_bpp_direct), so this kernel keeps no FP64 state.
+// kRedoSolve: a system the FP32 solve could not finish.  kRedoGoOn: with an ill-
+// conditioned G (cond >= 1e8) a row at a cap of at least 10 k exchanges has been
+// going round in circles on the solves' own rounding (an x_j within cond 2^-44 of 0
+// changes sign and back); the FP64 kernel, whose noise is ~500 times smaller, goes
+// on from the set it reached, with the same cap.  Which rows these are depends on
+// the last bits of G and R.
+enum : uint8_t { kRedoNone = 0, kRedoSolve = 1, kRedoGoOn = 2 };
+
 template <int KT>
 __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__restrict__ R,
                                             int64_t row, int k, float *__restrict__ X, int warm,
-                                            int max_piv, bool *failed_numeric_out,
+                                            int max_piv, uint8_t *redo_out,
                                             bool *failed_cap_out) {
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -825,6 +834,9 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
     }
     need_solve = true;
   }
+  const uint8_t redo = failed_numeric                                 ? kRedoSolve
+                       : failed_cap && w.refine && max_piv >= 10 * k ? kRedoGoOn
+                                                                      : kRedoNone;
   // a row handed to the fallback gets the passive set it had reached (1 on
   // it, 0 elsewhere), which the fallback starts from: in the first
   // iteration, whose previous iterate is the random start, that saves the
@@ -832,10 +844,10 @@ __device__ __forceinline__ int bpp_row_fast(const BppWarp &w, const float *__res
 #pragma unroll
   for (int t = 0; t < KT; ++t) {
     const int j = lane + 32 * t;
-    if (j < k) X[row * k + j] = failed_numeric ? (pas[t] ? 1.f : 0.f) : __fadd_rn(xh[t], xl[t]);
+    if (j < k) X[row * k + j] = redo ? (pas[t] ? 1.f : 0.f) : __fadd_rn(xh[t], xl[t]);
   }
-  *failed_numeric_out = failed_numeric;
-  *failed_cap_out = failed_cap;
+  *redo_out = redo;
+  *failed_cap_out = failed_cap && !redo;
   return it;
 }
 

@@ -343,14 +343,15 @@ __global__ void __launch_bounds__(32 * bpp::kBppWarps, 1)
     const float *R = side ? b.PHt : b.PW;
     float *X = side ? b.Ht : b.W;
     for (int64_t row = I.r0 + wib; row < I.r1; row += nwb) {
-      bool fnum, fcap;
+      uint8_t again;
+      bool fcap;
       // problems with k <= 32 take the one-index-per-lane form even in a
       // launch sized for larger ranks (fewer instructions per exchange)
       const int n_ex = (KT > 1 && k <= 32)
-                           ? bpp::bpp_row_fast<1>(w, R, row, k, X, warm, max_piv, &fnum, &fcap)
-                           : bpp::bpp_row_fast<KT>(w, R, row, k, X, warm, max_piv, &fnum, &fcap);
-      if (lane == 0) b.redo[row] = fnum ? 1 : 0;
-      if (!fnum) {
+                           ? bpp::bpp_row_fast<1>(w, R, row, k, X, warm, max_piv, &again, &fcap)
+                           : bpp::bpp_row_fast<KT>(w, R, row, k, X, warm, max_piv, &again, &fcap);
+      if (lane == 0) b.redo[row] = again;
+      if (again != bpp::kRedoSolve) {
         piv_total += n_ex;
         nonconv += fcap;
       }
@@ -400,8 +401,9 @@ __global__ void __launch_bounds__(256)
     for (int64_t row = I.r0 + wib; row < I.r1; row += nwb) {
       if (!b.redo[row]) continue;
       bool fnum, fcap;
-      const int n_ex = bpp::bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X, cold ? 0 : 1, max_piv,
-                                                    &fnum, &fcap);
+      const int warm = !cold || b.redo[row] == bpp::kRedoGoOn;
+      const int n_ex = bpp::bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X, warm, max_piv,
+                                               &fnum, &fcap);
       piv_total += n_ex;
       nonconv += fcap;
       numeric += fnum;

@@ -33,8 +33,9 @@
 // each right-hand side from the support of its previous iterate.  Rows whose
 // fast solve cannot finish (an FP32 system too ill-conditioned to refine, or
 // a passive set too large for the route) are redone by k_bpp_direct in FP64,
-// with full-size Cholesky factorisations of G_FF, warm-started from the row's
-// previous iterate (cold if that fails at once).
+// with full-size Cholesky factorisations of G_FF, warm-started from the set the
+// fast solve reached (cold if that fails at once, and when the run asks for cold
+// starts); rows that reach the cap on an ill-conditioned G go on there.
 #include <math.h>
 
 #include "internal.cuh"
@@ -64,19 +65,11 @@ __global__ void __launch_bounds__(32 * kBppWarps, 1)
   long long piv_total = 0, nonconv = 0;
   for (int64_t row = (int64_t)blockIdx.x * nwb + wib; row < rows;
        row += (int64_t)gridDim.x * nwb) {
-    bool fnum, fcap;
-    const int it = bpp_row_fast<KT>(w, R, row, k, X, warm, max_piv, &fnum, &fcap);
-    // with an ill-conditioned G (cond >= 1e8) a row at the full cap has been
-    // going round in circles on the solves' own rounding (an x_j within
-    // cond 2^-44 of 0 changes sign and back): the FP64 kernel, whose noise is
-    // ~500 times smaller, goes on from the set it reached.  Which rows these
-    // are depends on the last bits of G and R.
-    if (fcap && w.refine && max_piv >= 10 * k) {
-      fnum = true;
-      fcap = false;
-    }
-    if (lane == 0) redo[row] = fnum ? 1 : 0;
-    if (!fnum) {
+    uint8_t again;
+    bool fcap;
+    const int it = bpp_row_fast<KT>(w, R, row, k, X, warm, max_piv, &again, &fcap);
+    if (lane == 0) redo[row] = again;
+    if (again != kRedoSolve) {
       piv_total += it;
       nonconv += fcap;
     }
@@ -148,7 +141,8 @@ __global__ void __launch_bounds__(256)
        row += (int64_t)gridDim.x * nwb) {
     if (!redo[row]) continue;
     bool fnum, fcap;
-    const int it = bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X, warm, max_piv, &fnum, &fcap);
+    const int it = bpp_row_direct<KT>(G, L, v, rs, Fl, tri, R, row, k, X,
+                                      redo[row] == kRedoGoOn ? 1 : warm, max_piv, &fnum, &fcap);
     piv_total += it;
     nonconv += fcap;
     numeric += fnum;
