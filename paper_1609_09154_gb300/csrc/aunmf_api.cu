@@ -781,7 +781,7 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
     int prc = prepare_tc(h, c, kPrepAht | kPrepWta | kPrepNorm, s);
     if (prc != AUNMF_OK) return prc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(m, n, k, false));
+    ENS(h, h->parts, simt_parts_bytes(m, n, k, simt_aligned(A->dense, A->lda), false));
     c.parts = P<float>(h->parts);
     ENS(h, h->err, sizeof(int));
     c.err = P<int>(h->err);
@@ -988,7 +988,7 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
     int rc = prepare_tc(h, c, kPrepAht, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(A->m, A->n, k, true));
+    ENS(h, h->parts, simt_parts_bytes(A->m, A->n, k, simt_aligned(A->dense, A->lda), true));
     c.parts = P<float>(h->parts);
     c.even = true;
     ENS(h, h->err, sizeof(int));
@@ -1023,7 +1023,7 @@ int aunmf_wta(aunmf_handle *h, const aunmf_matrix *A, const float *W, int k, int
     int rc = prepare_tc(h, c, kPrepWta, h->stream);
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
-    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, true));
+    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, simt_aligned(A->dense, A->lda), true));
     c.parts = P<float>(h->parts);
     c.even = true;
     ENS(h, h->err, sizeof(int));
@@ -1173,7 +1173,7 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
   CK(h, launch_transpose(H, k, n, Ht, s));
   if (A->dense) {
     CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
-    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, false));
+    ENS(h, h->parts, simt_parts_bytes(A->m, n, k, simt_aligned(A->dense, A->lda), false));
     CK(h, launch_wta_simt(A->dense, m, n, A->lda, W, k, PHt, P<float>(h->parts), false,
                           P<int>(h->err), s));
   } else {
@@ -1243,7 +1243,7 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
   } else if (A->dense) {
     if (what & kPrepNorm)
       CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
-    ENS(h, h->parts, simt_parts_bytes(m, n, k, true));
+    ENS(h, h->parts, simt_parts_bytes(m, n, k, simt_aligned(A->dense, A->lda), true));
     c.parts = P<float>(h->parts);
     c.even = true;
     ENS(h, h->err, sizeof(int));

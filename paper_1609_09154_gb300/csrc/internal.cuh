@@ -122,13 +122,14 @@ cudaError_t launch_widen(const float *G32, int k, double *G64, cudaStream_t s);
 // SIMT FP32 products.
 //   aht: P_W (m x k, ld k) = A (m x n, lda) * Ht (n x k, ld k)
 //   wta: P_Ht (n x k, ld k) = A^T (n x m) * W (m x k, ld k)
-// parts: simt_parts_bytes(m, n, k, even) bytes for partial tiles and a copy of
-// the factor with rows padded to 4 floats (null: no split, and the
-// TMA-fed form is not used).  err: the device error flag that the TMA-fed
+// parts: simt_parts_bytes(m, n, k, simt_aligned(A, lda), even) bytes for
+// partial tiles and a copy of the factor with rows padded to 4 floats (null:
+// no split, and the TMA-fed form is not used).  err: the device error flag that the TMA-fed
 // form's bounded waits raise (null: that form is not used).
 // even: a tile is cut wherever equal work for every SM cuts it; else K is cut
 // into whole splits, the same ones in every form of the product.
-size_t simt_parts_bytes(int64_t m, int64_t n, int k, bool even);
+bool simt_aligned(const float *A, int64_t lda);
+size_t simt_parts_bytes(int64_t m, int64_t n, int k, bool aligned, bool even);
 cudaError_t launch_aht_simt(const float *A, int64_t m, int64_t n, int64_t lda, const float *Ht,
                             int k, float *P, float *parts, bool even, int *err, cudaStream_t s);
 cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, const float *W,

@@ -1482,83 +1482,98 @@ cudaError_t sum_parts(const float *parts, int S, int64_t len, float *C, cudaStre
   return cudaGetLastError();
 }
 
-// Whether a product with whole K splits keeps its slab sums in memory: few
-// tiles, and at most a quarter gigabyte of them.
-bool simt_keep_slabs(int64_t M, int64_t K, int bn, int gy) {
-  const int64_t tiles = (M + 255) / 256 * gy;
-  return tiles * 4 <= simt_sms() && tiles * ((K + 127) / 128) * 256 * bn <= (1LL << 26);
-}
+// The form of a product C (M x N) over K and what it takes from its workspace.
+struct SimtPlan {
+  enum Form {
+    kGeneric,  // k_gemm_simt: the whole K splits S0
+    kCluster,  // few output tiles: 128-row tiles, K cut over a cluster of S blocks
+    kRuns,     // equal runs of slabs, joined
+    kSlabs,    // equal runs whose slab sums are kept and folded as S0 splits would be
+    kSplits    // 256-row tiles, the whole K splits S0
+  } form;
+  int BN, gy, S0;
+  int64_t S, kchunk;
+  int64_t parts;  // floats before the factor's copy: partial sums or slab sums
+};
 
-// Floats of `parts` that the product's parts take before the factor's copy.
-int64_t simt_parts_floats(int64_t M, int64_t K, int N, bool even) {
-  const int bn = N <= 16 ? 16 : N <= 32 ? 32 : 64;
-  const int gy = (N + bn - 1) / bn;
-  const int64_t slabs = (M + 255) / 256 * gy * ((K + 127) / 128);
-  const int64_t splits = 4 * M * N;
-  const int64_t other = even                               ? 4 * std::min<int64_t>(slabs, simt_sms()) * 256 * bn
-                        : simt_keep_slabs(M, K, bn, gy) ? slabs * 256 * bn
-                                                          : 0;
-  return (std::max(other, splits) + 63) & ~63LL;
+// aligned: A's rows start on 16-byte boundaries; even: as for launch_aht_simt.
+SimtPlan simt_plan(int64_t M, int64_t K, int N, bool aligned, bool even) {
+  constexpr int BM = AUNMF_SIMT_BM, SLAB = 128;
+  SimtPlan p{};
+  p.BN = N <= 16 ? 16 : (N <= 32 ? 32 : 64);
+  p.gy = (N + p.BN - 1) / p.BN;
+  const int64_t sms = simt_sms(), tiles = (M + 255) / 256 * p.gy, nsl = (K + SLAB - 1) / SLAB;
+  // K splits: of 256-row tiles on the SMs where N > 32, else of BM-row tiles,
+  // two to an SM.  Each form sums the same splits, so a call's bits do not
+  // depend on which one it takes; `even` alone cuts K elsewhere.
+  p.S0 = aligned && N > 32 ? simt_wave_splits(tiles, K, sms)
+                           : simt_wave_splits((M + BM - 1) / BM * p.gy, K, 2 * sms);
+  p.S = p.S0;
+  p.kchunk = ((K + p.S0 - 1) / p.S0 + SLAB - 1) / SLAB * SLAB;
+  p.parts = 4 * M * N;
+  p.form = SimtPlan::kGeneric;
+  // TMA-fed forms: coordinates within int32
+  if (M >= (1LL << 31) || K >= (1LL << 31)) return p;
+  const int64_t tiles4 = (M + 127) / 128 * p.gy;
+  if (tiles4 * 2 <= sms) {
+    // few output tiles (one block per tile walked all of K, at 77-87 us for 2000 x
+    // 1500, k = 10, on 12-16 of the SMs; the cluster takes 13-15).  The line on K: a
+    // block's slab sums fit beside its ring in shared memory.
+    int64_t S = std::min<int64_t>(sms / tiles4, 8);
+    const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
+    if (kchunk / SLAB * 128 * p.BN * 4 <= 128 * 1024) {
+      p.form = SimtPlan::kCluster;
+      p.S = (K + kchunk - 1) / kchunk;
+      p.kchunk = kchunk;
+      return p;
+    }
+  }
+  if (!aligned) return p;
+  // Equal runs of slabs, one block per SM, for single products and losses
+  // (whole tiles left up to half of the last wave idle: W^T A 32,000 x 24,000,
+  // k = 50, 1659 -> 1594 us; A H^T at k = 64 2263 -> 1898; loss and gradients
+  // 20,000 x 10,000, k = 100, 2753 -> 2377).  Whole K splits (S0) in a
+  // factorisation: its sweeps amplify the sums' last bits (1e-5 in a trace-form
+  // residual after eight sweeps).  Where those splits leave a quarter of the SMs
+  // without a block, and the slab sums take at most a quarter gigabyte, equal runs
+  // whose slab sums are folded as the splits would be (8 HALS iterations, 15,000 x
+  // 1200, k = 20: 3100 -> 1543 us; at 12,000 x 8000, k = 64, 128 blocks, the kept
+  // slabs cost 4 %).
+  p.form = even                                                        ? SimtPlan::kRuns
+           : tiles * 4 <= sms && tiles * p.S0 * 4 <= sms * 3 &&
+                     tiles * nsl * 256 * p.BN <= (1LL << 26) ? SimtPlan::kSlabs
+                                                             : SimtPlan::kSplits;
+  if (p.form == SimtPlan::kSplits) return p;
+  p.S = std::min<int64_t>(sms, tiles * nsl);
+  p.kchunk = ((K + p.S - 1) / p.S + SLAB - 1) / SLAB * SLAB;
+  // (at most the sum and the remainder of two tiles a block, or every slab's sum)
+  p.parts = std::max<int64_t>(p.parts, (even ? 4 * p.S : tiles * nsl) * 256 * p.BN);
+  return p;
 }
 
 template <bool AK>
 cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const float *B, int N,
                       float *C, float *parts, bool even, int *err, cudaStream_t s) {
   constexpr int BM = AUNMF_SIMT_BM, BK = 16, SLAB = 128;
-  const int vec = (reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 4 == 0) ? 1 : 0;
-  const int BN = N <= 16 ? 16 : (N <= 32 ? 32 : 64);
-  const unsigned gy = (unsigned)((N + BN - 1) / BN);
-  // TMA-fed forms: 16-byte aligned rows, coordinates within int32
-  // (parts holds the split partials, then the factor's padded copy)
+  const int vec = simt_aligned(A, lda);
+  const SimtPlan p = simt_plan(M, K, N, vec, even);
+  const int BN = p.BN, S0 = parts ? p.S0 : 1;
+  const unsigned gy = (unsigned)p.gy;
+  const bool tma = err && parts;
+  const int group = (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB);  // slabs per K split
   CUtensorMap mapA, mapB;
-  const int sms = simt_sms();
-  // K splits: of 256-row tiles on the SMs where N > 32, else of BM-row tiles,
-  // two to an SM.  Each form sums the same splits, so a call's bits do not
-  // depend on which one it takes; `even` alone cuts K elsewhere.
-  const int S0 = !parts           ? 1
-                 : vec && N > 32 ? simt_wave_splits((M + 255) / 256 * gy, K, sms)
-                                 : simt_wave_splits((M + BM - 1) / BM * gy, K, 2 * (int64_t)sms);
-  const int64_t tiles4 = (M + 127) / 128 * gy;
-  if (err && parts && M < (1LL << 31) && K < (1LL << 31) && tiles4 * 2 <= sms) {
-    // few output tiles: 128-row tiles, K cut over a cluster of up to 8 blocks
-    // (one block per tile walked all of K, at 77-87 us for 2000 x 1500, k =
-    // 10, on 12-16 of the SMs; the cluster takes 13-15).  The line on K: a
-    // block's slab sums fit beside its ring in shared memory.
-    int64_t S = sms / tiles4;
-    if (S > 8) S = 8;
-    const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
-    S = (K + kchunk - 1) / kchunk;
-    if (kchunk / SLAB * 128 * BN * 4 <= 128 * 1024) {
-      // slabs per K group
-      const int group = (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB);
-      if (vec && simt_map(&mapA, A, lda, M, K, AK, 128))
-        return launch_simt_tma_n<AK, 4, true>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
-                                              group, nullptr, err, s);
-      memset(&mapA, 0, sizeof(mapA));
-      return launch_simt_tma_n<AK, 4, false>(BN, mapA, mapA, A, lda, B, M, K, N, C, kchunk, (int)S,
-                                             group, nullptr, err, s);
-    }
+  if (tma && p.form == SimtPlan::kCluster) {
+    if (vec && simt_map(&mapA, A, lda, M, K, AK, 128))
+      return launch_simt_tma_n<AK, 4, true>(BN, mapA, mapA, A, lda, B, M, K, N, C, p.kchunk, (int)p.S,
+                                            group, nullptr, err, s);
+    memset(&mapA, 0, sizeof(mapA));
+    return launch_simt_tma_n<AK, 4, false>(BN, mapA, mapA, A, lda, B, M, K, N, C, p.kchunk, (int)p.S,
+                                           group, nullptr, err, s);
   }
-  if (vec && err && parts && M < (1LL << 31) && K < (1LL << 31) &&
-      simt_map(&mapA, A, lda, M, K, AK, 256)) {
+  if (tma && p.form != SimtPlan::kGeneric && simt_map(&mapA, A, lda, M, K, AK, 256)) {
     const int ldp = (N + 3) & ~3;
     const bool direct = ldp == N && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-    const unsigned gx = (unsigned)((M + 255) / 256);
-    // Equal runs of slabs, one block per SM, for single products and losses
-    // (whole tiles left up to half of the last wave idle: W^T A 32,000 x 24,000,
-    // k = 50, 1659 -> 1594 us; A H^T at k = 64 2263 -> 1898; loss and gradients
-    // 20,000 x 10,000, k = 100, 2753 -> 2377).  Whole K splits (S0) in a
-    // factorisation: its sweeps amplify the sums' last bits (1e-5 in a trace-form
-    // residual after eight sweeps).  Where those splits leave a quarter of the SMs
-    // without a block, equal runs whose slab sums are folded as the splits would
-    // be (8 HALS iterations, 15,000 x 1200, k = 20: 3100 -> 1543 us; at 12,000 x
-    // 8000, k = 64, 128 blocks, the kept slabs cost 4 %).
-    int64_t S = S0;
-    even = even && K > 0;
-    const bool keep = !even && K > 0 && simt_keep_slabs(M, K, BN, (int)gy) &&
-                      (int64_t)gx * gy * S0 * 4 <= (int64_t)sms * 3;
-    const int group = keep ? (int)(((K + S0 - 1) / S0 + SLAB - 1) / SLAB) : 0;
-    if (even || keep) S = std::min<int64_t>(sms, (int64_t)gx * gy * ((K + SLAB - 1) / SLAB));
+    const bool runs = p.form == SimtPlan::kRuns || p.form == SimtPlan::kSlabs;
     // Column tiles of 48 or 56 where these take no more of them: padding columns
     // cost FMAs like any other.  W^T A at k = 50 (56 for 64), 32,000 x 24,000:
     // 1775 -> 1657 us.  AK keeps 64 for 56: its row fragments hold four K of one
@@ -1568,17 +1583,18 @@ cudaError_t gemm_simt(const float *A, int64_t lda, int64_t M, int64_t K, const f
                    : (N + 47) / 48 == (int)gy        ? 48
                    : !AK && (N + 55) / 56 == (int)gy ? 56
                                                      : 64;
-    float *Bp = parts + simt_parts_floats(M, K, N, even);
+    // (parts holds the parts, then the factor's padded copy)
+    float *Bp = parts + ((p.parts + 63) & ~63LL);
     const float *Bs = direct ? B : Bp;
     if (simt_factor_map(&mapB, Bs, K, N, ldp, bn)) {
-      const int64_t kchunk = ((K + S - 1) / S + SLAB - 1) / SLAB * SLAB;
       cudaError_t e = direct ? cudaSuccess : launch_copy2d(B, N, Bp, ldp, K, N, s);
       if (e == cudaSuccess)
         e = launch_simt_tma_n<AK, 8, true>(bn, mapA, mapB, A, lda, B, M, K, N,
-                                           !even && !keep && S > 1 ? parts : C, kchunk, (int)S, group,
-                                           even || keep ? parts : nullptr, err, s);
-      if (e != cudaSuccess || even || keep || S == 1) return e;
-      return sum_parts(parts, (int)S, M * (int64_t)N, C, s);
+                                           !runs && p.S > 1 ? parts : C, p.kchunk, (int)p.S,
+                                           p.form == SimtPlan::kSlabs ? group : 0,
+                                           runs ? parts : nullptr, err, s);
+      if (e != cudaSuccess || runs || p.S == 1) return e;
+      return sum_parts(parts, (int)p.S, M * (int64_t)N, C, s);
     }
   }
   const unsigned gx = (unsigned)((M + BM - 1) / BM);
@@ -1647,9 +1663,14 @@ cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, c
   return gemm_simt<false>(A, lda, n, m, W, k, P, parts, even, err, s);
 }
 
-size_t simt_parts_bytes(int64_t m, int64_t n, int k, bool even) {
-  const int64_t parts = std::max(simt_parts_floats(m, n, k, even), simt_parts_floats(n, m, k, even));
-  return sizeof(float) * (size_t)(parts + std::max(m, n) * ((k + 3) & ~3));
+bool simt_aligned(const float *A, int64_t lda) {
+  return reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 4 == 0;
+}
+
+size_t simt_parts_bytes(int64_t m, int64_t n, int k, bool aligned, bool even) {
+  const int64_t parts =
+      std::max(simt_plan(m, n, k, aligned, even).parts, simt_plan(n, m, k, aligned, even).parts);
+  return sizeof(float) * (size_t)(((parts + 63) & ~63LL) + std::max(m, n) * ((k + 3) & ~3));
 }
 
 // ------------------------------------------------------------------ transpose
