@@ -324,9 +324,10 @@ cudaError_t product_wta(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
 // rounding term are wanted now (kPrepNorm).
 enum { kPrepAht = 1, kPrepWta = 2, kPrepNorm = 4 };
 int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s);
-// Setup of the sparse products: the long rows of the CSR (A H^T); the CSC copy
-// of A and its long rows (W^T A).
-int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s);
+// Setup of the sparse products: the long rows of the CSR (A H^T; H, which may be
+// null, is transposed into c.Ht in the same launch); the CSC copy of A and its long
+// rows (W^T A).
+int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s, const float *H = nullptr);
 int prepare_csc(aunmf_handle *h, RunCtx &c, cudaStream_t s);
 
 cudaError_t update(RunCtx &c, float *X, const float *Pm, const float *G, const double *G64,
@@ -479,10 +480,11 @@ int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s) {
   return AUNMF_OK;
 }
 
-int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
+int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s, const float *H) {
   const aunmf_matrix *A = c.A;
   ENS_TC(h, h->splr, long_rows_bytes(A->nnz, c.k));
-  cudaError_t e = list_long_rows(A->rowptr, A->m, A->nnz, c.k, h->splr.p, &c.csr_long, s);
+  cudaError_t e = list_long_rows(A->rowptr, A->m, A->nnz, c.k, h->splr.p, &c.csr_long, s, H,
+                                 A->n, c.Ht);
   return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
 }
 
@@ -982,7 +984,7 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
   c.prec = prec;
   c.Ht = P<float>(h->Ht);
   c.PW = Pout;
-  CK(h, launch_transpose(H, k, n, c.Ht, h->stream));
+  if (A->dense) CK(h, launch_transpose(H, k, n, c.Ht, h->stream));
   if (prec != AUNMF_FP32) {
     c.direct = use_split(k);
     int rc = prepare_tc(h, c, kPrepAht, h->stream);
@@ -995,7 +997,7 @@ int aunmf_aht(aunmf_handle *h, const aunmf_matrix *A, const float *H, int k, int
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), h->stream));
   } else {
-    int rc = prepare_csr_rows(h, c, h->stream);
+    int rc = prepare_csr_rows(h, c, h->stream, H);
     if (rc != AUNMF_OK) return rc;
   }
   CK(h, product_aht(h, c, h->stream));

@@ -142,12 +142,19 @@ cudaError_t launch_wta_simt(const float *A, int64_t m, int64_t n, int64_t lda, c
 // nonzeros are cut into chunks over many warps.  The line: a warp walks ~50 ns
 // a nonzero, so 512 of them are ~25 us, the tail one row may add to a product.
 constexpr int64_t kLongRowNz = 512;
+constexpr int kSpMaxSegs = 256;
+struct SpSegment {                // of the rows: its chunks' first place, their number
+  int64_t base, chunks;
+};
 struct SpLongRows {               // device memory, filled by list_long_rows
-  unsigned long long *count = nullptr;  // [0]: long rows, [1]: their chunks
+  SpSegment *seg = nullptr;
   int64_t *row = nullptr;         // {row, first chunk, chunks} each
-  int64_t *chunk = nullptr;       // {first, end nonzero} each
+  int64_t *chunk = nullptr;       // {first, end nonzero, the row's place} each
   float *part = nullptr;          // partial sums, k per chunk
+  unsigned *left = nullptr;       // arrivals at each row, 0 between products
   int64_t cap_rows = 0, cap_chunks = 0;
+  int nseg = 0;
+  int blocks = 0;                 // blocks that the chunks alone would keep busy
 };
 // (n, m and nnz bound the gathered indices in the checked build.)
 cudaError_t launch_aht_csr(const int64_t *rowptr, const int32_t *colidx, const float *val,
@@ -159,14 +166,36 @@ cudaError_t launch_wta_csc(const int64_t *colptr, const uint2 *cnz, int64_t n, i
 // mem: long_rows_bytes(nnz, k) bytes (8-byte aligned), cut up into lr and
 // filled on the device; enqueues only.
 size_t long_rows_bytes(int64_t nnz, int k);
+// in (may be null): the same launch also transposes in (k x cols) into out.
 cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
-                           SpLongRows *lr, cudaStream_t s);
+                           SpLongRows *lr, cudaStream_t s, const float *in = nullptr,
+                           int64_t cols = 0, float *out = nullptr);
 size_t csc_scratch_bytes(int64_t n, int64_t nnz);
 cudaError_t launch_csr_to_csc(const int64_t *rowptr, const int32_t *colidx, const float *val,
                               int64_t m, int64_t n, int64_t nnz, int64_t *colptr, uint2 *cnz,
                               void *scratch, cudaStream_t s);
 
 // Transpose: out (cols x rows) = in (rows x cols)^T, both row-major, dense ld.
+// (transpose_tiles: block b of nb, 32 x ny threads (tx, ty), t their scratch)
+__device__ __forceinline__ void transpose_tiles(const float *__restrict__ in, int64_t rows,
+                                                int64_t cols, float *__restrict__ out, int64_t b,
+                                                int64_t nb, float (&t)[32][33], int tx, int ty,
+                                                int ny) {
+  const int64_t tr = (rows + 31) / 32, tc = (cols + 31) / 32;
+  for (int64_t tile = b; tile < tr * tc; tile += nb) {
+    const int64_t r0 = (tile / tc) * 32, c0 = (tile % tc) * 32;
+    __syncthreads();
+    for (int y = ty; y < 32; y += ny) {
+      const int64_t r = r0 + y, c = c0 + tx;
+      if (r < rows && c < cols) t[y][tx] = in[r * cols + c];
+    }
+    __syncthreads();
+    for (int y = ty; y < 32; y += ny) {
+      const int64_t c = c0 + y, r = r0 + tx;
+      if (r < rows && c < cols) out[c * rows + r] = t[tx][y];
+    }
+  }
+}
 cudaError_t launch_transpose(const float *in, int64_t rows, int64_t cols, float *out,
                              cudaStream_t s);
 

@@ -1678,20 +1678,8 @@ namespace {
 __global__ void k_transpose(const float *__restrict__ in, int64_t rows, int64_t cols,
                             float *__restrict__ out) {
   __shared__ float t[32][33];
-  const int64_t tr = (rows + 31) / 32, tc = (cols + 31) / 32;
-  for (int64_t tile = blockIdx.x; tile < tr * tc; tile += gridDim.x) {
-    const int64_t r0 = (tile / tc) * 32, c0 = (tile % tc) * 32;
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-      const int64_t r = r0 + y, c = c0 + threadIdx.x;
-      if (r < rows && c < cols) t[y][threadIdx.x] = in[r * cols + c];
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-      const int64_t c = c0 + y, r = r0 + threadIdx.x;
-      if (r < rows && c < cols) out[c * rows + r] = t[threadIdx.x][y];
-    }
-  }
+  transpose_tiles(in, rows, cols, out, blockIdx.x, gridDim.x, t, threadIdx.x, threadIdx.y,
+                  blockDim.y);
 }
 
 __global__ void k_copy2d(const float *__restrict__ in, int64_t ld_in, float *__restrict__ out,

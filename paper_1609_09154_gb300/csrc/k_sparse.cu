@@ -7,6 +7,8 @@
 //                     A^T), gathering rows of W (m x k).
 // The CSC copy is built once per run on the device (k_csc.cu), each nonzero
 // as an 8-byte {row, value}.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace aunmf {
@@ -14,6 +16,7 @@ namespace {
 
 constexpr int kSpThreads = 256;
 constexpr int kSpWarps = kSpThreads / kWarp;
+static_assert(kSpMaxSegs == kSpThreads, "a segment per thread");
 // Nonzeros per chunk of a long row of `len`: one warp's work.  Longer chunks
 // for the longest rows, whose partial sums one block then adds.
 __device__ __forceinline__ int64_t chunk_nz(int64_t len) { return len <= 32768 ? 256 : 512; }
@@ -91,16 +94,129 @@ __device__ __forceinline__ void spmm_range(const NZ &nz, const float *__restrict
   }
 }
 
+// Y's long row `i` from its chunks' partial sums, by a whole block: warp w adds the
+// w-th eighth of the chunks in order, eight loads in flight, and the eighths are
+// added in order.  (The partials were written by other blocks of this launch.)
+template <int KT>
+__device__ __forceinline__ void long_row_sum(const SpLongRows &lr, int64_t i, int64_t rows, int k,
+                                             float *__restrict__ Y, float (&sw)[kSpWarps][32 * KT]) {
+  (void)rows;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t r = lr.row[3 * i], base = lr.row[3 * i + 1], nc = lr.row[3 * i + 2];
+  const int64_t per = (nc + kSpWarps - 1) / kSpWarps;
+  const int64_t c0 = base + w * per, c1 = min(base + nc, c0 + per);
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < KT; ++t) {
+    const int col = lane + 32 * t;
+    float acc = 0.f;
+    if (col < k) {
+      int64_t c = c0;
+      for (; c + 8 <= c1; c += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcg(&lr.part[(c + u) * k + col]);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += v[u];
+      }
+      for (; c < c1; ++c) acc += __ldcg(&lr.part[c * k + col]);
+    }
+    sw[w][32 * t + lane] = acc;
+  }
+  __syncthreads();
+  if (!AUNMF_BOUND(r >= 0 && r < rows, AUNMF_CHECK_SPMM_RANGE)) return;
+  for (int col = threadIdx.x; col < k; col += kSpThreads) {
+    float y = sw[0][col];
+#pragma unroll
+    for (int q = 1; q < kSpWarps; ++q) y += sw[q][col];
+    Y[r * k + col] = y;
+  }
+}
+
 // Y (rows x k) = S (rows x ncols, row pointers and nonzeros, nnz of them) * X
-// (ncols x k), a warp per row.  Rows longer than kLongRowNz are left to the
-// chunked kernels below.
+// (ncols x k), a warp per row; before that, the first lr.blocks blocks (one wave)
+// take the long rows' chunks.
+//
+// Long rows (a power-law hub can hold 10^6 nonzeros, which one warp would walk
+// alone, ~50 ns a nonzero, while the rest of the GPU idles: 0.9 ms of a 2e7-
+// nonzero product with rows of up to 18,000) are cut into chunks: a warp per
+// chunk writes its partial sums, and the block that writes a row's last chunk adds
+// all of them in chunk order (so results do not depend on scheduling).  The list
+// is built on the device (k_list_long) in any order within a segment of the rows,
+// each row's chunks in consecutive slots; nothing returns to the host.  One launch
+// does all of it: as three (rows, chunks, sums) a matrix without long rows paid two
+// empty ones (A H^T at 2000 x 1500, 20,000 nonzeros, k = 10: 22 us, now 13; at
+// 300,001 x 200,003, 2e7 nonzeros with long rows, k = 32, both single products
+// together 1788 us, now 1704).
+// (Blocks an SM holds by the registers that the rows' part alone takes.)
 template <int KT, class NZ>
-__global__ void __launch_bounds__(kSpThreads)
+__global__ void __launch_bounds__(kSpThreads, KT == 2 ? 6 : KT <= 4 ? 5 : KT == 8 ? 4 : 2)
     k_spmm(const int64_t *__restrict__ ptr, const NZ nz, int64_t rows, int64_t ncols, int64_t nnz,
-           const float *__restrict__ X, int k, float *__restrict__ Y) {
+           const float *__restrict__ X, int k, float *__restrict__ Y, const SpLongRows lr) {
   (void)nnz;
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ float sw[kSpWarps][32 * KT];
+  __shared__ int first[kSpMaxSegs + 1];  // chunks before each segment
+  __shared__ int64_t fin[kSpWarps];      // the rows whose last chunk this block wrote
+  const bool chunks = (int)blockIdx.x < lr.blocks;
+  const int mine = chunks && (int)threadIdx.x < lr.nseg ? (int)lr.seg[threadIdx.x].chunks : 0;
+  if (chunks && __syncthreads_or(mine)) {
+    {  // prefix sums over the segments (at most one per thread)
+      int v = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+      }
+      if (lane == 31) fin[w] = v;
+      __syncthreads();
+      for (int q = 0; q < w; ++q) v += (int)fin[q];
+      first[threadIdx.x + 1] = v;
+      if (threadIdx.x == 0) first[0] = 0;
+      __syncthreads();
+    }
+    const int total = first[lr.nseg];
+    for (int c0 = blockIdx.x * kSpWarps; c0 < total; c0 += lr.blocks * kSpWarps) {
+      const int c = c0 + w;
+      int64_t done = -1;
+      if (c < total) {
+        int b = 0, e = lr.nseg;  // first[b] <= c < first[e]
+        while (e - b > 1) {
+          const int mid = (b + e) >> 1;
+          if (first[mid] <= c) b = mid; else e = mid;
+        }
+        const int64_t slot = lr.seg[b].base + (c - first[b]);
+        const int64_t e0 = lr.chunk[3 * slot], e1 = lr.chunk[3 * slot + 1];
+        const int64_t i = lr.chunk[3 * slot + 2];
+        if (AUNMF_BOUND(e0 >= 0 && e0 <= e1 && e1 <= nnz, AUNMF_CHECK_SPMM_RANGE)) {
+          float acc[KT];
+#pragma unroll
+          for (int t = 0; t < KT; ++t) acc[t] = 0.f;
+          spmm_range<KT>(nz, X, ncols, k, e0, e1, acc, lane);
+#pragma unroll
+          for (int t = 0; t < KT; ++t) {
+            const int col = lane + 32 * t;
+            if (col < k) lr.part[slot * k + col] = acc[t];
+          }
+        }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) {
+          const unsigned nc = (unsigned)lr.row[3 * i + 2];
+          if (atomicInc(&lr.left[i], nc - 1) == nc - 1) done = i;  // (wraps to 0)
+        }
+      }
+      if (lane == 0) fin[w] = done;
+      __syncthreads();
+      for (int q = 0; q < kSpWarps; ++q) {
+        if (fin[q] < 0) continue;
+        __threadfence();
+        long_row_sum<KT>(lr, fin[q], rows, k, Y, sw);
+      }
+      __syncthreads();  // fin has been read
+    }
+  }
+  const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + w;
   const int64_t ws = (int64_t)gridDim.x * kSpWarps;
   for (int64_t r = w0; r < rows; r += ws) {
     const int64_t e0 = ptr[r], e1 = ptr[r + 1];
@@ -118,115 +234,76 @@ __global__ void __launch_bounds__(kSpThreads)
   }
 }
 
-// Long rows (a power-law hub can hold 10^6 nonzeros, which one warp would walk
-// alone, ~50 ns a nonzero, while the rest of the GPU idles: 0.9 ms of a 2e7-
-// nonzero product with rows of up to 18,000): cut into chunks, a warp per
-// chunk writes its partial sums, and a block per long row adds its chunks in
-// chunk order (so results do not depend on scheduling).  The list is built on
-// the device (k_list_long) in any order, each row's chunks in consecutive
-// slots; nothing returns to the host.
-template <int KT, class NZ>
-__global__ void __launch_bounds__(kSpThreads)
-    k_spmm_chunks(const NZ nz, int64_t ncols, int64_t nnz, const float *__restrict__ X, int k,
-                  const SpLongRows lr) {
-  (void)nnz;
+// The long rows of a row-pointer array, a block per segment of `per` rows: {row,
+// first chunk, chunks} per row and {first, end nonzero, row's place} per chunk.  A
+// segment's places start where its first nonzero says: a row of more than 512
+// takes fewer than 1 / 512 places and 3 / 512 chunks a nonzero (ceil(n / 256) <= (n
+// + 255) / 256 < 3 n / 512), so segments cannot meet and no counter is shared.
+__device__ __forceinline__ void list_segment(const int64_t *__restrict__ ptr, int64_t rows,
+                                             int64_t per, const SpLongRows &lr) {
+  __shared__ int nlong, nchunks, bad;
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kSpWarps + (threadIdx.x >> 5);
-  const int64_t ws = (int64_t)gridDim.x * kSpWarps;
-  const int64_t nchunks = min((int64_t)lr.count[1], lr.cap_chunks);
-  for (int64_t c = w0; c < nchunks; c += ws) {
-    const int64_t e0 = lr.chunk[2 * c], e1 = lr.chunk[2 * c + 1];
-    if (!AUNMF_BOUND(e0 >= 0 && e0 <= e1 && e1 <= nnz, AUNMF_CHECK_SPMM_RANGE)) continue;
-    float acc[KT];
-#pragma unroll
-    for (int t = 0; t < KT; ++t) acc[t] = 0.f;
-    spmm_range<KT>(nz, X, ncols, k, e0, e1, acc, lane);
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int col = lane + 32 * t;
-      if (col < k) lr.part[c * k + col] = acc[t];
-    }
-  }
-}
-
-// Y's long rows: warp w of a row's block adds the w-th eighth of its chunks in
-// order, eight loads in flight, and the eighths are added in order.
-template <int KT>
-__global__ void __launch_bounds__(kSpThreads)
-    k_spmm_long_sum(const SpLongRows lr, int64_t rows, int k, float *__restrict__ Y) {
-  (void)rows;
-  __shared__ float sw[kSpWarps][32 * KT];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nlong = min((int64_t)lr.count[0], lr.cap_rows);
-  for (int64_t i = blockIdx.x; i < nlong; i += gridDim.x) {
-    const int64_t r = lr.row[3 * i], base = lr.row[3 * i + 1], nc = lr.row[3 * i + 2];
-    const int64_t per = (nc + kSpWarps - 1) / kSpWarps;
-    const int64_t c0 = base + w * per, c1 = min(base + nc, c0 + per);
-    float acc[KT];
-#pragma unroll
-    for (int t = 0; t < KT; ++t) {
-      const int col = lane + 32 * t;
-      acc[t] = 0.f;
-      if (col >= k) continue;
-      int64_t c = c0;
-      for (; c + 8 <= c1; c += 8) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = lr.part[(c + u) * k + col];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc[t] += v[u];
-      }
-      for (; c < c1; ++c) acc[t] += lr.part[c * k + col];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < KT; ++t) sw[w][32 * t + lane] = acc[t];
-    __syncthreads();
-    if (!AUNMF_BOUND(r >= 0 && r < rows, AUNMF_CHECK_SPMM_RANGE)) continue;
-    for (int col = threadIdx.x; col < k; col += kSpThreads) {
-      float y = sw[0][col];
-#pragma unroll
-      for (int q = 1; q < kSpWarps; ++q) y += sw[q][col];
-      Y[r * k + col] = y;
-    }
-  }
-}
-
-// The long rows of a row-pointer array: {row, first chunk, chunks} per row and
-// {first, end nonzero} per chunk, a warp per 32 rows.
-__global__ void k_list_long(const int64_t *__restrict__ ptr, int64_t rows, const SpLongRows lr) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t ws = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r0 = w0 * 32; r0 < rows; r0 += ws * 32) {
+  const int64_t s0 = blockIdx.x * per, s1 = min(rows, s0 + per);
+  const int64_t p0 = max(ptr[s0], (int64_t)0);
+  const int64_t row0 = p0 / kLongRowNz, chunk0 = 3 * p0 / kLongRowNz;
+  if (threadIdx.x == 0) nlong = nchunks = bad = 0;
+  __syncthreads();
+  for (int64_t r0 = s0 + (threadIdx.x & ~31); r0 < s1; r0 += kSpThreads) {
     const int64_t r = r0 + lane;
-    const int64_t e0 = r < rows ? ptr[r] : 0, e1 = r < rows ? ptr[r + 1] : 0;
+    const int64_t e0 = r < s1 ? ptr[r] : 0, e1 = r < s1 ? ptr[r + 1] : 0;
     unsigned todo = __ballot_sync(0xffffffffu, e1 - e0 > kLongRowNz);
     while (todo) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
       const int64_t a = __shfl_sync(0xffffffffu, e0, src), b = __shfl_sync(0xffffffffu, e1, src);
       const int64_t cz = chunk_nz(b - a), nc = (b - a + cz - 1) / cz;
-      long long i = 0, base = 0;
+      int64_t i = 0, base = 0;
       if (lane == 0) {
-        i = (long long)atomicAdd(&lr.count[0], 1ull);
-        base = (long long)atomicAdd(&lr.count[1], (unsigned long long)nc);
+        i = row0 + atomicAdd(&nlong, 1);
+        base = chunk0 + atomicAdd(&nchunks, (int)nc);
       }
       i = __shfl_sync(0xffffffffu, i, 0);
       base = __shfl_sync(0xffffffffu, base, 0);
       // (always true for a well-formed row-pointer array of nnz nonzeros)
-      if (i >= lr.cap_rows || base + nc > lr.cap_chunks) continue;
+      if (i >= lr.cap_rows || base + nc > lr.cap_chunks) {
+        bad = 1;
+        continue;
+      }
       if (lane == 0) {
         lr.row[3 * i] = r0 + src;
         lr.row[3 * i + 1] = base;
         lr.row[3 * i + 2] = nc;
+        lr.left[i] = 0;
       }
       for (int64_t c = lane; c < nc; c += 32) {
-        lr.chunk[2 * (base + c)] = a + c * cz;
-        lr.chunk[2 * (base + c) + 1] = min(b, a + (c + 1) * cz);
+        int64_t *d = lr.chunk + 3 * (base + c);
+        d[0] = a + c * cz;
+        d[1] = min(b, a + (c + 1) * cz);
+        d[2] = i;
       }
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) lr.seg[blockIdx.x] = {chunk0, bad ? 0 : nchunks};
+}
+
+__global__ void __launch_bounds__(kSpThreads)
+    k_list_long(const int64_t *__restrict__ ptr, int64_t rows, int64_t per, const SpLongRows lr) {
+  list_segment(ptr, rows, per, lr);
+}
+
+// The same, and in the blocks after the segments' out (fc x fr) = in (fr x fc)^T: the
+// factor that the product reads, in one launch (two took a small A H^T 2.5 us more).
+__global__ void __launch_bounds__(kSpThreads)
+    k_list_transpose(const int64_t *__restrict__ ptr, int64_t rows, int64_t per, const SpLongRows lr,
+                     const float *__restrict__ in, int64_t fr, int64_t fc,
+                     float *__restrict__ out) {
+  __shared__ float t[32][33];
+  if ((int)blockIdx.x < lr.nseg)
+    list_segment(ptr, rows, per, lr);
+  else
+    transpose_tiles(in, fr, fc, out, (int64_t)blockIdx.x - lr.nseg, (int64_t)gridDim.x - lr.nseg, t,
+                    threadIdx.x & 31, threadIdx.x >> 5, kSpThreads >> 5);
 }
 
 int sp_blocks(int64_t warps) {
@@ -251,22 +328,12 @@ cudaError_t spmm(const int64_t *ptr, const NZ nz, int64_t rows, int64_t ncols, i
                  const float *X, int k, float *Y, const SpLongRows &lr, cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
   const int kt = (k + 31) / 32;
-  const int nb = sp_blocks(rows);
+  const int nb = std::max(sp_blocks(rows), lr.blocks);
 #define AUNMF_SP_MAIN(KT) \
-  k_spmm<KT, NZ><<<nb, kSpThreads, 0, s>>>(ptr, nz, rows, ncols, nnz, X, k, Y)
+  k_spmm<KT, NZ><<<nb, kSpThreads, 0, s>>>(ptr, nz, rows, ncols, nnz, X, k, Y, lr)
   AUNMF_SP_SWITCH(kt, AUNMF_SP_MAIN)
 #undef AUNMF_SP_MAIN
   g_launches += 1;
-  if (nnz > kLongRowNz) {
-    const int nbc = sp_blocks(lr.cap_chunks);
-    const int nbl = (int)(lr.cap_rows < 152 * 4 ? lr.cap_rows : 152 * 4);
-#define AUNMF_SP_CH(KT)                                                                        \
-  k_spmm_chunks<KT, NZ><<<nbc, kSpThreads, 0, s>>>(nz, ncols, nnz, X, k, lr);                   \
-  k_spmm_long_sum<KT><<<nbl, kSpThreads, 0, s>>>(lr, rows, k, Y)
-    AUNMF_SP_SWITCH(kt, AUNMF_SP_CH)
-#undef AUNMF_SP_CH
-    g_launches += 2;
-  }
   return cudaGetLastError();
 }
 
@@ -284,26 +351,40 @@ cudaError_t launch_wta_csc(const int64_t *colptr, const uint2 *cnz, int64_t n, i
   return spmm(colptr, NzPacked{cnz}, n, m, nnz, W, k, P, lr, s);
 }
 
+namespace {
+int64_t cap_long_rows(int64_t nnz) { return nnz / kLongRowNz + 1; }
+int64_t cap_long_chunks(int64_t nnz) { return 3 * nnz / kLongRowNz + 1; }
+}  // namespace
+
 size_t long_rows_bytes(int64_t nnz, int k) {
-  const int64_t cr = nnz / kLongRowNz + 1, cc = nnz / 256 + cr + 1;
-  return sizeof(int64_t) * (size_t)(2 + 3 * cr + 2 * cc) + sizeof(float) * (size_t)cc * k;
+  const size_t cr = (size_t)cap_long_rows(nnz), cc = (size_t)cap_long_chunks(nnz);
+  return sizeof(SpSegment) * kSpMaxSegs + sizeof(int64_t) * (3 * cr + 3 * cc) +
+         sizeof(unsigned) * cr + sizeof(float) * cc * k;
 }
 
 cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
-                           SpLongRows *lr, cudaStream_t s) {
-  lr->cap_rows = nnz / kLongRowNz + 1;
-  lr->cap_chunks = nnz / 256 + lr->cap_rows + 1;
-  int64_t *p = static_cast<int64_t *>(mem);
-  lr->count = reinterpret_cast<unsigned long long *>(p);
-  lr->row = p + 2;
+                           SpLongRows *lr, cudaStream_t s, const float *in, int64_t cols,
+                           float *out) {
+  lr->cap_rows = cap_long_rows(nnz);
+  lr->cap_chunks = cap_long_chunks(nnz);
+  lr->seg = static_cast<SpSegment *>(mem);
+  lr->row = reinterpret_cast<int64_t *>(lr->seg + kSpMaxSegs);
   lr->chunk = lr->row + 3 * lr->cap_rows;
-  lr->part = reinterpret_cast<float *>(lr->chunk + 2 * lr->cap_chunks);
-  if (rows == 0 || nnz <= kLongRowNz) return cudaSuccess;  // no long row: spmm skips the pass
-  cudaError_t e = cudaMemsetAsync(lr->count, 0, 2 * sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  int64_t nb = (rows + 255) / 256;
-  if (nb > 152 * 16) nb = 152 * 16;
-  k_list_long<<<(unsigned)nb, 256, 0, s>>>(ptr, rows, *lr);
+  lr->part = reinterpret_cast<float *>(lr->chunk + 3 * lr->cap_chunks);
+  lr->left = reinterpret_cast<unsigned *>(lr->part + lr->cap_chunks * k);
+  lr->blocks = lr->nseg = 0;
+  if (rows == 0 || nnz <= kLongRowNz)  // no long row
+    return in ? launch_transpose(in, k, cols, out, s) : cudaSuccess;
+  lr->blocks = (int)std::min<int64_t>((lr->cap_chunks + kSpWarps - 1) / kSpWarps, 152 * 4);
+  const int64_t per = std::max<int64_t>(512, (rows + kSpMaxSegs - 1) / kSpMaxSegs);
+  lr->nseg = (int)((rows + per - 1) / per);
+  if (in) {
+    const int64_t tiles = (k + 31) / 32 * ((cols + 31) / 32);
+    k_list_transpose<<<(unsigned)(lr->nseg + std::min<int64_t>(tiles, 152 * 16)), kSpThreads, 0, s>>>(
+        ptr, rows, per, *lr, in, k, cols, out);
+  } else {
+    k_list_long<<<(unsigned)lr->nseg, kSpThreads, 0, s>>>(ptr, rows, per, *lr);
+  }
   g_launches += 1;
   return cudaGetLastError();
 }
