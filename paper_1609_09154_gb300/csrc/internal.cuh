@@ -103,19 +103,14 @@ __device__ __forceinline__ void two_fma_acc(float a, float b, float &hi, float &
 // err: the device error flag for the bounded waits of the wide-rank form
 // (k >= 96, which runs the TMA-fed product kernel on X^T X); null keeps the
 // k_gram_part form.
-// ticket: a zeroed counter (left at 0) that lets a small factor's last block
-// add the partials; null: always a second launch.  Launches that share a
-// ticket run in stream order, as they share the partials.
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr,
-                        unsigned *ticket = nullptr);
+                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr);
 int gram_partial_blocks(int64_t rows, int max_blocks);
 // The same Gram with every product formed exactly in FP64 (FP32 x FP32 fits a
 // double) and summed in FP64: G64 (k x k, FP64) for the BPP solves, and G32 =
 // G64 rounded to FP32 (may be null).  partials: max_blocks * k * k doubles.
 cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, double *G64,
-                          float *G32, double *partials, int max_blocks, cudaStream_t s,
-                          unsigned *ticket = nullptr);
+                          float *G32, double *partials, int max_blocks, cudaStream_t s);
 // G64 = G32 widened (k x k).
 cudaError_t launch_widen(const float *G32, int k, double *G64, cudaStream_t s);
 
@@ -242,7 +237,9 @@ cudaError_t launch_bpp(const double *G, const float *R, int64_t rows, int k, flo
 
 // Reductions for the relative residual.
 // sum of squares of A (dense) or of val (CSR) into *out (device double).
-// (ticket as for launch_gram, never null here; partials: 2 nparts doubles.)
+// (ticket: a zeroed counter, left at 0, by which the last block finishes the sum;
+// launches that share one run in stream order, as they share the partials, 2
+// nparts doubles.)
 cudaError_t launch_norm2(const float *A, int64_t m, int64_t n, int64_t lda, double *partials,
                          int nparts, double *out, unsigned *ticket, cudaStream_t s);
 cudaError_t launch_norm2_vec(const float *v, int64_t len, double *partials, int nparts,

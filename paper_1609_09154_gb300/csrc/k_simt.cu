@@ -64,14 +64,10 @@ __device__ __forceinline__ int gram_groups(int ntiles) {
 //     positive definite.
 // The next 64-row slab is loaded into registers while the current one is
 // consumed from shared memory.  Dynamic shared memory: gram_smem_bytes().
-// ticket (may be null): the last block to finish adds all partials in FP64,
-// in block order, and writes G32 (FP64 form: G64, and G32 unless null), which
-// spares the reduction's launch; *ticket starts at 0 and is 0 again after.
 template <bool FP64>
 __global__ void __launch_bounds__(kGramThreads, 2)
     k_gram_part(const float *__restrict__ X, int64_t rows, int k, int64_t ldx, int64_t chunk,
-                typename std::conditional<FP64, double, float>::type *__restrict__ partials,
-                float *__restrict__ G32, double *__restrict__ G64, unsigned *ticket) {
+                typename std::conditional<FP64, double, float>::type *__restrict__ partials) {
   using T = typename std::conditional<FP64, double, float>::type;
   extern __shared__ __align__(16) float sX[];  // [kGramRows][kp], then the group sums
   constexpr int kPre = (kGramRows * 64 + kGramThreads - 1) / kGramThreads;  // k <= 64 prefetch
@@ -132,6 +128,9 @@ __global__ void __launch_bounds__(kGramThreads, 2)
         }
         if (c0 + kGramRows < r1) fetch(c0 + kGramRows);
       } else {
+        // (eight loads in flight; left to the compiler, the loop's form depended on
+        // code elsewhere in the kernel: 20,000 rows, k = 90: 55 against 49 us)
+#pragma unroll 8
         for (int idx = threadIdx.x; idx < slab; idx += kGramThreads) {
           const int rr = __float2int_rz(((float)idx + 0.5f) * inv_kp), cc = idx - rr * kp;
           sX[idx] = (rr < nr && cc < k) ? X[(c0 + rr) * ldx + cc] : 0.f;
@@ -220,20 +219,6 @@ __global__ void __launch_bounds__(kGramThreads, 2)
           }
         }
     }
-  }
-  if (!ticket) return;
-  if (!last_block(ticket)) return;
-  const int kk = k * k, nb = gridDim.x;
-  for (int e = threadIdx.x; e < kk; e += kGramThreads) {
-    double a[8] = {};
-    int b = 0;
-    for (; b + 8 <= nb; b += 8)
-#pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] += (double)__ldcg(&partials[(int64_t)(b + u) * kk + e]);
-    for (; b < nb; ++b) a[0] += (double)__ldcg(&partials[(int64_t)b * kk + e]);
-    const double v = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-    if constexpr (FP64) G64[e] = v;
-    if (G32) G32[e] = (float)v;
   }
 }
 
@@ -409,7 +394,10 @@ size_t gram_smem_bytes(int k) {
 // ascending within each), and the chains and then the warps' sums are added
 // in a fixed order, so the result does not depend on scheduling.  32 warps for
 // many partials (with eight, 188 partials at k = 50 took 10 us a call), eight
-// for few (a wide Gram's 13-19 partials: 11 us at k = 256, 29 us with 32).
+// for few (a wide Gram's 13-19 partials: 11 us at k = 256, 29 us with 32).  A
+// launch of its own: the last block of k_gram_part adding the partials reads them on
+// one SM (2000 rows, both in a graph: 22.7 against 12.4 us at k = 32, 43 against 15
+// at k = 50; no faster at k = 10).
 int gram_red_threads(int nb) { return nb >= 64 ? 1024 : 256; }
 __global__ void __launch_bounds__(1024)
     k_gram_reduce_d(const double *__restrict__ partials, int nb, int k, double *__restrict__ G64,
@@ -485,17 +473,12 @@ int gram_partial_blocks(int64_t rows, int max_blocks) {
 }
 
 namespace {
-// The last block's sum of nb partials replaces the reduction's launch (~2 us)
-// while one block's reads of nb k^2 values take less.
-bool fused_final(int nb, int k) { return (int64_t)nb * k * k <= 24000; }
-
 bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partials, int max_blocks,
                    int *err, cudaStream_t s, cudaError_t *status);
 }  // namespace
 
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err,
-                        unsigned *ticket) {
+                        float *partials, int max_blocks, cudaStream_t s, int *err) {
   // wide ranks: the TMA-fed FP32 product kernel on X^T X (below)
   if (ldx == k && err) {
     cudaError_t st = cudaSuccess;
@@ -530,17 +513,14 @@ cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float 
   const size_t smem = gram_smem_bytes<false>(k);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_gram_part<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (!fused_final(nb, k)) ticket = nullptr;
-  k_gram_part<false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, G, nullptr,
-                                                   ticket);
-  if (!ticket) k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G);
-  g_launches += ticket ? 1 : 2;
+  k_gram_part<false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
+  k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G);
+  g_launches += 2;
   return cudaGetLastError();
 }
 
 cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, double *G64,
-                          float *G32, double *partials, int max_blocks, cudaStream_t s,
-                          unsigned *ticket) {
+                          float *G32, double *partials, int max_blocks, cudaStream_t s) {
   // 64 rows (one stage) per block while 128 would leave most SMs idle
   int nb = gram_partial_blocks(rows, max_blocks);
   if (nb <= max_blocks / 4) nb = (int)((rows + 63) / 64);
@@ -548,12 +528,9 @@ cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, doub
   const size_t smem = gram_smem_bytes<true>(k);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_gram_part<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (!fused_final(nb, k)) ticket = nullptr;
-  k_gram_part<true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, G32, G64,
-                                                  ticket);
-  if (!ticket)
-    k_gram_reduce_d<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G64, G32);
-  g_launches += ticket ? 1 : 2;
+  k_gram_part<true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
+  k_gram_reduce_d<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G64, G32);
+  g_launches += 2;
   return cudaGetLastError();
 }
 
