@@ -15,6 +15,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <string>
@@ -65,7 +66,7 @@ struct aunmf_handle {
   Buf Ht, PW, PHt, GH, GW, G64, gpart, dpart, n2a, ctr, relres, last;
   Buf Ax, At, Hk, Wt, parts, err;  // tensor-core path: layout copies, split partials, error flag
   Buf tcacc;                       // tensor-core path, k > 64: partial sums of wide products
-  Buf colptr, cnz, cscratch;  // sparse path: CSC copy of A
+  Buf colptr, cnz, cscratch;  // sparse path: CSC copy of A; sort scratch, then partial sums
   Buf bppq;                            // BPP: G^{-1} in FP64
   Buf dHt;                             // loss backward: (dL/dH)^T
   Buf batch, batch_meta;               // batched runs: arena, descriptors
@@ -76,7 +77,7 @@ struct aunmf_handle {
   std::map<std::tuple<int, int64_t, int64_t, int, int>, std::pair<int, int>> gemm_tuned;
   Buf hA, hW, hH;  // device copies for aunmf_run_host
   Buf aux;         // printed HALS sweep / projected gradient: partials, barrier, values
-  Buf splr, splc;  // sparse: long rows of the CSR and of the CSC, with their partial sums
+  Buf splr, splc;  // sparse: long rows of the CSR and of the CSC
   int max_gram_blocks = 2 * 152;
   int n_dparts = 2 * 152;
 };
@@ -479,24 +480,28 @@ int prepare_tc(aunmf_handle *h, RunCtx &c, int what, cudaStream_t s) {
 
 int prepare_csr_rows(aunmf_handle *h, RunCtx &c, cudaStream_t s, const float *H) {
   const aunmf_matrix *A = c.A;
-  ENS_TC(h, h->splr, long_rows_bytes(A->nnz, c.k));
-  cudaError_t e = list_long_rows(A->rowptr, A->m, A->nnz, c.k, h->splr.p, &c.csr_long, s, H,
-                                 A->n, c.Ht);
+  ENS_TC(h, h->splr, long_rows_bytes(A->nnz));
+  ENS_TC(h, h->cscratch, long_part_bytes(A->nnz, c.k));
+  cudaError_t e = list_long_rows(A->rowptr, A->m, A->nnz, c.k, h->splr.p, P<float>(h->cscratch),
+                                 &c.csr_long, s, H, A->n, c.Ht);
   return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
 }
 
+// The products' partial sums of long rows (at worst 3 k / 128 bytes a nonzero) take
+// the sort's scratch (24 bytes a nonzero), which is done with by then; it is sized
+// for both here, so a prepare_csr_rows that follows does not move it.
 int prepare_csc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   const aunmf_matrix *A = c.A;
   ENS_TC(h, h->colptr, sizeof(int64_t) * (size_t)(A->n + 1));
   ENS_TC(h, h->cnz, sizeof(uint2) * (size_t)(A->nnz > 0 ? A->nnz : 1));
-  ENS_TC(h, h->cscratch, csc_scratch_bytes(A->n, A->nnz));
-  ENS_TC(h, h->splc, long_rows_bytes(A->nnz, c.k));
+  ENS_TC(h, h->cscratch, std::max(csc_scratch_bytes(A->n, A->nnz), long_part_bytes(A->nnz, c.k)));
+  ENS_TC(h, h->splc, long_rows_bytes(A->nnz));
   cudaError_t e = launch_csr_to_csc(A->rowptr, A->colidx, A->val, A->m, A->n, A->nnz,
                                     P<int64_t>(h->colptr), P<uint2>(h->cnz), h->cscratch.p, s);
   if (e != cudaSuccess) return fail_cuda(h, e, "csr_to_csc");
   c.colptr = P<int64_t>(h->colptr);
   c.cnz = P<uint2>(h->cnz);
-  e = list_long_rows(c.colptr, A->n, A->nnz, c.k, h->splc.p, &c.csc_long, s);
+  e = list_long_rows(c.colptr, A->n, A->nnz, c.k, h->splc.p, P<float>(h->cscratch), &c.csc_long, s);
   return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
 }
 
@@ -787,8 +792,8 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));
   }
   if (!A->dense) {
-    int prc = prepare_csr_rows(h, c, s);
-    if (prc == AUNMF_OK) prc = prepare_csc(h, c, s);
+    int prc = prepare_csc(h, c, s);
+    if (prc == AUNMF_OK) prc = prepare_csr_rows(h, c, s);
     if (prc != AUNMF_OK) return prc;
   }
   if (!c.err) {  // the bounded waits of the wide-rank Gram report here too
@@ -1251,8 +1256,8 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
     CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, h->tick, s));
   }
   if (!A->dense) {
-    int rc = what & kPrepAht ? prepare_csr_rows(h, c, s) : AUNMF_OK;
-    if (rc == AUNMF_OK && (what & kPrepWta)) rc = prepare_csc(h, c, s);
+    int rc = what & kPrepWta ? prepare_csc(h, c, s) : AUNMF_OK;
+    if (rc == AUNMF_OK && (what & kPrepAht)) rc = prepare_csr_rows(h, c, s);
     if (rc != AUNMF_OK) return rc;
   }
   return AUNMF_OK;

@@ -158,12 +158,14 @@ cudaError_t launch_aht_csr(const int64_t *rowptr, const int32_t *colidx, const f
 cudaError_t launch_wta_csc(const int64_t *colptr, const uint2 *cnz, int64_t n, int64_t m,
                            int64_t nnz, const float *W, int k, float *P, const SpLongRows &lr,
                            cudaStream_t s);
-// mem: long_rows_bytes(nnz, k) bytes (8-byte aligned), cut up into lr and
-// filled on the device; enqueues only.
-size_t long_rows_bytes(int64_t nnz, int k);
+// mem: long_rows_bytes(nnz) bytes (8-byte aligned), cut up into lr and filled on
+// the device; part: long_part_bytes(nnz, k) bytes, used by the products alone (a
+// handle's products run in stream order and share them); enqueues only.
 // in (may be null): the same launch also transposes in (k x cols) into out.
+size_t long_rows_bytes(int64_t nnz);
+size_t long_part_bytes(int64_t nnz, int k);
 cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
-                           SpLongRows *lr, cudaStream_t s, const float *in = nullptr,
+                           float *part, SpLongRows *lr, cudaStream_t s, const float *in = nullptr,
                            int64_t cols = 0, float *out = nullptr);
 size_t csc_scratch_bytes(int64_t n, int64_t nnz);
 cudaError_t launch_csr_to_csc(const int64_t *rowptr, const int32_t *colidx, const float *val,

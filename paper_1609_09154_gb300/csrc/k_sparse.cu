@@ -356,22 +356,26 @@ int64_t cap_long_rows(int64_t nnz) { return nnz / kLongRowNz + 1; }
 int64_t cap_long_chunks(int64_t nnz) { return 3 * nnz / kLongRowNz + 1; }
 }  // namespace
 
-size_t long_rows_bytes(int64_t nnz, int k) {
+size_t long_rows_bytes(int64_t nnz) {
   const size_t cr = (size_t)cap_long_rows(nnz), cc = (size_t)cap_long_chunks(nnz);
   return sizeof(SpSegment) * kSpMaxSegs + sizeof(int64_t) * (3 * cr + 3 * cc) +
-         sizeof(unsigned) * cr + sizeof(float) * cc * k;
+         sizeof(unsigned) * cr;
+}
+
+size_t long_part_bytes(int64_t nnz, int k) {
+  return nnz <= kLongRowNz ? 0 : sizeof(float) * (size_t)cap_long_chunks(nnz) * k;
 }
 
 cudaError_t list_long_rows(const int64_t *ptr, int64_t rows, int64_t nnz, int k, void *mem,
-                           SpLongRows *lr, cudaStream_t s, const float *in, int64_t cols,
-                           float *out) {
+                           float *part, SpLongRows *lr, cudaStream_t s, const float *in,
+                           int64_t cols, float *out) {
   lr->cap_rows = cap_long_rows(nnz);
   lr->cap_chunks = cap_long_chunks(nnz);
   lr->seg = static_cast<SpSegment *>(mem);
   lr->row = reinterpret_cast<int64_t *>(lr->seg + kSpMaxSegs);
   lr->chunk = lr->row + 3 * lr->cap_rows;
-  lr->part = reinterpret_cast<float *>(lr->chunk + 3 * lr->cap_chunks);
-  lr->left = reinterpret_cast<unsigned *>(lr->part + lr->cap_chunks * k);
+  lr->left = reinterpret_cast<unsigned *>(lr->chunk + 3 * lr->cap_chunks);
+  lr->part = part;
   lr->blocks = lr->nseg = 0;
   if (rows == 0 || nnz <= kLongRowNz)  // no long row
     return in ? launch_transpose(in, k, cols, out, s) : cudaSuccess;

@@ -38,3 +38,20 @@ def test_fp32_products_without_kept_slabs(aunmf, n):
     # factor's copy m (k + 3): 4 bytes each, and some 2 MB pages
     need = 4 * (3 * n * k + 304 * k * k + 4 * m * k + m * (k + 3))
     assert growth(aunmf, lambda h: h.relres(A, W, H)) <= need + (40 << 20)
+
+@pytest.mark.parametrize("k", [50, 512])
+def test_sparse_products(aunmf, k):
+    """The CSC (8 bytes a nonzero) and its sort (24) are all that grows with the
+    nonzeros, besides the list of long rows (at worst 72 / 512 + 28 / 512): the
+    long rows' partial sums, at worst 12 k / 512 bytes, share the sort's memory."""
+    m, n, per = 1 << 19, 3000, 32
+    nnz = m * per
+    ptr = torch.arange(0, nnz + 1, per, device="cuda", dtype=torch.int64)
+    idx = (torch.arange(m, device="cuda")[:, None] * 7 + torch.arange(per, device="cuda") * 93) % n
+    idx = idx.sort(1).values.int().reshape(-1).contiguous()
+    val = torch.rand(nnz, device="cuda")
+    S = aunmf.csr_matrix(ptr, idx, val, (m, n))
+    W = torch.rand((m, k), device="cuda")
+    torch.empty((k, n), device="cuda")  # (wta's output then comes from torch's cache)
+    used = growth(aunmf, lambda h: h.wta(S, W))
+    assert used <= 32.2 * nnz + 4 * 2 * n * k + (24 << 20)
