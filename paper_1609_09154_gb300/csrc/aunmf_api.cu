@@ -57,10 +57,7 @@ struct aunmf_handle {
   cudaStream_t cap_stream = nullptr;  // private stream used only for graph capture
   cudaEvent_t moved = nullptr;        // the last work of the stream bound before
   std::string cuda_err;
-  // The ticket counter of the norm and residual kernels.  Zeroed by aunmf_create;
-  // each launch leaves it at 0, and a handle's launches are in one order
-  // (aunmf_set_stream keeps it).
-  unsigned *tick = nullptr;
+  unsigned *tick = nullptr;  // zeroed counters of the kernels whose last block finishes up
   // workspace
   Buf GWr;                          // HALS: W^T W before the normalisation
   Buf Ht, PW, PHt, GH, GW, G64, gpart, dpart, n2a, ctr, relres, last;
@@ -136,6 +133,12 @@ template <class T>
 T *P(Buf &b) {
   return reinterpret_cast<T *>(b.p);
 }
+
+// The handle's ticket counters: one for the Gram kernels, one for the norm and
+// residual kernels.  Zeroed by aunmf_create; each launch leaves its own at 0, and
+// a handle's launches are in one order (aunmf_set_stream keeps it).
+unsigned *gram_tick(aunmf_handle *h) { return h->tick; }
+unsigned *sum_tick(aunmf_handle *h) { return h->tick + 1; }
 
 bool valid_matrix(const aunmf_matrix *A) {
   if (!A || A->m < 1 || A->n < 1) return false;
@@ -398,7 +401,7 @@ cudaError_t iterate(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   {
     PhaseTimer t(c, s, kPhOther);
     e = launch_relres(c.PHt, c.Ht, n * (int64_t)k, c.GW, c.GH, k, c.n2a, c.dpart, h->n_dparts,
-                      c.relres_dev, c.ctr, c.last, h->tick, s);
+                      c.relres_dev, c.ctr, c.last, sum_tick(h), s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -575,8 +578,8 @@ int aunmf_create(aunmf_handle **out, void *stream) {
   h->stream = reinterpret_cast<cudaStream_t>(stream);
   e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->moved, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&h->tick), sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->tick, 0, sizeof(unsigned), h->cap_stream);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&h->tick), 2 * sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->tick, 0, 2 * sizeof(unsigned), h->cap_stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->cap_stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -765,9 +768,9 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
   if (A->dense && o.prec != AUNMF_FP32) {
     // ||A||^2 comes out of the layout pass (prepare_tc below)
   } else if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, h->tick, s));
+    CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   } else {
-    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, h->tick, s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (o.prec != AUNMF_FP32) {
     // Short TF32 runs (k <= 64) read A itself and save the layout pass (12 m n
@@ -954,7 +957,7 @@ int aunmf_gram_w(aunmf_handle *h, const float *W, int64_t m, int k, float *G) {
   ENS(h, h->err, sizeof(int));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
   CK(h, launch_gram(W, m, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   return AUNMF_OK;
 }
 
@@ -966,7 +969,7 @@ int aunmf_gram_h(aunmf_handle *h, const float *H, int k, int64_t n, float *G) {
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
   CK(h, launch_transpose(H, k, n, P<float>(h->Ht), h->stream));
   CK(h, launch_gram(P<float>(h->Ht), n, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   return AUNMF_OK;
 }
 
@@ -1088,7 +1091,8 @@ int aunmf_update_w(aunmf_handle *h, int algo, float *W, const float *PW, const f
   if (algo == AUNMF_HALS) {
     ENS(h, h->GW, sizeof(float) * k * k);
     ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
-    CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s));
+    CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s, nullptr,
+                      gram_tick(h)));
     if (H && n > 0) {
       ENS(h, h->Ht, sizeof(float) * n * k);
       CK(h, launch_transpose(H, k, n, P<float>(h->Ht), s));
@@ -1175,12 +1179,12 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), s));
   CK(h, launch_transpose(H, k, n, Ht, s));
   if (A->dense) {
-    CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), h->tick, s));
+    CK(h, launch_norm2(A->dense, m, n, A->lda, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     ENS(h, h->parts, simt_parts_bytes(A->m, n, k, simt_aligned(A->dense, A->lda), false));
     CK(h, launch_wta_simt(A->dense, m, n, A->lda, W, k, PHt, P<float>(h->parts), false,
                           P<int>(h->err), s));
   } else {
-    CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), h->tick, s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, dp, h->n_dparts, P<double>(h->n2a), sum_tick(h), s));
     RunCtx c{};
     c.A = A;
     c.k = k;
@@ -1189,12 +1193,12 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
     CK(h, launch_wta_csc(c.colptr, c.cnz, n, m, A->nnz, W, k, PHt, c.csc_long, s));
   }
   CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   CK(h, launch_gram(Ht, n, k, k, P<float>(h->GH), P<float>(h->gpart), h->max_gram_blocks, s,
-                    P<int>(h->err)));
+                    P<int>(h->err), gram_tick(h)));
   CK(h, launch_relres(PHt, Ht, n * (int64_t)k, P<float>(h->GW), P<float>(h->GH), k,
                       P<double>(h->n2a), dp, h->n_dparts, nullptr, P<DevCounters>(h->ctr),
-                      P<double>(h->last), h->tick, s));
+                      P<double>(h->last), sum_tick(h), s));
   int herr = 0;
   CK(h, cudaMemcpyAsync(&herr, h->err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(h, cudaMemcpyAsync(relres, h->last.p, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1245,7 +1249,7 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
     if (rc != AUNMF_OK) return rc;
   } else if (A->dense) {
     if (what & kPrepNorm)
-      CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, h->tick, s));
+      CK(h, launch_norm2(A->dense, m, n, A->lda, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
     ENS(h, h->parts, simt_parts_bytes(m, n, k, simt_aligned(A->dense, A->lda), true));
     c.parts = P<float>(h->parts);
     c.even = true;
@@ -1253,7 +1257,7 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
     c.err = P<int>(h->err);
     CK(h, cudaMemsetAsync(c.err, 0, sizeof(int), s));
   } else if (what & kPrepNorm) {
-    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, h->tick, s));
+    CK(h, launch_norm2_vec(A->val, A->nnz, c.dpart, h->n_dparts, c.n2a, sum_tick(h), s));
   }
   if (!A->dense) {
     int rc = what & kPrepWta ? prepare_csc(h, c, s) : AUNMF_OK;
@@ -1273,10 +1277,10 @@ int aunmf_loss_fwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;
   CK(h, product_wta(h, c, s));
-  CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err));
-  CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err));
+  CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
+  CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
   CK(h, launch_loss(c.PHt, c.Ht, n * (int64_t)k, c.GW, c.GH, k, c.n2a, c.dpart, h->n_dparts, loss,
-                    h->tick, s));
+                    sum_tick(h), s));
   if (WtA) CK(h, launch_transpose(c.PHt, n, k, WtA, s));
   return AUNMF_OK;
 }
@@ -1290,13 +1294,13 @@ int aunmf_loss_bwd(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W
   cudaStream_t s = h->stream;
   const int64_t m = A->m, n = A->n;
   if (dW) {  // dL/dW = W (H H^T) - A H^T
-    CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err));
+    CK(h, launch_gram(c.Ht, n, k, k, c.GH, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
     CK(h, product_aht(h, c, s));
     CK(h, launch_xg_minus_p(c.W, c.PW, c.GH, m, k, grad_out, dW, s));
   }
   if (dH) {  // dL/dH = (W^T W) H - W^T A, formed transposed
     ENS(h, h->dHt, sizeof(float) * n * k);
-    CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err));
+    CK(h, launch_gram(c.W, m, k, k, c.GW, c.gpart, h->max_gram_blocks, s, c.err, gram_tick(h)));
     if (WtA) {
       CK(h, launch_transpose(WtA, k, n, c.PHt, s));
     } else {

@@ -103,8 +103,13 @@ __device__ __forceinline__ void two_fma_acc(float a, float b, float &hi, float &
 // err: the device error flag for the bounded waits of the wide-rank form
 // (k >= 96, which runs the TMA-fed product kernel on X^T X); null keeps the
 // k_gram_part form.
+// ticket: a zeroed counter (left at 0) that lets a very small factor's last block
+// add the partials, which spares a launch: for calls by themselves (in a captured
+// iteration the launch costs less than the wait, 0.25 us a Gram at k = 10).
+// Launches that share a ticket run in stream order, as they share the partials.
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr);
+                        float *partials, int max_blocks, cudaStream_t s, int *err = nullptr,
+                        unsigned *ticket = nullptr);
 int gram_partial_blocks(int64_t rows, int max_blocks);
 // The same Gram with every product formed exactly in FP64 (FP32 x FP32 fits a
 // double) and summed in FP64: G64 (k x k, FP64) for the BPP solves, and G32 =

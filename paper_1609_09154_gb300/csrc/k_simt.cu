@@ -64,10 +64,13 @@ __device__ __forceinline__ int gram_groups(int ntiles) {
 //     positive definite.
 // The next 64-row slab is loaded into registers while the current one is
 // consumed from shared memory.  Dynamic shared memory: gram_smem_bytes().
-template <bool FP64>
+// LAST (FP32): the last block to finish adds all partials in FP64 and writes G;
+// *ticket starts at 0 and is 0 again after (see launch_gram on when).
+template <bool FP64, bool LAST>
 __global__ void __launch_bounds__(kGramThreads, 2)
     k_gram_part(const float *__restrict__ X, int64_t rows, int k, int64_t ldx, int64_t chunk,
-                typename std::conditional<FP64, double, float>::type *__restrict__ partials) {
+                typename std::conditional<FP64, double, float>::type *__restrict__ partials,
+                float *__restrict__ G, unsigned *ticket) {
   using T = typename std::conditional<FP64, double, float>::type;
   extern __shared__ __align__(16) float sX[];  // [kGramRows][kp], then the group sums
   constexpr int kPre = (kGramRows * 64 + kGramThreads - 1) / kGramThreads;  // k <= 64 prefetch
@@ -218,6 +221,19 @@ __global__ void __launch_bounds__(kGramThreads, 2)
             out[j * k + i] = v;
           }
         }
+    }
+  }
+  if constexpr (LAST) {
+    if (!last_block(ticket)) return;
+    const int kk = k * k, nb = gridDim.x;
+    for (int e = threadIdx.x; e < kk; e += kGramThreads) {
+      double a[8] = {};
+      int b = 0;
+      for (; b + 8 <= nb; b += 8)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u] += (double)__ldcg(&partials[(int64_t)(b + u) * kk + e]);
+      for (; b < nb; ++b) a[0] += (double)__ldcg(&partials[(int64_t)b * kk + e]);
+      G[e] = (float)(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
     }
   }
 }
@@ -394,14 +410,16 @@ size_t gram_smem_bytes(int k) {
 // ascending within each), and the chains and then the warps' sums are added
 // in a fixed order, so the result does not depend on scheduling.  32 warps for
 // many partials (with eight, 188 partials at k = 50 took 10 us a call), eight
-// for few (a wide Gram's 13-19 partials: 11 us at k = 256, 29 us with 32).  A
-// launch of its own: the last block of k_gram_part adding the partials reads them on
-// one SM (2000 rows, both in a graph: 22.7 against 12.4 us at k = 32, 43 against 15
-// at k = 50; no faster at k = 10).
+// for few (a wide Gram's 13-19 partials: 11 us at k = 256, 29 us with 32).
 int gram_red_threads(int nb) { return nb >= 64 ? 1024 : 256; }
+// chains8 (few values, kChainValues): eight warps sum the partials b = w mod 8 each,
+// the last nb mod 8 after warp 0's, and the chains are added pairwise -- an order
+// that small ABPP Grams keep, whose last bits (1e-16) decide the fifth digit of a
+// residual near 2e-3.
+constexpr int64_t kChainValues = 24000;
 __global__ void __launch_bounds__(1024)
-    k_gram_reduce_d(const double *__restrict__ partials, int nb, int k, double *__restrict__ G64,
-                    float *__restrict__ G32) {
+    k_gram_reduce_d(const double *__restrict__ partials, int nb, int k, bool chains8,
+                    double *__restrict__ G64, float *__restrict__ G32) {
   __shared__ double sw[32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int kk = k * k;
@@ -411,7 +429,13 @@ __global__ void __launch_bounds__(1024)
   // four independent chains (loads in flight, FP64 latency overlapped),
   // combined in a fixed order
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  if (e < kk) {
+  if (e < kk && chains8) {
+    const int nb8 = nb & ~7;
+#pragma unroll 4
+    for (int b = w; b < nb8; b += 8) a0 += partials[(int64_t)b * kk + e];
+    if (w == 0)
+      for (int b = nb8; b < nb; ++b) a0 += partials[(int64_t)b * kk + e];
+  } else if (e < kk) {
     int b = b0;
     for (; b + 4 <= b1; b += 4) {
       a0 += partials[(int64_t)b * kk + e];
@@ -425,7 +449,11 @@ __global__ void __launch_bounds__(1024)
   __syncthreads();
   if (w == 0 && e < kk) {
     double s = 0.0;
-    for (int q = 0; q < nw; ++q) s += sw[q][lane];
+    if (chains8)
+      s = ((sw[0][lane] + sw[1][lane]) + (sw[2][lane] + sw[3][lane])) +
+          ((sw[4][lane] + sw[5][lane]) + (sw[6][lane] + sw[7][lane]));
+    else
+      for (int q = 0; q < nw; ++q) s += sw[q][lane];
     G64[e] = s;
     if (G32) G32[e] = (float)s;
   }
@@ -478,7 +506,8 @@ bool gram_via_gemm(const float *X, int64_t rows, int k, float *G, float *partial
 }  // namespace
 
 cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float *G,
-                        float *partials, int max_blocks, cudaStream_t s, int *err) {
+                        float *partials, int max_blocks, cudaStream_t s, int *err,
+                        unsigned *ticket) {
   // wide ranks: the TMA-fed FP32 product kernel on X^T X (below)
   if (ldx == k && err) {
     cudaError_t st = cudaSuccess;
@@ -512,8 +541,20 @@ cudaError_t launch_gram(const float *X, int64_t rows, int k, int64_t ldx, float 
   const int64_t chunk = (rows + nb - 1) / nb;
   const size_t smem = gram_smem_bytes<false>(k);
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_gram_part<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_gram_part<false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
+    cudaFuncSetAttribute(k_gram_part<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+  // An entry a thread and at most three rounds of loads: the last block's sum takes
+  // no longer than the reduction's launch.  Beyond, one SM reading the partials is
+  // slower (2000 rows, both in a graph: 22.7 against 12.4 us at k = 32, 43 against 15
+  // at k = 50).
+  if (ticket && k <= 16 && nb <= 24) {
+    k_gram_part<false, true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, G,
+                                                            ticket);
+    g_launches += 1;
+    return cudaGetLastError();
+  }
+  k_gram_part<false, false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, nullptr,
+                                                           nullptr);
   k_gram_reduce<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G);
   g_launches += 2;
   return cudaGetLastError();
@@ -527,9 +568,13 @@ cudaError_t launch_gram_d(const float *X, int64_t rows, int k, int64_t ldx, doub
   const int64_t chunk = (rows + nb - 1) / nb;
   const size_t smem = gram_smem_bytes<true>(k);
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_gram_part<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_gram_part<true><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials);
-  k_gram_reduce_d<<<(k * k + 31) / 32, gram_red_threads(nb), 0, s>>>(partials, nb, k, G64, G32);
+    cudaFuncSetAttribute(k_gram_part<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+  k_gram_part<true, false><<<nb, kGramThreads, smem, s>>>(X, rows, k, ldx, chunk, partials, nullptr,
+                                                          nullptr);
+  const bool chains8 = (int64_t)nb * k * k <= kChainValues;
+  k_gram_reduce_d<<<(k * k + 31) / 32, chains8 ? 256 : gram_red_threads(nb), 0, s>>>(
+      partials, nb, k, chains8, G64, G32);
   g_launches += 2;
   return cudaGetLastError();
 }
