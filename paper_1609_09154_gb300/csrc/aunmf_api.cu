@@ -57,8 +57,9 @@ struct aunmf_handle {
   cudaStream_t cap_stream = nullptr;  // private stream used only for graph capture
   cudaEvent_t moved = nullptr;        // the last work of the stream bound before
   std::string cuda_err;
-  unsigned *tick = nullptr;  // zeroed counters of the kernels whose last block finishes up
   // workspace
+  Buf tick;  // counters of the kernels whose last block finishes up
+  bool tick_zeroed = false;
   Buf GWr;                          // HALS: W^T W before the normalisation
   Buf Ht, PW, PHt, GH, GW, G64, gpart, dpart, n2a, ctr, relres, last;
   Buf Ax, At, Hk, Wt, parts, err;  // tensor-core path: layout copies, split partials, error flag
@@ -100,6 +101,15 @@ size_t dpart_bytes(const aunmf_handle *h) {
   return sizeof(double) * (a > b ? a : b);
 }
 
+// Whether work enqueued on s is captured into a graph (or, for the legacy stream,
+// refused because another capture is under way).
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 int ensure(aunmf_handle *h, Buf &b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (b.cap >= bytes) return AUNMF_OK;
@@ -135,10 +145,22 @@ T *P(Buf &b) {
 }
 
 // The handle's ticket counters: one for the Gram kernels, one for the norm and
-// residual kernels.  Zeroed by aunmf_create; each launch leaves its own at 0, and
+// residual kernels.  Zeroed by the first call; each launch leaves its own at 0, and
 // a handle's launches are in one order (aunmf_set_stream keeps it).
-unsigned *gram_tick(aunmf_handle *h) { return h->tick; }
-unsigned *sum_tick(aunmf_handle *h) { return h->tick + 1; }
+int ensure_tick(aunmf_handle *h) {
+  if (h->tick_zeroed) return AUNMF_OK;
+  ENS(h, h->tick, 2 * sizeof(unsigned));
+  CK(h, cudaMemsetAsync(h->tick.p, 0, 2 * sizeof(unsigned), h->stream));
+  h->tick_zeroed = !capturing(h->stream);  // (captured zeroing is still to come)
+  return AUNMF_OK;
+}
+#define ENS_TICK(h)                        \
+  do {                                     \
+    int rc_ = ensure_tick(h);              \
+    if (rc_ != AUNMF_OK) return rc_;       \
+  } while (0)
+unsigned *gram_tick(aunmf_handle *h) { return P<unsigned>(h->tick); }
+unsigned *sum_tick(aunmf_handle *h) { return P<unsigned>(h->tick) + 1; }
 
 bool valid_matrix(const aunmf_matrix *A) {
   if (!A || A->m < 1 || A->n < 1) return false;
@@ -508,16 +530,8 @@ int prepare_csc(aunmf_handle *h, RunCtx &c, cudaStream_t s) {
   return e == cudaSuccess ? AUNMF_OK : fail_cuda(h, e, "list_long_rows");
 }
 
-// Everything of a handle but its workspace.
-void free_handle(aunmf_handle *h) {
-  if (h->tick) cudaFree(h->tick);
-  if (h->moved) cudaEventDestroy(h->moved);
-  if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-  delete h;
-}
-
 // Whatever the handle has enqueued on `from` comes before what it enqueues on
-// `to`: calls share the workspace and the ticket counter, which two launches that
+// `to`: calls share the workspace and the ticket counters, which two launches that
 // overlap would leave at a value other than 0 for good.  A stream that is
 // being captured cannot wait for work outside its graph: the host waits for that
 // work instead; work captured so far runs when its graph is launched, and that
@@ -526,26 +540,20 @@ void order_streams(aunmf_handle *h, cudaStream_t from, cudaStream_t to) {
   int dev = h->device;
   cudaGetDevice(&dev);
   if (dev != h->device) cudaSetDevice(h->device);
-  bool failed = false;
-  auto capturing = [&](cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    const cudaError_t e = cudaStreamIsCapturing(s, &st);
-    failed |= e != cudaSuccess;
-    return e != cudaSuccess || st != cudaStreamCaptureStatusNone;
-  };
   if (!capturing(from)) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaError_t e = cudaEventRecord(h->moved, from);
+    cudaError_t e = cudaSuccess;
+    if (!h->moved) e = cudaEventCreateWithFlags(&h->moved, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(h->moved, from);
     if (e == cudaSuccess)
       e = capturing(to) ? cudaEventSynchronize(h->moved) : cudaStreamWaitEvent(to, h->moved, 0);
     if (e != cudaSuccess) {
-      failed = true;
       cudaDeviceSynchronize();
+      cudaGetLastError();
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
   }
-  if (failed) cudaGetLastError();
   if (dev != h->device) cudaSetDevice(dev);
 }
 
@@ -577,16 +585,7 @@ int aunmf_create(aunmf_handle **out, void *stream) {
   if (e != cudaSuccess) { int rc = fail_cuda(h, e, "cudaGetDevice"); delete h; return rc; }
   h->stream = reinterpret_cast<cudaStream_t>(stream);
   e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->moved, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&h->tick), 2 * sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->tick, 0, 2 * sizeof(unsigned), h->cap_stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->cap_stream);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    int rc = e == cudaErrorMemoryAllocation ? AUNMF_E_NOMEM : fail_cuda(h, e, "aunmf_create");
-    free_handle(h);
-    return rc;
-  }
+  if (e != cudaSuccess) { int rc = fail_cuda(h, e, "cudaStreamCreate"); delete h; return rc; }
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   // Gram partials: one per block of a single resident wave (two 256-thread
@@ -609,13 +608,15 @@ int aunmf_set_stream(aunmf_handle *h, void *stream) {
 int aunmf_destroy(aunmf_handle *h) {
   if (!h) return AUNMF_E_INVAL;
   cudaStreamSynchronize(h->stream);
-  Buf *bufs[] = {&h->GWr, &h->Ht, &h->PW, &h->PHt, &h->GH, &h->GW, &h->G64, &h->gpart, &h->dpart, &h->n2a,
+  Buf *bufs[] = {&h->tick, &h->GWr, &h->Ht, &h->PW, &h->PHt, &h->GH, &h->GW, &h->G64, &h->gpart, &h->dpart, &h->n2a,
                  &h->ctr, &h->relres, &h->last, &h->Ax, &h->At, &h->Hk, &h->Wt, &h->parts,
                  &h->err, &h->tcacc, &h->aux, &h->splr, &h->splc, &h->colptr, &h->cnz, &h->cscratch, &h->bppq, &h->dHt,
                  &h->batch, &h->batch_meta, &h->hA, &h->hW, &h->hH};
   for (Buf *b : bufs)
     if (b->p) cudaFree(b->p);
-  free_handle(h);
+  if (h->moved) cudaEventDestroy(h->moved);
+  if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+  delete h;
   return AUNMF_OK;
 }
 
@@ -700,6 +701,7 @@ static int run_impl(aunmf_handle *h, const aunmf_matrix *A, int k, int algo, int
   ENS(h, h->GH, sizeof(float) * k * k);
   ENS(h, h->GW, sizeof(float) * k * k);
   ENS(h, h->GWr, sizeof(float) * k * k);
+  ENS_TICK(h);
   ENS(h, h->G64, 2 * sizeof(double) * k * k);
   ENS(h, h->gpart, sizeof(double) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->dpart, dpart_bytes(h));
@@ -956,6 +958,7 @@ int aunmf_gram_w(aunmf_handle *h, const float *W, int64_t m, int k, float *G) {
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->err, sizeof(int));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
+  ENS_TICK(h);
   CK(h, launch_gram(W, m, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
                     P<int>(h->err), gram_tick(h)));
   return AUNMF_OK;
@@ -967,6 +970,7 @@ int aunmf_gram_h(aunmf_handle *h, const float *H, int k, int64_t n, float *G) {
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->err, sizeof(int));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), h->stream));
+  ENS_TICK(h);
   CK(h, launch_transpose(H, k, n, P<float>(h->Ht), h->stream));
   CK(h, launch_gram(P<float>(h->Ht), n, k, k, G, P<float>(h->gpart), h->max_gram_blocks, h->stream,
                     P<int>(h->err), gram_tick(h)));
@@ -1091,6 +1095,7 @@ int aunmf_update_w(aunmf_handle *h, int algo, float *W, const float *PW, const f
   if (algo == AUNMF_HALS) {
     ENS(h, h->GW, sizeof(float) * k * k);
     ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
+    ENS_TICK(h);
     CK(h, launch_gram(W, m, k, k, P<float>(h->GW), P<float>(h->gpart), h->max_gram_blocks, s, nullptr,
                       gram_tick(h)));
     if (H && n > 0) {
@@ -1175,6 +1180,7 @@ int aunmf_relres(aunmf_handle *h, const aunmf_matrix *A, const float *W, const f
   float *Ht = P<float>(h->Ht), *PHt = P<float>(h->PHt);
   double *dp = P<double>(h->dpart);
   ENS(h, h->err, sizeof(int));
+  ENS_TICK(h);
   CK(h, cudaMemsetAsync(h->ctr.p, 0, sizeof(DevCounters), s));
   CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), s));
   CK(h, launch_transpose(H, k, n, Ht, s));
@@ -1228,6 +1234,7 @@ int loss_setup(aunmf_handle *h, const aunmf_matrix *A, int k, const float *W, co
   ENS(h, h->gpart, sizeof(float) * (size_t)h->max_gram_blocks * k * k);
   ENS(h, h->dpart, dpart_bytes(h));
   ENS(h, h->n2a, 2 * sizeof(double));
+  ENS_TICK(h);
   c.A = A;
   c.k = k;
   c.prec = prec;

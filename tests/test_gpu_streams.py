@@ -98,3 +98,24 @@ def test_calls_captured_in_a_graph(aunmf):
     assert torch.equal(big, GX)
     h.set_stream(torch.cuda.current_stream())
     h.close()
+
+
+def test_first_call_captured(aunmf):
+    """A handle whose first call of all is captured: its counters start at 0 for the
+    calls that follow, whether or not the graph has run."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    X, Y = ints(g, 1500, 10), ints(g, 900, 9)
+    GX, GY = (X.double().T @ X.double()).float(), (Y.double().T @ Y.double()).float()
+    h = aunmf.Handle()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+        h.set_stream(torch.cuda.current_stream())
+        G1 = h.gram_w(X)
+    h.set_stream(torch.cuda.current_stream())
+    assert torch.equal(h.gram_w(Y), GY)
+    for _ in range(2):
+        graph.replay()
+        assert torch.equal(h.gram_w(Y), GY)
+        assert torch.equal(G1, GX)
+    h.close()
