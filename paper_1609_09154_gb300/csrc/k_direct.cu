@@ -34,9 +34,10 @@
 //
 // What bounds it: HBM, and close behind it each tile's way through a CTA (TF32,
 // k = 50: the copy in, the converters' read and write, the MMAs' operand reads
-// and the Y copy move ~174 KB through shared memory per 32 KB tile).  A H^T at
-// 96,000 x 64,000, k = 50: 3.95 ms, 92 % of the measured copy rate, against
-// 14.4 + 3.65 ms for the layout pass and the product.  Measured on the way: all
+// and the Y copy move ~174 KB through shared memory per 32 KB tile, by count; the
+// loads and stores among them, 81 KB, by measurement).  A H^T at 96,000 x 64,000,
+// k = 50: the call takes 4.04 ms, 90 % of the measured copy rate, against 14.4 +
+// 3.65 ms for the layout pass and the product.  Measured on the way: all
 // eight converter warps on one stage at a time 4.25 ms (each stage's latency
 // chain in series); X through TMEM instead of shared memory 4.55 ms (room for
 // one operand stage only beside the accumulators: conversion waits for the

@@ -813,7 +813,7 @@ __global__ void __launch_bounds__(256, AUNMF_SIMT_MINB)
 // k_gemm_simt_tma: the same product and the same compensated summation as
 // k_gemm_simt, when A's rows are 16-byte aligned; and, in its short form, for
 // few output tiles whatever the alignment.  FP32 issue bounds it (k = 50,
-// W^T A at 32,000 x 24,000: 46 TFLOP/s of useful FMAs against the 73 a loop
+// W^T A at 32,000 x 24,000: 48 TFLOP/s of useful FMAs against the 73 a loop
 // of packed FMAs reaches).  A's tiles and the fixed factor's 16 x BN tiles
 // arrive by TMA in a seven-stage shared-memory ring with mbarriers (full:
 // one arrival + the copies' bytes; empty: all 256 threads).  The factor is
@@ -1296,11 +1296,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
   }
 }
 
-// Tensor map of A's tiles for k_gemm_simt_tma: AK, a box of 16 K x bm rows
-// over A (M x K, ld lda), 64-byte swizzle; !AK, bm rows x 16 K over A
-// stored K x M, no swizzle.  FP32, zero fill outside the matrix.
-// Tensor map of the factor's tiles: bn columns x 16 K rows over the padded
-// copy (K x N, ld ldp), no swizzle, zero fill past N and K.
+// Tensor map of the factor's tiles for k_gemm_simt_tma: bn columns x 16 K rows over
+// the factor or its padded copy (K x N, ld ldp), no swizzle, zero fill past N and K.
 bool simt_factor_map(CUtensorMap *map, const float *Bp, int64_t K, int N, int ldp, int bn) {
   ptx::EncodeTiledFn fn = ptx::encode_fn();
   if (!fn) return false;
@@ -1313,6 +1310,9 @@ bool simt_factor_map(CUtensorMap *map, const float *Bp, int64_t K, int N, int ld
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tensor map of A's tiles: AK, a box of 16 K x bm rows over A (M x K, ld lda),
+// 64-byte swizzle; !AK, bm rows x 16 K over A stored K x M, no swizzle.  FP32, zero
+// fill outside the matrix.
 bool simt_map(CUtensorMap *map, const float *A, int64_t lda, int64_t M, int64_t K, bool AK,
               int bm) {
   ptx::EncodeTiledFn fn = ptx::encode_fn();

@@ -180,9 +180,10 @@ __global__ void __launch_bounds__(kWThreads, 1)
 //      chain's entries, forms T_q = ((chain + s1) + s2) + s3, two shuffles give (x
 //      G)_i = (T_0 + T_2) + (T_1 + T_3), and the thread whose chain holds x_i
 //      updates it.  Meanwhile the next block's rows of G are copied in.
-// Bound by step 2's dependent chain (~150 clocks a coordinate) and step 1's FMA
-// issue, both at two warps a scheduler.  HALS at k = 256, 7,999 rows: 115 us, 12,001 rows: 193 us
-// (two rounds of tiles on 152 SMs); a warp per two rows 321 and 327 us.
+// Bound by latency, step 2's dependent chain and step 1's loads at two warps a
+// scheduler (k = 256, 7,999 rows, one tile an SM: 870 clocks a coordinate, 28 %
+// issue).  HALS at k = 256, 7,999 rows: 115 us, 12,001 rows: 193 us (two rounds of
+// tiles on 152 SMs); a warp per two rows 321 and 327 us.
 constexpr int kHR = 64;
 constexpr int kHQ = 3 * kNB * kHR + 8;  // floats of one class in sS (+ 8: classes in other banks)
 
